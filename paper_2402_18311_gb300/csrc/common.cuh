@@ -138,6 +138,54 @@ __device__ __forceinline__ double block_sum_fc(float v, float2 *sm) {
   return r;
 }
 
+
+// The same for N values at once: one pair of barriers for all of them and N
+// independent chains in every step of the tree.  sm: N * NT / 32 entries; the
+// results are valid in thread 0.
+template <int NT, int N>
+__device__ __forceinline__ void block_sums_fc(float (&v)[N], float2 *sm, double (&out)[N]) {
+  float c[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) c[k] = 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const float w = __shfl_xor_sync(0xffffffffu, v[k], o), wc = __shfl_xor_sync(0xffffffffu, c[k], o);
+      float e;
+      two_sum(v[k], w, v[k], e);
+      c[k] = __fadd_rn(c[k], __fadd_rn(wc, e));
+    }
+  }
+  const int wi = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) sm[k * (NT / 32) + wi] = make_float2(v[k], c[k]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const float2 p = l < NT / 32 ? sm[k * (NT / 32) + l] : make_float2(0.f, 0.f);
+      v[k] = p.x;
+      c[k] = p.y;
+    }
+#pragma unroll
+    for (int o = NT / 64; o > 0; o >>= 1) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const float w = __shfl_xor_sync(0xffffffffu, v[k], o), wc = __shfl_xor_sync(0xffffffffu, c[k], o);
+        float e;
+        two_sum(v[k], w, v[k], e);
+        c[k] = __fadd_rn(c[k], __fadd_rn(wc, e));
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) out[k] = (double)v[k] + (double)c[k];
+}
+
 typedef unsigned __int128 u128;
 
 __device__ __forceinline__ u128 shfl_xor_u128(u128 v, int o) {
@@ -184,6 +232,20 @@ __device__ __forceinline__ bool arrive_last(unsigned int *ctr, int *sm_flag) {
   const bool last = *sm_flag != 0;
   if (last) __threadfence();
   return last;
+}
+
+// The same where thread 0 alone wrote everything that the last block reads: it
+// alone has to order its writes before the arrival, so the block's other
+// threads do not wait for their own stores.
+__device__ __forceinline__ bool arrive_last_t0(unsigned int *ctr, int *sm_flag) {
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned int prev = atomicAdd(ctr, 1u);
+    __threadfence();
+    *sm_flag = (prev == gridDim.x - 1) ? 1 : 0;
+  }
+  __syncthreads();
+  return *sm_flag != 0;
 }
 
 // floor(a / b) for b > 0 and |a| below 2^40: a float estimate of the

@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, i
     p[1] = (unsigned long long)(r >> 64);
     d.conc_part[(size_t)c * d.nb_red + blockIdx.x] = q2;
   }
-  if (!arrive_last(d.ctr + (size_t)c * C_COUNT + C_FINISH, &flag)) return;
+  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_FINISH, &flag)) return;
   u128 v = 0;
   q2 = 0.f;
 #pragma unroll 4

@@ -55,7 +55,9 @@ struct CopyState {
 
 // Reduction slots (FP64) per copy: each kernel that reduces writes one value
 // per block into its slot range; a reducer sums them in a fixed order.
-enum Slot { S_TAU = 0, S_HPWL, S_WL, S_GW1, S_GD1, S_DG2, S_DV2, S_G2, S_HP64, S_COUNT };
+// S_PH, S_PW and S_PV: the cell-gradient blocks' shares of the WA kernels' and
+// of the step norm's partials (see k_cell_grad).
+enum Slot { S_TAU = 0, S_HPWL, S_WL, S_GW1, S_GD1, S_DG2, S_DV2, S_G2, S_HP64, S_PH, S_PW, S_PV, S_COUNT };
 
 // Last-block counters per copy.
 enum Counter { C_FINISH = 0, C_CELL, C_PRE0, C_UPDATE, C_COUNT };
@@ -94,6 +96,7 @@ struct Dev {
   int BW32, BH32;             // BW, BH (below 2^26: nx, ny >= 16 and nx BW < 2^30)
   float ibw_q, ibh_q;         // 1 / BW, 1 / BH
   double w_bin, dref;
+  double lg_mu;               // log2 mu_base where it is finite and not 0, else 0 (pow takes over)
   int nb_red;                 // partial slots per reduction per copy
   int cell_blocks;            // blocks per copy for per-cell kernels
   int cg_blocks;              // blocks per copy of the cell-gradient kernel (one wave)
@@ -320,10 +323,37 @@ cudaStream_t handle_stream(place_t *h);
 int save_xy(place_t *h, float2 *dst);
 int load_xy(place_t *h, const float2 *src);
 
+// b^y for |y log2 b| below 1000, from lh + ll = log2 b (lh rounded to double, ll
+// the rest): y log2 b = n + f with n an integer and |f| <= 1/2, and 2^f is the
+// Taylor series of exp(f ln 2) to the 14th power (the next term is below
+// 2e-19), summed pairwise so that the chain of dependent FP64 operations is
+// short.  The library's pow takes about 5 us here, on one thread at GB300's
+// FP64 rate and latency, and every iteration waits for it twice.
+__device__ __forceinline__ double pow_log2(double y, double lh, double ll) {
+  const double t = __dmul_rn(y, lh);
+  const double tl = __fma_rn(y, lh, -t) + y * ll;
+  const double n = rint(t);
+  const double r = ((t - n) + tl) * 0.69314718055994530942;
+  const double r2 = r * r, r4 = r2 * r2, r8 = r4 * r4;
+  const double p01 = 1.0 + r;
+  const double p23 = fma(r, 1.0 / 6, 0.5);
+  const double p45 = fma(r, 1.0 / 120, 1.0 / 24);
+  const double p67 = fma(r, 1.0 / 5040, 1.0 / 720);
+  const double p89 = fma(r, 1.0 / 362880, 1.0 / 40320);
+  const double pab = fma(r, 1.0 / 39916800, 1.0 / 3628800);
+  const double pce = fma(r2, 1.0 / 87178291200.0, fma(r, 1.0 / 6227020800.0, 1.0 / 479001600));
+  const double q0 = fma(p23, r2, p01), q1 = fma(p67, r2, p45), q2 = fma(pab, r2, p89);
+  const double e = fma(fma(pce, r4, q2), r8, fma(q1, r4, q0));
+  return e * __longlong_as_double((long long)((int)n + 1023) << 52);
+}
+
 // gamma of the weighted-average model from the previous overflow (Eq. 3)
 __device__ __forceinline__ double gamma_of(const Dev &d, double tau_prev) {
   if (d.prm.constant_gamma > 0.f) return (double)d.prm.constant_gamma;
-  return (double)d.prm.gamma_base * d.w_bin * pow(10.0, (20.0 / 9.0) * tau_prev - 11.0 / 9.0);
+  const double y = (20.0 / 9.0) * tau_prev - 11.0 / 9.0;
+  // log2 10 to 106 bits
+  const double p = fabs(y) < 300.0 ? pow_log2(y, 3.321928094887362, 1.661617516973592e-16) : pow(10.0, y);
+  return (double)d.prm.gamma_base * d.w_bin * p;
 }
 
 }  // namespace hp

@@ -65,28 +65,87 @@ __device__ double sum_slot(const Dev &d, int c, int slot, int n, double *sm) {
   return out[0];
 }
 
-// Step length, momentum and lambda schedule of iteration k (thread 0 only).
-__device__ void advance_scalars(const Dev &d, CopyState *cs, bool first, double g2, double dv2,
-                                double dg2) {
+// Sums of NS slots' partials (n[s] of them) by a whole block, all slots in
+// one pass: their loads, their trees' FP64 steps and their barriers overlap.
+// Fixed order; out[s] valid in every thread.  sm: NS * NT / 32 + NS entries.
+template <int NT, int NS>
+__device__ __forceinline__ void sum_slots_all(const Dev &d, int c, const int (&slots)[NS],
+                                              const int (&n)[NS], double (&out)[NS], double *sm) {
+  const double *p[NS];
+  int nmax = 0;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    p[s] = part_ptr(d, c, slots[s]);
+    out[s] = 0.0;
+    nmax = max(nmax, n[s]);
+  }
+#pragma unroll 2
+  for (int i = threadIdx.x; i < nmax; i += NT) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (i < n[s]) out[s] += __ldcg(p[s] + i);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) out[s] += __shfl_xor_sync(0xffffffffu, out[s], o);
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) sm[s * (NT / 32) + (threadIdx.x >> 5)] = out[s];
+  }
+  __syncthreads();
+  if (threadIdx.x < NS) {
+    double v[NT / 32];
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) v[i] = sm[threadIdx.x * (NT / 32) + i];
+#pragma unroll
+    for (int o = NT / 64; o > 0; o >>= 1) {
+#pragma unroll
+      for (int i = 0; i < o; ++i) v[i] += v[i + o];
+    }
+    sm[NS * (NT / 32) + threadIdx.x] = v[0];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < NS; ++s) out[s] = sm[NS * (NT / 32) + s];
+}
+
+// The schedule's scalars that do not depend on one another, each by a thread
+// of its own warp so that their FP64 chains run side by side: momentum, gamma
+// and (k >= 1) lambda's factor.  Every thread of the block calls it.
+struct NextScalars {
+  double a_next, coef, gamma, mu;
+};
+__device__ __forceinline__ void next_scalars(const Dev &d, const CopyState *cs, bool first,
+                                             double hpwl, NextScalars *s) {
   const place_params &P = d.prm;
-  double alpha;
-  if (first) {
-    double rms = sqrt(g2 / (2.0 * d.n_mov));
-    alpha = rms > 0 ? (double)P.alpha0 * d.w_bin / rms : 0.0;
-  } else {
-    alpha = dg2 > 0 ? sqrt(dv2) / sqrt(dg2) : cs->alpha;
+  if (threadIdx.x == 32) {
+    const double a = cs->a;
+    s->a_next = (1.0 + sqrt(4.0 * a * a + 1.0)) / 2.0;
+    s->coef = (a - 1.0) / s->a_next;
+  } else if (threadIdx.x == 64) {
+    s->gamma = gamma_of(d, cs->tau);
+  } else if (threadIdx.x == 96 && !first) {
+    const double y = 1.0 - (hpwl - cs->hpwl_prev) / d.dref;
+    const double mu = d.lg_mu != 0.0 ? pow_log2(fmin(fmax(y * d.lg_mu, -900.0), 900.0), 1.0, 0.0)
+                                     : pow((double)P.mu_base, y);
+    s->mu = fmin(fmax(mu, (double)P.mu_lo), (double)P.mu_hi);
   }
+}
+
+// Momentum, lambda schedule and gamma after iteration k, whose step length is
+// alpha (thread 0, after a barrier behind next_scalars).
+__device__ __forceinline__ void advance_scalars(CopyState *cs, bool first, double alpha,
+                                                const NextScalars &s) {
   cs->alpha = alpha;
-  cs->a_next = (1.0 + sqrt(4.0 * cs->a * cs->a + 1.0)) / 2.0;
-  cs->coef = (cs->a - 1.0) / cs->a_next;
-  if (!first) {
-    double mu = pow((double)P.mu_base, 1.0 - (cs->hpwl - cs->hpwl_prev) / d.dref);
-    mu = fmin(fmax(mu, (double)P.mu_lo), (double)P.mu_hi);
-    cs->lam *= mu;
-  }
+  cs->a_next = s.a_next;
+  cs->coef = s.coef;
+  if (!first) cs->lam *= s.mu;
   cs->hpwl_prev = cs->hpwl;
   cs->tau_prev = cs->tau;
-  cs->gamma = gamma_of(d, cs->tau);
+  cs->gamma = s.gamma;
 }
 
 // Gradient of the wirelength (the cell's packed fixed-point pin-gradient sum,
@@ -97,8 +156,10 @@ __device__ void advance_scalars(const Dev &d, CopyState *cs, bool first, double 
 // stretched rectangle and scaled by its density scale R / 2^31.
 template <bool STRETCH>
 __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int eval) {
-  __shared__ double smd[32];
-  __shared__ float2 smc[32];
+  __shared__ double smd[6 * (kThreads / 32) + 6];
+  __shared__ float2 smc[3 * (kThreads / 32)];
+  __shared__ double s_pre[3];
+  __shared__ NextScalars s_next;
   __shared__ int flag;
   pdl_wait();
   const int c = copy0 + blockIdx.y;
@@ -128,6 +189,33 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
   float2 pan = zero2, gon = zero2;
   if (full && i < d.n_mov) {
     pan = pa[i]; gon = go[i];
+  }
+  // A large design has thousands of WA partials: each block adds up its share
+  // (a warp, while the loads above are in flight), and the last block sums one
+  // value per block.  Left to the last block alone they are 3.5 us of one SM's
+  // FP64 pipe at 2.1M cells (5163 partials, two values each); at 210k cells
+  // (1925) the blocks' extra FP64 work costs a batched handle what it saves, so
+  // the line lies between.  It does not depend on the number of copies, so that
+  // a copy sums in the same order in every batch.
+  const bool pre = !eval && d.wa_blocks_total > 2048 && gridDim.x >= 64;
+  if (pre && threadIdx.x >= kThreads - 32) {
+    double h = 0.0, w = 0.0, v = 0.0;
+    const int step = gridDim.x * 32, j0 = blockIdx.x + gridDim.x * (threadIdx.x & 31);
+    for (int j = j0; j < d.wa_blocks_total; j += step) {
+      h += part_ptr(d, c, S_HPWL)[j];
+      w += part_ptr(d, c, S_WL)[j];
+    }
+    if (k > 0)
+      for (int j = j0; j < d.cell_blocks; j += step) v += part_ptr(d, c, S_DV2)[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      h += __shfl_xor_sync(0xffffffffu, h, o);
+      w += __shfl_xor_sync(0xffffffffu, w, o);
+      v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    if (threadIdx.x == kThreads - 1) {
+      s_pre[0] = h; s_pre[1] = w; s_pre[2] = v;
+    }
   }
   for (; i < d.n_mov; i += stride) {
     const unsigned long long gs = gsn;
@@ -217,35 +305,52 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
   }
   // per-thread sums in FP32 (a few cells each), compensated block sums:
   // these norms set lambda_0 and every step length
-  const double r0 = block_sum_fc<kThreads>(n1, smc);
-  const double r1 = block_sum_fc<kThreads>(d1, smc);
-  const double r2 = block_sum_fc<kThreads>(dg2, smc);
+  float nv[3] = {n1, d1, dg2};
+  double nr[3];
+  block_sums_fc<kThreads, 3>(nv, smc, nr);
   if (threadIdx.x == 0) {
-    part_ptr(d, c, S_GW1)[blockIdx.x] = r0;
-    part_ptr(d, c, S_GD1)[blockIdx.x] = r1;
-    part_ptr(d, c, S_DG2)[blockIdx.x] = r2;
+    part_ptr(d, c, S_GW1)[blockIdx.x] = nr[0];
+    part_ptr(d, c, S_GD1)[blockIdx.x] = nr[1];
+    part_ptr(d, c, S_DG2)[blockIdx.x] = nr[2];
+    if (pre) {
+      part_ptr(d, c, S_PH)[blockIdx.x] = s_pre[0];
+      part_ptr(d, c, S_PW)[blockIdx.x] = s_pre[1];
+      part_ptr(d, c, S_PV)[blockIdx.x] = s_pre[2];
+    }
   }
   if (eval) return;
-  if (!arrive_last(d.ctr + (size_t)c * C_COUNT + C_CELL, &flag)) return;
-  const int wa_slots[2] = {S_HPWL, S_WL};
-  const int cg_slots[3] = {S_GW1, S_GD1, S_DG2};
-  double wa_sum[2], cg_sum[3];
-  sum_slots<kThreads, 2>(d, c, wa_slots, d.wa_blocks_total, wa_sum, smd);
-  sum_slots<kThreads, 3>(d, c, cg_slots, gridDim.x, cg_sum, smd);
-  // |v_k - v_{k-1}|^2: the partials of the step that led here (k_update or
-  // k_redo_step, one per block of their grid)
-  const double s4 = k > 0 ? sum_slot<kThreads>(d, c, S_DV2, d.cell_blocks, smd) : 0.0;
-  const double hp = wa_sum[0], wl = wa_sum[1];
-  const double s1 = cg_sum[0], s2 = cg_sum[1], s3 = cg_sum[2];
+  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_CELL, &flag)) return;
+  // The serial end of the iteration: k_update waits for it.  Its FP64 work is
+  // spread over the block (all sums in one pass, the scalars on four warps, no
+  // pow): with one sum after another and all scalars on thread 0 an iteration
+  // took 74.6 us at 1k cells, 113 at 210k and 337 at 2.1M; so, 64.0, 100 and
+  // 321.
+  // |v_k - v_{k-1}|^2 (S_DV2): the partials of the step that led here
+  // (k_update or k_redo_step, one per block of their grid)
+  const int ng = gridDim.x;
+  const int slots[6] = {pre ? S_PH : S_HPWL, pre ? S_PW : S_WL, S_GW1, S_GD1, S_DG2, pre ? S_PV : S_DV2};
+  const int cnt[6] = {pre ? ng : d.wa_blocks_total, pre ? ng : d.wa_blocks_total, ng, ng, ng,
+                      k > 0 ? (pre ? ng : d.cell_blocks) : 0};
+  double sum[6];
+  sum_slots_all<kThreads, 6>(d, c, slots, cnt, sum, smd);
+  next_scalars(d, cs, k == 0, sum[0], &s_next);
+  const double s1 = sum[2], s2 = sum[3], s3 = sum[4], s4 = sum[5];
+  double lam0 = 0.0, est = 0.0;
   if (threadIdx.x == 0) {
-    cs->hpwl = hp;
-    cs->wl = wl;
+    if (k == 0)
+      lam0 = s2 > 0 ? (double)d.prm.lambda_eta * s1 / s2 : (double)d.prm.lambda_eta;
+    else
+      est = s3 > 0 ? sqrt(s4) / sqrt(s3) : cs->alpha;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    cs->hpwl = sum[0];
+    cs->wl = sum[1];
     if (k == 0) {
-      cs->lam = s2 > 0 ? (double)d.prm.lambda_eta * s1 / s2 : (double)d.prm.lambda_eta;
+      cs->lam = lam0;
     } else {
       // backtracking: a step-length estimate below 0.95 times the step that
       // led here sends k_update back to redo that step with the estimate
-      const double est = s3 > 0 ? sqrt(s4) / sqrt(s3) : cs->alpha;
       if (d.prm.max_backtracks > 0 && cs->n_back < d.prm.max_backtracks && est < 0.95 * cs->alpha) {
         cs->alpha = est;
         cs->n_back += 1;
@@ -253,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
         cs->reject = 1;
       } else {
         cs->n_back = 0;
-        advance_scalars(d, cs, false, 0.0, s4, s3);
+        advance_scalars(cs, false, est, s_next);
       }
     }
     d.ctr[(size_t)c * C_COUNT + C_CELL] = 0u;
@@ -263,8 +368,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
 // k == 0 only: preconditioned gradient once lambda_0 is known, |g|^2, and the
 // first step length.
 __global__ void __launch_bounds__(kThreads) k_precond0(Dev d, int copy0) {
-  __shared__ double smd[32];
+  __shared__ double smd[kThreads / 32 + 1];
   __shared__ float2 smc[32];
+  __shared__ NextScalars s_next;
   __shared__ int flag;
   pdl_wait();
   const int c = copy0 + blockIdx.y;
@@ -284,10 +390,19 @@ __global__ void __launch_bounds__(kThreads) k_precond0(Dev d, int copy0) {
   }
   const double r = block_sum_fc<kThreads>(g2, smc);
   if (threadIdx.x == 0) part_ptr(d, c, S_G2)[blockIdx.x] = r;
-  if (!arrive_last(d.ctr + (size_t)c * C_COUNT + C_PRE0, &flag)) return;
-  const double s = sum_slot<kThreads>(d, c, S_G2, gridDim.x, smd);
+  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_PRE0, &flag)) return;
+  const int slots[1] = {S_G2}, cnt[1] = {(int)gridDim.x};
+  double s[1];
+  sum_slots_all<kThreads, 1>(d, c, slots, cnt, s, smd);
+  next_scalars(d, cs, true, 0.0, &s_next);
+  double alpha = 0.0;
   if (threadIdx.x == 0) {
-    advance_scalars(d, cs, true, s, 0.0, 0.0);
+    const double rms = sqrt(s[0] / (2.0 * d.n_mov));
+    alpha = rms > 0 ? (double)d.prm.alpha0 * d.w_bin / rms : 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    advance_scalars(cs, true, alpha, s_next);
     d.ctr[(size_t)c * C_COUNT + C_PRE0] = 0u;
   }
 }
@@ -335,7 +450,7 @@ __global__ void __launch_bounds__(kThreads) k_update(Dev d, int copy0) {
   // update knows both points, so v_k need not be stored and read back
   const double r = block_sum_fc<kThreads>(dv2, smc);
   if (threadIdx.x == 0) part_ptr(d, c, S_DV2)[blockIdx.x] = r;
-  if (!arrive_last(d.ctr + (size_t)c * C_COUNT + C_UPDATE, &flag)) return;
+  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_UPDATE, &flag)) return;
   if (threadIdx.x == 0) {
     // the iteration's record: its HPWL (WA pass) and overflow at v_k, the
     // step length taken, and the lambda and gamma the next iteration uses
@@ -388,7 +503,7 @@ __global__ void __launch_bounds__(kThreads) k_redo_step(Dev d, int copy0) {
   }
   const double r = block_sum_fc<kThreads>(dv2, smc);  // the redone step's |v_k - v_{k-1}|^2
   if (threadIdx.x == 0) part_ptr(d, c, S_DV2)[blockIdx.x] = r;
-  if (!arrive_last(d.ctr + (size_t)c * C_COUNT + C_UPDATE, &flag)) return;
+  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_UPDATE, &flag)) return;
   if (threadIdx.x == 0) {
     cs->reject = 0;
     d.ctr[(size_t)c * C_COUNT + C_UPDATE] = 0u;
