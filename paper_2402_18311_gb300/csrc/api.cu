@@ -175,6 +175,18 @@ int resolve_dct_mode(int mode, int nx, int ny) {
   return (nx % 128 == 0 && ny % 128 == 0) ? PLACE_DCT_BF16X3 : PLACE_DCT_FP32;
 }
 
+// The Poisson solve of a grid.  In FP32 mode, and where PLACE_DCT_AUTO and the
+// full split of the transforms (dct_fold) leave it to the library: one cluster
+// for a small grid, else the fast transforms on the sides they take.
+// PLACE_DCT_BF16X3 and dct_fold = 0 ask for the tensor cores' GEMMs.  mode:
+// the caller's, before resolve_dct_mode.
+int choose_solve(int mode, int fold, int nx, int ny) {
+  const bool fp32 = resolve_dct_mode(mode, nx, ny) == PLACE_DCT_FP32;
+  if (fp32 && small_grid(nx, ny)) return SOLVE_SMALL;
+  if (fft_side(nx) && fft_side(ny) && (fp32 || (mode == PLACE_DCT_AUTO && fold))) return SOLVE_FFT;
+  return SOLVE_GEMM;
+}
+
 // The even/odd split of the tensor-core solve: each half of a side must
 // hold whole 128-row tiles (and each half of a contraction whole pairs of
 // 64-element K-blocks), so both sides are multiples of 256.
@@ -207,6 +219,9 @@ struct place_t {
   cudaGraph_t graph0 = nullptr;
   cudaGraphExec_t exec0 = nullptr;
   bool k0_pending = true;
+  // handles with a fused solve: M may hold an evaluation's map and has to be zero
+  // before the next iteration (which leaves it zero itself)
+  bool m_dirty = true;
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
@@ -342,6 +357,12 @@ void layout(Dev &d, Arena &a, int n_copies) {
   d.sel_idx = a.take<unsigned int>(d.sort_n);
   d.px_tmp = a.take<float>(C);
   d.py_tmp = a.take<float>(C);
+  if (d.solve == SOLVE_FFT) {
+    d.fft_wx = a.take<float2>(d.nx);
+    d.fft_wy = a.take<float2>(d.ny);
+    d.fft_cx = a.take<float2>(d.nx);
+    d.fft_cy = a.take<float2>(d.ny);
+  }
   d.err = a.take<int>(4);  // [0]: bounded waits gave up; [1]: a sink for measurement kernels;
                            // [2], [3]: a failed index check (bounds-checking build)
   if (d.tc) {
@@ -538,6 +559,7 @@ int enqueue_reset(place_t *h, int c0, int n) {
   Dev &d = h->d;
   cudaStream_t st = h->stream;
   h->k0_pending = true;  // the next iteration preconditions these copies' first step
+  h->m_dirty = true;
   launch_reset(d, c0, n, st);
   CK(cudaMemsetAsync(d.M + (size_t)c0 * d.Gm, 0, sizeof(unsigned long long) * d.Gm * n, st));
   launch_scatter(d, c0, n, 1, st);
@@ -559,10 +581,11 @@ void enqueue_iteration(const Dev &d, cudaStream_t st, const cudaStream_t *wst, c
   for (int b = 0; b < nb; ++b) cudaStreamWaitEvent(wst[b], fork, 0);
   launch_wa_branches(d, 0, K, wst);
   for (int b = 0; b < nb; ++b) cudaEventRecord(join[b], wst[b]);
-  cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
+  // a fused solve zeroes the map that it has read; the GEMM handles clear it
+  // here (clear_map has the other half of that rule)
+  if (!d.solve) cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
   launch_scatter(d, 0, K, 0, st);
-  launch_density_finish(d, 0, K, FIN_ITER, st);
-  launch_spectral(d, 0, K, 0, 0, st);
+  launch_field(d, 0, K, FIN_ITER, 0, st);
   for (int b = 0; b < nb; ++b) cudaStreamWaitEvent(st, join[b], 0);
   launch_cell_grad(d, 0, K, 0, st);
   if (with_precond0) launch_precond0(d, 0, K, st);
@@ -586,11 +609,22 @@ int ensure_graph(place_t *h) {
   return PLACE_OK;
 }
 
+// On a handle with a fused solve the map is zero before an iteration: cleared here
+// after a call that left one in it, by the iteration itself otherwise.
+cudaError_t clear_map(place_t *h) {
+  const Dev &d = h->d;
+  if (!d.solve || !h->m_dirty) return cudaSuccess;
+  h->m_dirty = false;
+  return cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * d.K, h->stream);
+}
+
 // One iteration of every copy: the graph with the k = 0 preconditioning pass
 // when a reset since the last iteration may have left a copy at k = 0, the
 // one without it otherwise (the two compute the same: the pass does nothing
 // for a copy past k = 0).  ensure_graph must have succeeded.
 cudaError_t launch_iter(place_t *h) {
+  const cudaError_t e = clear_map(h);
+  if (e != cudaSuccess) return e;
   if (h->k0_pending) {
     h->k0_pending = false;
     return cudaGraphLaunch(h->exec0, h->stream);
@@ -687,6 +721,17 @@ void host_dct_tables(int n, double h, std::vector<float> &C, std::vector<float> 
       S[(size_t)k * n + i] = sv;
       ST[(size_t)i * n + k] = sv;
     }
+  }
+}
+
+// w[k] = exp(-2 pi i k / n), c[k] = exp(-i pi k / 2n)
+void host_fft_tables(int n, std::vector<float2> &w, std::vector<float2> &c) {
+  w.resize(n);
+  c.resize(n);
+  for (int k = 0; k < n; ++k) {
+    const double a = 2.0 * M_PI * k / n, b = 0.5 * M_PI * k / n;
+    w[k] = make_float2((float)std::cos(a), (float)-std::sin(a));
+    c[k] = make_float2((float)std::cos(b), (float)-std::sin(b));
   }
 }
 
@@ -819,6 +864,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   if (prm.fillers != 0 && prm.fillers != 1) return fail(PLACE_EINVAL, "fillers must be 0 or 1");
   if (!(prm.macro_precond > 0.f) || !std::isfinite(prm.macro_precond))
     return fail(PLACE_EINVAL, "macro_precond must be positive and finite");
+  const int solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny);
   prm.dct_mode = resolve_dct_mode(prm.dct_mode, bins->nx, bins->ny);
   if (prm.dct_mode != PLACE_DCT_FP32 && prm.dct_mode != PLACE_DCT_BF16X3)
     return fail(PLACE_EINVAL, "unknown dct_mode %d", prm.dct_mode);
@@ -895,6 +941,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.has_net_w = nl->net_w ? 1 : 0;
   d.tc = prm.dct_mode == PLACE_DCT_BF16X3 ? 1 : 0;
   d.bfly = use_fold(d.tc, prm.dct_fold, bins->nx, bins->ny);
+  d.solve = solve;
   h->stream = (cudaStream_t)stream;
 
   // quantised sizes and movable area
@@ -924,6 +971,11 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.n_cells = Ci; d.n_mov = Mo; d.n_real = Mv; d.n_fill = nf;
   d.Gm = nf ? 2 * d.G : d.G;
   d.fill_area_q = (double)nf * (double)fp.Wf * (double)fp.Hf;
+  {
+    double fixed_q = 0.0;
+    for (int i = Mv; i < C; ++i) fixed_q += (double)Wq[i] * (double)Hq[i];
+    d.rho_mean = (float)((d.mov_area_q + d.fill_area_q + d.t * fixed_q) / (d.abin_q * (double)d.G));
+  }
   std::vector<float> wi(Ci), hi(Ci);
   std::vector<int> Wqi(Ci), Hqi(Ci);
   std::vector<unsigned char> macro(Ci, 0);
@@ -1106,7 +1158,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || d.sms <= 0)
       d.sms = 152;
     // the cell-gradient kernel runs as one resident wave (grid-stride)
-    d.cg_blocks = std::max(1, std::min(d.cell_blocks, d.sms * cell_grad_blocks_per_sm()));
+    d.cg_blocks = std::max(1, std::min(d.cell_blocks, d.sms * cell_grad_blocks_per_sm(d.solve)));
   }
   // four blocks per SM: more bins per thread amortise the per-block exact
   // reductions of the density finish (measured on the 2.1M-cell design:
@@ -1114,6 +1166,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   // blocks; 304 blocks were in between)
   d.bin_blocks = std::max(1, std::min((d.G + kThreads - 1) / kThreads, 4 * std::max(d.sms, 1)));
   d.nb_red = std::max(std::max(2 * d.cell_blocks + 2, d.bin_blocks), std::max(d.wa_blocks_total, 1));
+  if (d.solve) d.nb_red = std::max(d.nb_red, std::max(nx / 2, 8));  // blocks of the fused finish
   int sn = 2;
   while (sn < Ci) sn <<= 1;
   d.sort_n = sn;
@@ -1188,6 +1241,15 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     up(d.wv, wv.data(), sizeof(float) * ny);
     up(d.cu, cu.data(), sizeof(float) * nx);
     up(d.cv, cv.data(), sizeof(float) * ny);
+    if (d.solve == SOLVE_FFT) {
+      std::vector<float2> wt, ct;
+      host_fft_tables(nx, wt, ct);
+      up(d.fft_wx, wt.data(), sizeof(float2) * nx);
+      up(d.fft_cx, ct.data(), sizeof(float2) * nx);
+      host_fft_tables(ny, wt, ct);
+      up(d.fft_wy, wt.data(), sizeof(float2) * ny);
+      up(d.fft_cy, ct.data(), sizeof(float2) * ny);
+    }
     if (rc == PLACE_OK && d.bfly)
       rc = upload_fold_tables(d, h->stream, Cn, CTn, STn, Cm, CTm, STm, wu, wv, cu, cv);
   }
@@ -1213,6 +1275,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   if (ce == cudaSuccess)
     ce = cudaMemsetAsync(d.gacc, 0, sizeof(unsigned long long) * (size_t)d.K * std::max(Mo, 1), h->stream);
   if (ce == cudaSuccess && wa_prepare(d.wa_big_cap)) ce = cudaErrorInvalidValue;
+  if (ce == cudaSuccess && d.solve == SOLVE_SMALL && small_prepare()) ce = cudaErrorInvalidValue;
   if (ce == cudaSuccess) ce = cudaMemsetAsync(d.cs, 0, sizeof(CopyState) * d.K, h->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(d.ctr, 0, sizeof(unsigned int) * d.K * C_COUNT, h->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(d.err, 0, 4 * sizeof(int), h->stream);
@@ -1281,7 +1344,9 @@ int place_get_info(const place_t *h, place_info *o) {
   // scatter, finish, 4 GEMMs, WA classes, cell grad, precond0, update; the
   // stretched scatter with density stretching, the step redo with backtracking
   // the steady graph (the first iteration after a reset adds k_precond0)
-  o->kernels_per_iter = 2 + 4 + wa + 2 + (d.Ms ? 1 : 0) + (d.up ? 1 : 0);
+  // (a fused solve has the finish in its three kernels or its one)
+  const int dens = d.solve == SOLVE_FFT ? 1 + 3 : (d.solve == SOLVE_SMALL ? 1 + 1 : 2 + 4);
+  o->kernels_per_iter = dens + wa + 2 + (d.Ms ? 1 : 0) + (d.up ? 1 : 0);
   o->dct_mode = d.tc ? PLACE_DCT_BF16X3 : PLACE_DCT_FP32;
   for (int s = 0; s < 4; ++s) {
     o->gemm_bn[s] = d.tc ? d.tc_bn[s] : 0;
@@ -1352,12 +1417,18 @@ int place_step_timed(place_t *h, int32_t n_iters, float *stage_ms) {
   std::vector<double> acc(PLACE_N_STAGES, 0.0);
   int rc = PLACE_OK;
   for (int it = 0; it < n_iters && rc == PLACE_OK; ++it) {
+    clear_map(h);
     cudaEventRecord(ev[0], st);
-    cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
+    if (!d.solve) cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
     launch_scatter(d, 0, K, 0, st);
-    launch_density_finish(d, 0, K, FIN_ITER, st);
+    // the stages' line within a fused solve: behind the first transform with
+    // the fast transforms, before the one kernel of a small grid
+    if (d.solve == SOLVE_FFT) launch_fft_rows(d, 0, K, FIN_ITER, st);
+    if (d.solve == SOLVE_GEMM) launch_density_finish(d, 0, K, FIN_ITER, st);
     cudaEventRecord(ev[1], st);
-    launch_spectral(d, 0, K, 0, 0, st);
+    if (d.solve == SOLVE_FFT) launch_fft_solve(d, 0, K, 0, 0, st);
+    if (d.solve == SOLVE_GEMM) launch_spectral(d, 0, K, 0, 0, st);
+    if (d.solve == SOLVE_SMALL) launch_solve_small(d, 0, K, FIN_ITER, 0, st);
     cudaEventRecord(ev[2], st);
     launch_wa(d, 0, K, 0, nullptr, st);
     cudaEventRecord(ev[3], st);
@@ -1741,12 +1812,11 @@ int place_eval_wirelength(place_t *h, int32_t copy, float gamma, double *wl, flo
 
 namespace {
 
-int density_at(place_t *h, int copy) {
+int scatter_at(place_t *h, int copy) {
   Dev &d = h->d;
+  h->m_dirty = true;
   CK(cudaMemsetAsync(d.M + (size_t)copy * d.Gm, 0, sizeof(unsigned long long) * d.Gm, h->stream));
   launch_scatter(d, copy, 1, 1, h->stream);
-  launch_density_finish(d, copy, 1, FIN_EVAL, h->stream);
-  CKL();
   return PLACE_OK;
 }
 
@@ -1759,7 +1829,9 @@ int place_eval_density(place_t *h, int32_t copy, int64_t *map, double *overflow)
   int rc = check_copy(h, copy, false);
   if (rc) return rc;
   Dev &d = h->d;
-  if ((rc = density_at(h, copy))) return rc;
+  if ((rc = scatter_at(h, copy))) return rc;
+  launch_density_finish(d, copy, 1, FIN_EVAL, h->stream);
+  CKL();
   if (map) CK(cudaMemcpyAsync(map, d.M + (size_t)copy * d.Gm, sizeof(int64_t) * d.G, cudaMemcpyDefault, h->stream));
   double s = 0;
   CK(cudaMemcpyAsync(&s, d.scal + (size_t)copy * S_COUNT + S_TAU, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -1780,8 +1852,8 @@ int place_eval_field(place_t *h, int32_t copy, float *psi, float *ex, float *ey)
   int rc = check_copy(h, copy, false);
   if (rc) return rc;
   Dev &d = h->d;
-  if ((rc = density_at(h, copy))) return rc;
-  launch_spectral(d, copy, 1, 1, 1, h->stream);
+  if ((rc = scatter_at(h, copy))) return rc;
+  launch_field(d, copy, 1, FIN_EVAL, 1, h->stream);
   CKL();
   const size_t G = d.G;
   const float *E = d.E + (size_t)copy * 3 * G;
@@ -1797,8 +1869,8 @@ int place_eval_density_grad(place_t *h, int32_t copy, float *gx, float *gy) {
   int rc = check_copy(h, copy, false);
   if (rc) return rc;
   Dev &d = h->d;
-  if ((rc = density_at(h, copy))) return rc;
-  launch_spectral(d, copy, 1, 0, 1, h->stream);
+  if ((rc = scatter_at(h, copy))) return rc;
+  launch_field(d, copy, 1, FIN_EVAL, 0, h->stream);
   launch_cell_grad(d, copy, 1, 1, h->stream);
   CKL();
   const size_t Mo = d.n_mov, Mv = d.n_real;  // per-copy stride, the design's movable cells
@@ -1815,6 +1887,7 @@ int place_eval_hpwl_overflow(place_t *h, double *hpwl, double *overflow) {
   const int K = d.K;
   launch_hpwl64(d, 0, K, h->stream);
   launch_reduce_slot(d, S_HP64, d.cell_blocks + 2 * std::max(d.cell_blocks / 2, 1), 0, K, h->stream);
+  h->m_dirty = true;
   CK(cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, h->stream));
   launch_scatter(d, 0, K, 1, h->stream);
   launch_density_finish(d, 0, K, FIN_EVAL, h->stream);
@@ -1998,6 +2071,7 @@ extern "C" int place_estimate_device_bytes(const place_netlist *nl, const place_
   d.nx = bins->nx; d.ny = bins->ny; d.G = bins->nx * bins->ny;
   d.Gm = nf ? 2 * d.G : d.G;
   d.has_net_w = nl->net_w ? 1 : 0;
+  d.solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny);
   prm.dct_mode = resolve_dct_mode(prm.dct_mode, bins->nx, bins->ny);
   d.tc = prm.dct_mode == PLACE_DCT_BF16X3 ? 1 : 0;
   d.bfly = use_fold(d.tc, prm.dct_fold, bins->nx, bins->ny);

@@ -132,7 +132,7 @@ struct Timer {
 
 int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut *out) {
   const auto t0 = std::chrono::steady_clock::now();
-  const Key key{d.nx,           d.ny,           d.K,           d.tc,
+  const Key key{d.nx,           d.ny,           d.K,           d.tc + 2 * d.solve,
                 lg2(d.n_mov),   lg2(d.n_pins),  lg2(max_deg),  d.prm.stretch,
                 d.prm.gemm_bn,  d.prm.gemm_split, d.prm.wa_big_cap, d.prm.scatter_mode,
                 d.prm.wa_streams, d.bfly};
@@ -160,7 +160,7 @@ int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut 
   // with the wirelength kernels on the iteration's second stream, so the
   // objective is the whole iteration: each candidate is timed over iterations
   // of the captured graph from the same start.
-  if (d.tc && (d.prm.gemm_bn == 0 || d.prm.gemm_split == 0)) {
+  if (d.tc && !d.solve && (d.prm.gemm_bn == 0 || d.prm.gemm_split == 0)) {
     // tile width per stage, and split-K on the stages with few tiles (the
     // first two, or all four, where the workspace allows it)
     struct Cand { int bn[4], split[4]; };

@@ -11,6 +11,7 @@
 // overflow sum is exact too: with t = m 2^-s (m < 2^24), every bin's excess
 // times 2^s is an integer below 2^100, summed in 128-bit integers.
 #include "common.cuh"
+#include "density_finish.cuh"
 #include "internal.cuh"
 
 namespace hp {
@@ -295,62 +296,6 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// A nonnegative 64-bit integer as FP32 from its two 32-bit halves (two fast
-// conversions and one FMA instead of the multi-instruction 64-bit one; the
-// result may differ from the correctly rounded one in the last bit).
-__device__ __forceinline__ float u64_to_float(unsigned long long v) {
-  return fmaf((float)(unsigned int)(v >> 32), 4294967296.0f, (float)(unsigned int)v);
-}
-
-// Excess contribution of one bin: bins without fixed cells are counted into
-// (m_over, n_over) and closed after the loop; the others are summed exactly
-// in 128 bits.
-__device__ __forceinline__ void bin_excess(const Dev &d, unsigned long long m, long long f, u128 tA,
-                                           u128 &acc, unsigned long long &m_over,
-                                           unsigned int &n_over) {
-  if (f == 0) {
-    if (m > d.tA_floor) {
-      m_over += m;
-      ++n_over;
-    }
-  } else {
-    // excess * 2^s = m 2^s + t_mant F - t_mant A: exact in unsigned 128
-    // bits (below 2^124, and valid when overlapping fixed cells make F > A)
-    u128 lhs = (u128)m << d.t_shift;
-    lhs += (u128)(unsigned long long)d.t_mant * (u128)(unsigned long long)f;
-    if (lhs > tA) acc += lhs - tA;
-  }
-}
-
-// One pair of bins (2 b2, 2 b2 + 1): their excess into the sums and rho.
-template <bool STRETCH>
-__device__ __forceinline__ float2 finish_pair(const Dev &d, int c, int b2, const ulonglong2 *M2,
-                                              const ulonglong2 *Mf2, const longlong2 *F2,
-                                              u128 tA, float inv_a, float tf, u128 &acc,
-                                              unsigned long long &m_over, unsigned int &n_over,
-                                              float &q2) {
-  const ulonglong2 m = M2[b2];
-  const longlong2 f = F2[b2];
-  float mq0 = u64_to_float(m.x) * inv_a, mq1 = u64_to_float(m.y) * inv_a;
-  if (Mf2) {
-    const ulonglong2 mf = Mf2[b2];
-    mq0 = u64_to_float(m.x + mf.x) * inv_a;
-    mq1 = u64_to_float(m.y + mf.y) * inv_a;
-  }
-  q2 = fmaf(mq0, mq0, q2);
-  q2 = fmaf(mq1, mq1, q2);
-  bin_excess(d, m.x, f.x, tA, acc, m_over, n_over);
-  bin_excess(d, m.y, f.y, tA, acc, m_over, n_over);
-  float mf0 = mq0, mf1 = mq1;
-  if constexpr (STRETCH) {
-    const ulonglong2 ms = reinterpret_cast<const ulonglong2 *>(d.Ms + (size_t)c * d.G)[b2];
-    mf0 = u64_to_float(ms.x) * inv_a;
-    mf1 = u64_to_float(ms.y) * inv_a;
-  }
-  return make_float2(fmaf(tf, u64_to_float((unsigned long long)f.x) * inv_a, mf0),
-                     fmaf(tf, u64_to_float((unsigned long long)f.y) * inv_a, mf1));
-}
-
 __device__ __forceinline__ void store_bf16_pair(__nv_bfloat16 *hp, __nv_bfloat16 *lp, size_t b2,
                                                 float v0, float v1) {
   const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
@@ -359,51 +304,32 @@ __device__ __forceinline__ void store_bf16_pair(__nv_bfloat16 *hp, __nv_bfloat16
   reinterpret_cast<__nv_bfloat162 *>(lp)[b2] = lo;
 }
 
-// Per bin: exact overflow excess and rho in FP32; the last block of each copy
-// reduces the excess and, by mode, records the overflow as the iteration's
-// tau (with the stop test), as an evaluation result, or as the reset value
-// tau_{-1} that sets the first gamma.  STRETCH: rho comes from the
-// stretched map (density stretching on); the overflow always from M.  Two
+// Per bin: exact overflow excess and rho in FP32 (density_finish.cuh has both
+// and what the last block does with the overflow).  STRETCH: rho comes from
+// the stretched map (density stretching on); the overflow always from M.  Two
 // bins per thread and step (G is even): 16-byte loads and paired bf16
 // conversions and stores.  FOLD (the even/odd split of the tensor-core
 // solve): four bins per step, (x, y), (x, y+1) and their mirrors
 // (x, ny-1-y), (x, ny-2-y), and rho leaves as the sums rho_y + rho_{ny-1-y}
-// at y and the differences at ny/2 + y (y < ny/2).
+// at y and the differences at ny/2 + y (y < ny/2).  Handles with a fused
+// solve form rho there and come here for the overflow alone.
 template <bool STRETCH, bool FOLD>
 __global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, int mode) {
-  __shared__ u128 sm[32];
-  __shared__ float smf[32];
-  __shared__ int flag;
+  __shared__ FinishShared fs;
   pdl_wait();
   const int c = copy0 + blockIdx.y;
-  CopyState *cs = d.cs + c;
-  if (mode == FIN_ITER && cs->stopped) return;
-  const ulonglong2 *M2 = reinterpret_cast<const ulonglong2 *>(d.M + (size_t)c * d.Gm);
-  // with fillers their map (following M) joins rho and the concentration
-  const ulonglong2 *Mf2 = d.n_fill ? M2 + (d.G >> 1) : nullptr;
-  const longlong2 *F2 = reinterpret_cast<const longlong2 *>(d.Fmap);
-  const u128 tA = ((u128)d.tA_hi << 64) | d.tA_lo;  // t_mant * A_bin
-  const float inv_a = (float)(1.0 / d.abin_q);
-  const float tf = (float)d.t;
-  u128 acc = 0;
-  // bins without fixed cells: their excess times 2^s is m 2^s - t_mant A,
-  // positive exactly when m > floor(t_mant A / 2^s); the sum over those bins
-  // is 2^s (sum of m) - count * t_mant A, formed once after the loop (the
-  // sum of m stays below the movable area, below 2^62)
-  unsigned long long m_over = 0ull;
-  unsigned int n_over = 0u;
-  float q2 = 0.f;
+  if (mode == FIN_ITER && d.cs[c].stopped) return;
+  const FinishArgs fa = finish_args(d, c);
+  BinSums sums;
   if constexpr (FOLD) {
     __nv_bfloat16 *rh = d.rho_h + (size_t)c * d.G, *rl = d.rho_l + (size_t)c * d.G;
     const int q4 = d.ny >> 2, nq = d.G >> 2, hy = d.ny >> 1;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nq; t += gridDim.x * blockDim.x) {
       const int x = t / q4, y = 2 * (t - x * q4);  // y even, below ny/2
       const int row = x * d.ny;
-      const float2 a = finish_pair<STRETCH>(d, c, (row + y) >> 1, M2, Mf2, F2, tA, inv_a, tf, acc,
-                                            m_over, n_over, q2);
+      const float2 a = finish_pair<STRETCH>(d, fa, (row + y) >> 1, sums);
       // bins ny-2-y and ny-1-y
-      const float2 b = finish_pair<STRETCH>(d, c, (row + d.ny - 2 - y) >> 1, M2, Mf2, F2, tA,
-                                            inv_a, tf, acc, m_over, n_over, q2);
+      const float2 b = finish_pair<STRETCH>(d, fa, (row + d.ny - 2 - y) >> 1, sums);
       store_bf16_pair(rh, rl, (size_t)(row + y) >> 1, __fadd_rn(a.x, b.y), __fadd_rn(a.y, b.x));
       store_bf16_pair(rh, rl, (size_t)(row + hy + y) >> 1, __fsub_rn(a.x, b.y),
                       __fsub_rn(a.y, b.x));
@@ -411,50 +337,15 @@ __global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, i
   } else {
     const int G2 = d.G >> 1;
     for (int b2 = blockIdx.x * blockDim.x + threadIdx.x; b2 < G2; b2 += gridDim.x * blockDim.x) {
-      const float2 rv = finish_pair<STRETCH>(d, c, b2, M2, Mf2, F2, tA, inv_a, tf, acc, m_over,
-                                             n_over, q2);
+      const float2 rv = finish_pair<STRETCH>(d, fa, b2, sums);
+      if (d.solve) continue;
       if (d.tc)
         store_bf16_pair(d.rho_h + (size_t)c * d.G, d.rho_l + (size_t)c * d.G, b2, rv.x, rv.y);
       else
         reinterpret_cast<float2 *>(d.rho + (size_t)c * d.G)[b2] = rv;
     }
   }
-  acc += ((u128)m_over << d.t_shift) - (u128)n_over * tA;
-  q2 = block_sum_f<kThreads>(q2, smf);
-  u128 r = block_sum_u128<kThreads>(acc, sm);
-  if (threadIdx.x == 0) {
-    unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + blockIdx.x) * 2;
-    p[0] = (unsigned long long)r;
-    p[1] = (unsigned long long)(r >> 64);
-    d.conc_part[(size_t)c * d.nb_red + blockIdx.x] = q2;
-  }
-  if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_FINISH, &flag)) return;
-  u128 v = 0;
-  q2 = 0.f;
-#pragma unroll 4
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-    const unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + i) * 2;
-    v += ((u128)p[1] << 64) | p[0];
-    q2 += d.conc_part[(size_t)c * d.nb_red + i];
-  }
-  v = block_sum_u128<kThreads>(v, sm);
-  q2 = block_sum_f<kThreads>(q2, smf);
-  if (threadIdx.x == 0) {
-    const double tau = ldexp(u128_to_double(v), -d.t_shift) / d.mov_area_q;
-    const double s1 = (d.mov_area_q + d.fill_area_q) / d.abin_q;
-    if (mode != FIN_EVAL) cs->n_eff = q2 > 0.f ? s1 * s1 / (double)q2 : 0.0;
-    if (mode == FIN_ITER) {
-      cs->tau = tau;
-      if (tau <= (double)d.prm.tau_stop) cs->converged = cs->stopped = 1;
-    } else if (mode == FIN_RESET) {
-      cs->tau = cs->tau_prev = tau;
-      cs->gamma = gamma_of(d, tau);
-      if (d.prm.max_iters <= 0) cs->stopped = 1;
-    } else {
-      d.scal[(size_t)c * S_COUNT + S_TAU] = tau;
-    }
-    d.ctr[(size_t)c * C_COUNT + C_FINISH] = 0u;
-  }
+  finish_reduce<kThreads>(d, c, mode, sums, &fs);
 }
 
 // Floor of the scatter's memory work at the current positions: per movable
@@ -510,11 +401,12 @@ void launch_scatter_fixed(const Dev &d, const float2 *xy, int n0, int n1,
 
 void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st) {
   dim3 grid(d.bin_blocks, ncopy);
-  if (d.Ms && d.bfly)
+  const bool fold = d.bfly && !d.solve;
+  if (d.Ms && fold)
     launch_pdl(k_density_finish<true, true>, grid, dim3(kThreads), 0, st, d, copy0, mode);
   else if (d.Ms)
     launch_pdl(k_density_finish<true, false>, grid, dim3(kThreads), 0, st, d, copy0, mode);
-  else if (d.bfly)
+  else if (fold)
     launch_pdl(k_density_finish<false, true>, grid, dim3(kThreads), 0, st, d, copy0, mode);
   else
     launch_pdl(k_density_finish<false, false>, grid, dim3(kThreads), 0, st, d, copy0, mode);

@@ -65,6 +65,11 @@ enum Counter { C_FINISH = 0, C_CELL, C_PRE0, C_UPDATE, C_COUNT };
 // The density scatter's ways of adding overlaps to the map (density.cu).
 enum ScatterMode { SCAT_MERGED = 0, SCAT_TABLE = 1, SCAT_DIRECT = 2 };
 
+// Poisson solves: tiled GEMMs on the density finish's rho (spectral.cu and, on
+// the tensor cores, spectral_tc.cu), fast transforms (spectral_fft.cu), one
+// cluster for a small grid (spectral_small.cu).
+enum Solve { SOLVE_GEMM = 0, SOLVE_FFT = 1, SOLVE_SMALL = 2 };
+
 // What the density-finish kernel does with the overflow it reduces.
 enum FinishMode { FIN_ITER = 0, FIN_EVAL = 1, FIN_RESET = 2 };
 
@@ -150,6 +155,14 @@ struct Dev {
   float *Cn, *Cm, *CTn, *STn, *STm, *CTm;  // transform matrices
   float *wu, *wv;                          // wavenumbers
   float *cu, *cv;                          // c_k / n factors
+
+  // the Poisson solve the handle runs.  The fused ones (not SOLVE_GEMM) finish
+  // the density pass themselves, keep M zero between density passes and hold
+  // the field as (Ex, Ey) pairs
+  int solve;
+  float rho_mean;           // the mean bin density, up to cells beyond the die
+  float2 *fft_wx, *fft_wy;  // [nx], [ny] exp(-2 pi i k / n)
+  float2 *fft_cx, *fft_cy;  // [nx], [ny] exp(-i pi k / 2n)
 
   // tensor-core spectral path (BF16x3): split operands, host tensor maps
   int tc;
@@ -268,6 +281,17 @@ void launch_pack_xy(float2 *dst, const float *x, const float *y, int n, cudaStre
 void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t st);
 void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st);
 void launch_spectral(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st);
+// Fast transforms: the sides they take; the first kernel (which is also the
+// density finish in mode), and the other two.
+bool fft_side(int n);
+void launch_fft_rows(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st);
+void launch_fft_solve(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st);
+// One cluster per copy: the grids it takes; finish and field in one kernel.
+bool small_grid(int nx, int ny);
+int small_prepare();
+void launch_solve_small(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cudaStream_t st);
+// The density finish and the field behind a scatter, by the handle's solve.
+void launch_field(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cudaStream_t st);
 void launch_spectral_tc_stalled(const Dev &d, cudaStream_t st);
 void launch_test_bounds(const Dev &d, cudaStream_t st);
 void launch_wa(const Dev &d, int copy0, int ncopy, int eval, const float *gamma_override,
@@ -304,7 +328,7 @@ struct TuneHooks {
   void *ctx;
 };
 int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut *out);
-int cell_grad_blocks_per_sm();
+int cell_grad_blocks_per_sm(int solve);
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st);
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st);

@@ -154,7 +154,9 @@ __device__ __forceinline__ void advance_scalars(CopyState *cs, bool first, doubl
 // norms are formed here too, and the last block advances the scalars.
 // STRETCH (density stretching on): the field is gathered over the cell's
 // stretched rectangle and scaled by its density scale R / 2^31.
-template <bool STRETCH>
+// PAIR: the field as (Ex, Ey) pairs (fused solves), one 8-byte load
+// per bin instead of two of 4 bytes from two planes.
+template <bool STRETCH, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int eval) {
   __shared__ double smd[6 * (kThreads / 32) + 6];
   __shared__ float2 smc[3 * (kThreads / 32)];
@@ -173,6 +175,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
   const float2 *xy = d.xy + cn;
   unsigned long long *ga = d.gacc + cm;
   const float *ex = d.E + (size_t)c * 3 * d.G, *ey = ex + d.G;
+  const float2 *exy = reinterpret_cast<const float2 *>(ex);
+  auto field = [&](size_t b) { return PAIR ? exy[b] : make_float2(ex[b], ey[b]); };
   float n1 = 0.f, d1 = 0.f, dg2 = 0.f;
   const float2 *wh = d.wh, *pa = d.pa, *go = d.g[par ^ 1] + cm;
   // every load of the next cell is issued while this cell's field gather is
@@ -263,25 +267,23 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
       if (!HP_IN(d.err, (long long)b0 + (ox1 > 0.f ? d.ny : 0) + (oy1 > 0.f ? 1 : 0), d.G,
                  BS_FIELD_BIN))
         continue;
-      const float e00x = ex[b0], e00y = ey[b0];
-      const float e01x = oy1 > 0.f ? ex[b0 + 1] : 0.f, e01y = oy1 > 0.f ? ey[b0 + 1] : 0.f;
-      const float e10x = ox1 > 0.f ? ex[b0 + d.ny] : 0.f, e10y = ox1 > 0.f ? ey[b0 + d.ny] : 0.f;
       const bool far = ox1 > 0.f && oy1 > 0.f;
-      const float e11x = far ? ex[b0 + d.ny + 1] : 0.f, e11y = far ? ey[b0 + d.ny + 1] : 0.f;
-      dx = -(ox0 * fmaf(oy0, e00x, oy1 * e01x) + ox1 * fmaf(oy0, e10x, oy1 * e11x));
-      dy = -(ox0 * fmaf(oy0, e00y, oy1 * e01y) + ox1 * fmaf(oy0, e10y, oy1 * e11y));
+      const float2 e00 = field(b0), e01 = oy1 > 0.f ? field(b0 + 1) : zero2;
+      const float2 e10 = ox1 > 0.f ? field(b0 + d.ny) : zero2, e11 = far ? field(b0 + d.ny + 1) : zero2;
+      dx = -(ox0 * fmaf(oy0, e00.x, oy1 * e01.x) + ox1 * fmaf(oy0, e10.x, oy1 * e11.x));
+      dy = -(ox0 * fmaf(oy0, e00.y, oy1 * e01.y) + ox1 * fmaf(oy0, e10.y, oy1 * e11.y));
     } else {
       for (int kx = 0, ix = ix0; ix < d.nx && (float)kx * d.fbw < rx1; ++kx, ++ix) {
         const float ox = fminf(rx1, (float)(kx + 1) * d.fbw) - fmaxf(rx, (float)kx * d.fbw);
         if (!(ox > 0.f)) continue;
-        const float *exr = ex + (size_t)ix * d.ny, *eyr = ey + (size_t)ix * d.ny;
         for (int ky = 0, iy = iy0; iy < d.ny && (float)ky * d.fbh < ry1; ++ky, ++iy) {
           const float oy = fminf(ry1, (float)(ky + 1) * d.fbh) - fmaxf(ry, (float)ky * d.fbh);
           if (!(oy > 0.f)) continue;
           const float a = ox * oy;
           if (!HP_IN(d.err, (long long)ix * d.ny + iy, d.G, BS_FIELD_BIN)) continue;
-          dx = fmaf(-a, exr[iy], dx);
-          dy = fmaf(-a, eyr[iy], dy);
+          const float2 e = field((size_t)ix * d.ny + iy);
+          dx = fmaf(-a, e.x, dx);
+          dy = fmaf(-a, e.y, dy);
         }
       }
     }
@@ -565,10 +567,15 @@ void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t
 }
 
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
-  if (d.Ms)
-    launch_pdl(k_cell_grad<true>, dim3(d.cg_blocks, ncopy), dim3(kThreads), 0, st, d, copy0, eval);
+  const dim3 grid(d.cg_blocks, ncopy), block(kThreads);
+  if (d.Ms && d.solve)
+    launch_pdl(k_cell_grad<true, true>, grid, block, 0, st, d, copy0, eval);
+  else if (d.Ms)
+    launch_pdl(k_cell_grad<true, false>, grid, block, 0, st, d, copy0, eval);
+  else if (d.solve)
+    launch_pdl(k_cell_grad<false, true>, grid, block, 0, st, d, copy0, eval);
   else
-    launch_pdl(k_cell_grad<false>, dim3(d.cg_blocks, ncopy), dim3(kThreads), 0, st, d, copy0, eval);
+    launch_pdl(k_cell_grad<false, false>, grid, block, 0, st, d, copy0, eval);
 }
 // One failing index check and no access (place_test_bounds_check).
 __global__ void k_test_bounds(Dev d) {
@@ -579,10 +586,12 @@ __global__ void k_test_bounds(Dev d) {
 }
 void launch_test_bounds(const Dev &d, cudaStream_t st) { k_test_bounds<<<1, 32, 0, st>>>(d); }
 
-int cell_grad_blocks_per_sm() {
+int cell_grad_blocks_per_sm(int solve) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cell_grad<false>, kThreads, 0) != cudaSuccess || n < 1)
-    n = 1;
+  const cudaError_t e =
+      solve ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cell_grad<false, true>, kThreads, 0)
+          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cell_grad<false, false>, kThreads, 0);
+  if (e != cudaSuccess || n < 1) n = 1;
   return n;
 }
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st) {

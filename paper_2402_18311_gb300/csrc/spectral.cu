@@ -248,4 +248,17 @@ void launch_spectral(const Dev &d, int copy0, int ncopy, int with_psi, int eval,
     launch_spectral_fp32(d, copy0, ncopy, with_psi, eval, st);
 }
 
+void launch_field(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cudaStream_t st) {
+  const int eval = mode != FIN_ITER;
+  if (d.solve == SOLVE_SMALL) {
+    launch_solve_small(d, copy0, ncopy, mode, with_psi, st);
+  } else if (d.solve == SOLVE_FFT) {
+    launch_fft_rows(d, copy0, ncopy, mode, st);
+    launch_fft_solve(d, copy0, ncopy, with_psi, eval, st);
+  } else {
+    launch_density_finish(d, copy0, ncopy, mode, st);
+    launch_spectral(d, copy0, ncopy, with_psi, eval, st);
+  }
+}
+
 }  // namespace hp
