@@ -352,9 +352,7 @@ void layout(Dev &d, Arena &a, int n_copies) {
   d.cu = a.take<float>(d.nx);
   d.cv = a.take<float>(d.ny);
   d.bxy = a.take<float2>(K * C);
-  d.sort_key = a.take<unsigned long long>(d.sort_n);
-  d.sort_idx = a.take<unsigned int>(d.sort_n);
-  d.sel_idx = a.take<unsigned int>(d.sort_n);
+  d.sh = a.take<unsigned int>(K * (size_t)d.sh_stride);
   d.px_tmp = a.take<float>(C);
   d.py_tmp = a.take<float>(C);
   if (d.solve == SOLVE_FFT) {
@@ -1167,9 +1165,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.bin_blocks = std::max(1, std::min((d.G + kThreads - 1) / kThreads, 4 * std::max(d.sms, 1)));
   d.nb_red = std::max(std::max(2 * d.cell_blocks + 2, d.bin_blocks), std::max(d.wa_blocks_total, 1));
   if (d.solve) d.nb_red = std::max(d.nb_red, std::max(nx / 2, 8));  // blocks of the fused finish
-  int sn = 2;
-  while (sn < Ci) sn <<= 1;
-  d.sort_n = sn;
+  shuffle_plan(d);
 
   // device memory: one allocation carved into arrays
   Arena a;
@@ -1939,13 +1935,9 @@ int place_perturb(place_t *h, int32_t op, float p, uint64_t seed, int32_t copy) 
   int k = (int)std::floor((double)p * ncand + 0.5);
   k = std::max(0, std::min(k, ncand));
   int c0 = copy < 0 ? 0 : copy, n = copy < 0 ? d.K : 1;
-  for (int c = c0; c < c0 + n; ++c) {
-    uint64_t sd = copy < 0 ? seed + (uint64_t)c : seed;
-    if (k > 0) {
-      launch_shuffle(d, c, op, p, sd, h->stream);
-      launch_shuffle_finish(d, c, k, h->stream);
-      CKL();
-    }
+  if (k > 0) {
+    launch_shuffle(d, c0, n, op, k, seed, h->stream);
+    CKL();
   }
   return enqueue_reset(h, c0, n);
 }
@@ -1993,10 +1985,9 @@ int place_hybro(place_t *h, int32_t n_rounds, int32_t op, float p, uint64_t seed
       }
     }
     if (r < n_rounds) {
-      for (int c = 0; c < K; ++c) {
-        int rc2 = place_perturb(h, op, p, seed + (uint64_t)r * K + c, c);
-        if (rc2) return rc2;
-      }
+      // copy c draws from seed + r K + c
+      const int rc2 = place_perturb(h, op, p, seed + (uint64_t)r * K, -1);
+      if (rc2) return rc2;
     }
   }
   CK(cudaStreamSynchronize(h->stream));
@@ -2079,9 +2070,7 @@ extern "C" int place_estimate_device_bytes(const place_netlist *nl, const place_
   const int cb = std::max(1, std::min((d.n_mov + kThreads - 1) / kThreads, kMaxCellBlocks));
   const int bb = std::max(1, std::min((d.G + kThreads - 1) / kThreads, kMaxCellBlocks));
   d.nb_red = std::max(std::max(2 * cb + 2, bb), 4 * kMaxCellBlocks + kMaxBigNetBlocks);
-  int sn = 2;
-  while (sn < d.n_cells) sn <<= 1;
-  d.sort_n = sn;
+  shuffle_plan(d);
   Arena a;
   layout(d, a, d.K);
   *bytes = (int64_t)(a.off + 256);

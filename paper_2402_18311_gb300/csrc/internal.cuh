@@ -191,11 +191,11 @@ struct Dev {
   int hist_cap;
 
   // perturbation scratch
-  unsigned long long *sort_key;  // [2^ceil(log2 n_cells)]
-  unsigned int *sort_idx;
-  unsigned int *sel_idx;          // [pow2]
+  unsigned int *sh;               // [K][sh_stride] Shuffle's counters (perturb.cu)
+  int sh_lg, sh_nb;               // its buckets: 2^sh_lg = sh_nb
+  int sh_words, sh_tiles;         // words and tiles of its selection mask
+  int sh_stride;
   float *px_tmp, *py_tmp;         // [n_cells]
-  int sort_n;                      // padded length
 
   // WA launch plan: nets [cls_begin[c], cls_begin[c+1]) belong to class c
   int cls_begin[8];
@@ -334,8 +334,8 @@ void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_reset(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_reduce_slot(const Dev &d, int slot, int nvals, int copy0, int ncopy, cudaStream_t st);
-int launch_shuffle(const Dev &d, int copy, int op, float p, uint64_t seed, cudaStream_t st);
-void launch_shuffle_finish(const Dev &d, int copy, int kcount, cudaStream_t st);
+void shuffle_plan(Dev &d);
+void launch_shuffle(const Dev &d, int copy0, int ncopy, int op, int k, uint64_t seed, cudaStream_t st);
 int wm_select_blocks(int G);
 void launch_wiremask(const Dev &d, const WmDev &w, const int *mptr_host, int copy0, int ncopy,
                      cudaStream_t st);

@@ -11,8 +11,18 @@
 //   - taking the selected cells in key order t_0, t_1, ... and in index order
 //     s_0 < s_1 < ..., cell t_j receives the centre of cell s_j, clamped into
 //     the die.  New corners are computed in FP64 and rounded once.
-// Selection and permutation are integer work and bit-exact; they run as a
-// bitonic sort over (key, index) pairs.
+// Selection and permutation are integer work and bit-exact.
+//
+// The keys are the outputs of a bijective 64-bit mix, so they are distinct and
+// spread evenly.  That makes a full sort unnecessary: the cells go to buckets
+// by their key's leading bits (48 to 96 a bucket), only the buckets that start
+// below rank k are kept, and a warp ranks each bucket in shared memory by
+// counting the smaller keys.  The selected cells in index order are a bit mask
+// and its prefix counts.  All copies of a batched handle go through the same
+// launches (blockIdx.y).  What bounds it: the two passes of one L2 atomic per
+// cell.  Against a bitonic sort of (key, index) pairs, one copy after another
+// (324 passes at 210k cells), eight copies of 210k cells restored, shuffled at
+// p = 0.5 and read back: 11.3 -> 0.65 ms.
 #include "common.cuh"
 #include "internal.cuh"
 
@@ -26,63 +36,188 @@ __device__ __forceinline__ unsigned long long splitmix64_at(unsigned long long s
   return z ^ (z >> 31);
 }
 
-constexpr unsigned int kNotCand = 0x80000000u;
+namespace {
 
-__global__ void k_keys(Dev d, int op, unsigned long long seed) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.sort_n; i += gridDim.x * blockDim.x) {
-    bool cand = i < d.n_real && (op == PLACE_SHUFFLE_ALL || d.is_macro[i]);
-    if (cand) {
-      d.sort_key[i] = splitmix64_at(seed, (unsigned long long)i);
-      d.sort_idx[i] = (unsigned int)i;
-    } else {
-      d.sort_key[i] = ~0ull;
-      d.sort_idx[i] = kNotCand | (unsigned int)(i & 0x7fffffff);
+constexpr int kShufBucket = 96;   // most cells a bucket holds on average (at least half of it)
+constexpr int kShufCap = 256;     // keys of a bucket kept in shared memory
+constexpr int kShufTile = 256;    // mask words (of 32 cells) per tile of the prefix counts
+
+// One copy's scratch.  Keys, indices and both orders live in the copy's
+// gradient arrays, whose contents the reset behind the perturbation drops;
+// the counters in d.sh.
+struct Shuf {
+  unsigned long long *key;  // [n_real] bucket by bucket
+  unsigned int *id;         // [n_real]
+  unsigned int *recv;       // [k] receivers in key order
+  unsigned int *donor;      // [k] donors in index order
+  float2 *moved;            // [k] the receivers' new corners
+  unsigned int *start;      // [nb + 1] first rank of each bucket
+  unsigned int *cursor;     // [nb] counts, then the next free slot
+  unsigned int *mask;       // [words] selected cells
+  unsigned int *tile;       // [tiles] selected cells per tile
+};
+__device__ __forceinline__ Shuf shuf(const Dev &d, int c) {
+  const size_t cm = (size_t)c * d.n_mov;
+  unsigned int *w = d.sh + (size_t)c * d.sh_stride;
+  Shuf s;
+  s.key = reinterpret_cast<unsigned long long *>(d.g[0] + cm);
+  s.moved = d.g[1] + cm;
+  s.id = reinterpret_cast<unsigned int *>(d.gwx + cm);
+  s.recv = reinterpret_cast<unsigned int *>(d.gwy + cm);
+  s.donor = reinterpret_cast<unsigned int *>(d.gdx + cm);
+  s.cursor = w;
+  s.mask = w + d.sh_nb;
+  s.tile = s.mask + d.sh_words;
+  s.start = s.tile + d.sh_tiles;
+  return s;
+}
+
+__device__ __forceinline__ unsigned int bucket_of(const Dev &d, unsigned long long key) {
+  return d.sh_lg ? (unsigned int)(key >> (64 - d.sh_lg)) : 0u;
+}
+__device__ __forceinline__ bool candidate(const Dev &d, int op, int i) {
+  return op == PLACE_SHUFFLE_ALL || d.is_macro[i];
+}
+
+__global__ void __launch_bounds__(kThreads) k_shuf_count(Dev d, int copy0, int op, unsigned long long seed) {
+  const Shuf s = shuf(d, copy0 + blockIdx.y);
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < d.n_real; i += gridDim.x * kThreads)
+    if (candidate(d, op, i)) atomicAdd(&s.cursor[bucket_of(d, splitmix64_at(seed + blockIdx.y, i))], 1u);
+}
+
+// Exclusive scan of one value per thread over a block of NT threads.
+template <int NT>
+__device__ __forceinline__ unsigned int block_scan(unsigned int v, unsigned int *sm) {
+  unsigned int x = v;
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (l >= o) x += y;
+  }
+  __syncthreads();
+  if (l == 31) sm[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    unsigned int t = l < NT / 32 ? sm[l] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int y = __shfl_up_sync(0xffffffffu, t, o);
+      if (l >= o) t += y;
     }
+    if (l < NT / 32) sm[l] = t;
+  }
+  __syncthreads();
+  return x - v + (w ? sm[w - 1] : 0u);
+}
+
+// Counts -> first ranks, one block per copy.
+__global__ void __launch_bounds__(1024) k_shuf_scan(Dev d, int copy0) {
+  __shared__ unsigned int sm[32];
+  const Shuf s = shuf(d, copy0 + blockIdx.x);
+  const int per = (d.sh_nb + 1023) / 1024, b0 = threadIdx.x * per;
+  unsigned int sum = 0u;
+  for (int b = b0; b < min(b0 + per, d.sh_nb); ++b) sum += s.cursor[b];
+  unsigned int at = block_scan<1024>(sum, sm);
+  for (int b = b0; b < min(b0 + per, d.sh_nb); ++b) {
+    const unsigned int n = s.cursor[b];
+    s.start[b] = at;
+    s.cursor[b] = at;
+    at += n;
   }
 }
 
-// One compare-exchange pass of a bitonic sort on (key, idx) pairs, ascending.
-__global__ void k_bitonic(unsigned long long *key, unsigned int *idx, int n, int j, int k) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    int p = t ^ j;
-    if (p <= t) continue;
-    unsigned long long ka = key[t], kb = key[p];
-    unsigned int ia = idx[t], ib = idx[p];
-    bool a_gt_b = (ka > kb) || (ka == kb && ia > ib);
-    bool up = (t & k) == 0;
-    if (a_gt_b == up) {
-      key[t] = kb; key[p] = ka;
-      idx[t] = ib; idx[p] = ia;
+// The candidates of every bucket that starts below rank k (the buckets end
+// below n_real, the number of cells).
+__global__ void __launch_bounds__(kThreads)
+    k_shuf_scatter(Dev d, int copy0, int op, unsigned long long seed, unsigned int k) {
+  const Shuf s = shuf(d, copy0 + blockIdx.y);
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < d.n_real; i += gridDim.x * kThreads) {
+    if (!candidate(d, op, i)) continue;
+    const unsigned long long key = splitmix64_at(seed + blockIdx.y, i);
+    const unsigned int b = bucket_of(d, key);
+    if (s.start[b] >= k) continue;
+    unsigned int at = atomicAdd(&s.cursor[b], 1u);
+    HP_FIX(d.err, at, d.n_real, BS_PERM);
+    s.key[at] = key;
+    s.id[at] = (unsigned int)i;
+  }
+}
+
+// One warp per bucket: every cell's rank is its bucket's first rank plus the
+// number of smaller (key, index) pairs in the bucket.
+__global__ void __launch_bounds__(kThreads) k_shuf_rank(Dev d, int copy0, unsigned int k) {
+  __shared__ unsigned long long sk[kThreads / 32][kShufCap];
+  const Shuf s = shuf(d, copy0 + blockIdx.y);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  for (int b = blockIdx.x * (kThreads / 32) + w; b < d.sh_nb; b += gridDim.x * (kThreads / 32)) {
+    const unsigned int at = s.start[b];
+    if (at >= k) break;  // the starts ascend
+    const int n = (int)(s.cursor[b] - at);
+    const unsigned long long *keys = s.key + at;
+    const unsigned int *ids = s.id + at;
+    const bool staged = n <= kShufCap;
+    if (staged) {
+      for (int e = l; e < n; e += 32) sk[w][e] = keys[e];
+      __syncwarp();
     }
-  }
-}
-
-// Index-order copy of the k selected cells (keys = index, padding = max).
-__global__ void k_sel_init(Dev d, int k, int n2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += gridDim.x * blockDim.x) {
-    unsigned int v = i < k ? d.sort_idx[i] : 0xffffffffu;
-    d.sel_idx[i] = v;
-  }
-}
-
-__global__ void k_bitonic_u32(unsigned int *v, int n, int j, int k) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    int p = t ^ j;
-    if (p <= t) continue;
-    unsigned int a = v[t], b = v[p];
-    bool up = (t & k) == 0;
-    if ((a > b) == up) {
-      v[t] = b;
-      v[p] = a;
+    for (int e = l; e < n; e += 32) {
+      const unsigned long long key = keys[e];
+      const unsigned int id = ids[e];
+      unsigned int r = 0u;
+      if (staged) {
+#pragma unroll 8
+        for (int f = 0; f < n; ++f) r += sk[w][f] < key ? 1u : 0u;
+      } else {  // (a bucket far above the mean: the same count from memory)
+        for (int f = 0; f < n; ++f) r += keys[f] < key ? 1u : 0u;
+      }
+      r += at;
+      if (r < k) {
+        s.recv[r] = id;
+        atomicOr(&s.mask[id >> 5], 1u << (id & 31));
+      }
     }
+    __syncwarp();
   }
 }
 
-__global__ void k_shuffle_compute(Dev d, int copy, int k) {
-  const float2 *xy = d.xy + (size_t)copy * d.n_cells;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < k; j += gridDim.x * blockDim.x) {
-    int r = (int)d.sort_idx[j];  // receiver (key order)
-    int s = (int)d.sel_idx[j];   // donor (index order)
+__global__ void __launch_bounds__(kShufTile) k_shuf_tiles(Dev d, int copy0) {
+  __shared__ unsigned int sm[32];
+  const Shuf s = shuf(d, copy0 + blockIdx.y);
+  const int word = blockIdx.x * kShufTile + threadIdx.x;
+  const unsigned int v = word < d.sh_words ? __popc(s.mask[word]) : 0u;
+  const unsigned int before = block_scan<kShufTile>(v, sm);
+  if (threadIdx.x == kShufTile - 1) s.tile[blockIdx.x] = before + v;
+}
+
+// The selected cells in index order: a tile's first position is the sum of
+// the tiles before it.
+__global__ void __launch_bounds__(kShufTile) k_shuf_donors(Dev d, int copy0, unsigned int k) {
+  __shared__ unsigned int sm[32];
+  const Shuf s = shuf(d, copy0 + blockIdx.y);
+  unsigned int sum = 0u;
+  for (int t = threadIdx.x; t < (int)blockIdx.x; t += kShufTile) sum += s.tile[t];
+  const unsigned int part = block_scan<kShufTile>(sum, sm);
+  __shared__ unsigned int base;
+  if (threadIdx.x == kShufTile - 1) base = part + sum;
+  const int word = blockIdx.x * kShufTile + threadIdx.x;
+  unsigned int m = word < d.sh_words ? s.mask[word] : 0u;
+  unsigned int at = block_scan<kShufTile>(__popc(m), sm) + base;  // (its barriers publish base)
+  while (m) {
+    const int bit = __ffs(m) - 1;
+    m &= m - 1;
+    if (at < k) s.donor[at] = (unsigned int)(word * 32 + bit);
+    ++at;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_shuf_move(Dev d, int copy0, int k) {
+  const int c = copy0 + blockIdx.y;
+  const Shuf sh = shuf(d, c);
+  const float2 *xy = d.xy + (size_t)c * d.n_cells;
+  for (int j = blockIdx.x * kThreads + threadIdx.x; j < k; j += gridDim.x * kThreads) {
+    int r = (int)sh.recv[j];   // receiver (key order)
+    int s = (int)sh.donor[j];  // donor (index order)
     HP_FIX(d.err, r, d.n_real, BS_PERM);
     HP_FIX(d.err, s, d.n_real, BS_PERM);
     const float2 ps = xy[s];
@@ -92,47 +227,53 @@ __global__ void k_shuffle_compute(Dev d, int copy, int k) {
     double ny = cy - 0.5 * (double)d.h[r];
     nx = fmax(d.die_xl, fmin(nx, d.die_xh - (double)d.w[r]));
     ny = fmax(d.die_yl, fmin(ny, d.die_yh - (double)d.h[r]));
-    d.px_tmp[j] = (float)nx;
-    d.py_tmp[j] = (float)ny;
+    sh.moved[j] = make_float2((float)nx, (float)ny);
   }
 }
 
-__global__ void k_shuffle_apply(Dev d, int copy, int k) {
-  float2 *xy = d.xy + (size_t)copy * d.n_cells;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < k; j += gridDim.x * blockDim.x) {
-    const int r = (int)d.sort_idx[j];
+__global__ void __launch_bounds__(kThreads) k_shuf_apply(Dev d, int copy0, int k) {
+  const int c = copy0 + blockIdx.y;
+  const Shuf sh = shuf(d, c);
+  float2 *xy = d.xy + (size_t)c * d.n_cells;
+  for (int j = blockIdx.x * kThreads + threadIdx.x; j < k; j += gridDim.x * kThreads) {
+    const int r = (int)sh.recv[j];
     if (!HP_IN(d.err, r, d.n_real, BS_PERM)) continue;
-    xy[r] = make_float2(d.px_tmp[j], d.py_tmp[j]);
+    xy[r] = sh.moved[j];
   }
 }
 
-static int grid_for(int n) {
-  int b = (n + kThreads - 1) / kThreads;
-  return b < 1 ? 1 : (b > 8192 ? 8192 : b);
+int grid_for(int n) {
+  const int b = (n + kThreads - 1) / kThreads;
+  return b < 1 ? 1 : (b > 4096 ? 4096 : b);
 }
 
-// Returns the number of moved cells (>= 0); candidates counted on the host.
-int launch_shuffle(const Dev &d, int copy, int op, float p, uint64_t seed, cudaStream_t st) {
-  const int n = d.sort_n;
-  k_keys<<<grid_for(n), kThreads, 0, st>>>(d, op, (unsigned long long)seed);
-  for (int k = 2; k <= n; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1)
-      k_bitonic<<<grid_for(n / 2 + 1), kThreads, 0, st>>>(d.sort_key, d.sort_idx, n, j, k);
-  return 0;
+}  // namespace
+
+// Buckets, mask words, tiles and 32-bit words of scratch per copy.
+void shuffle_plan(Dev &d) {
+  d.sh_lg = 0;
+  while (((long long)kShufBucket << d.sh_lg) < d.n_real) ++d.sh_lg;
+  d.sh_nb = 1 << d.sh_lg;
+  d.sh_words = (d.n_real + 31) / 32;
+  d.sh_tiles = (d.sh_words + kShufTile - 1) / kShufTile;
+  d.sh_stride = 2 * d.sh_nb + 1 + d.sh_words + d.sh_tiles;
 }
 
-// Second half: given the candidate count, select k and move the cells.
-void launch_shuffle_finish(const Dev &d, int copy, int kcount, cudaStream_t st) {
-  if (kcount <= 0) return;
-  int n2 = 1;
-  while (n2 < kcount) n2 <<= 1;
-  if (n2 < 2) n2 = 2;
-  k_sel_init<<<grid_for(n2), kThreads, 0, st>>>(d, kcount, n2);
-  for (int k = 2; k <= n2; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1)
-      k_bitonic_u32<<<grid_for(n2 / 2 + 1), kThreads, 0, st>>>(d.sel_idx, n2, j, k);
-  k_shuffle_compute<<<grid_for(kcount), kThreads, 0, st>>>(d, copy, kcount);
-  k_shuffle_apply<<<grid_for(kcount), kThreads, 0, st>>>(d, copy, kcount);
+// Shuffle of copies [copy0, copy0 + ncopy): copy copy0 + y draws from seed + y;
+// k (at least 1) of the candidates exchange places.
+void launch_shuffle(const Dev &d, int copy0, int ncopy, int op, int k, uint64_t seed, cudaStream_t st) {
+  const dim3 cells(grid_for(d.n_real), ncopy), sel(grid_for(k), ncopy);
+  const unsigned long long sd = seed;
+  // counts and mask
+  cudaMemsetAsync(d.sh + (size_t)copy0 * d.sh_stride, 0, sizeof(unsigned int) * (size_t)d.sh_stride * ncopy, st);
+  k_shuf_count<<<cells, kThreads, 0, st>>>(d, copy0, op, sd);
+  k_shuf_scan<<<ncopy, 1024, 0, st>>>(d, copy0);
+  k_shuf_scatter<<<cells, kThreads, 0, st>>>(d, copy0, op, sd, (unsigned int)k);
+  k_shuf_rank<<<dim3(grid_for(d.sh_nb * 32), ncopy), kThreads, 0, st>>>(d, copy0, (unsigned int)k);
+  k_shuf_tiles<<<dim3(d.sh_tiles, ncopy), kShufTile, 0, st>>>(d, copy0);
+  k_shuf_donors<<<dim3(d.sh_tiles, ncopy), kShufTile, 0, st>>>(d, copy0, (unsigned int)k);
+  k_shuf_move<<<sel, kThreads, 0, st>>>(d, copy0, k);
+  k_shuf_apply<<<sel, kThreads, 0, st>>>(d, copy0, k);
 }
 
 }  // namespace hp
