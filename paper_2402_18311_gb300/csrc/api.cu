@@ -1882,7 +1882,7 @@ int place_eval_hpwl_overflow(place_t *h, double *hpwl, double *overflow) {
   Dev &d = h->d;
   const int K = d.K;
   launch_hpwl64(d, 0, K, h->stream);
-  launch_reduce_slot(d, S_HP64, d.cell_blocks + 2 * std::max(d.cell_blocks / 2, 1), 0, K, h->stream);
+  launch_reduce_slot(d, S_HP64, d.wa_blocks_total, 0, K, h->stream);
   h->m_dirty = true;
   CK(cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, h->stream));
   launch_scatter(d, 0, K, 1, h->stream);
