@@ -1139,6 +1139,18 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     h->wm_obst.insert(h->wm_obst.end(), mo.begin(), mo.end());
   }
 
+  // cells that may cover more than 32 bins (their size in bins and up to three
+  // more per axis; with stretching every cell is at least sqrt(2) bins)
+  d.has_big = 0;
+  for (int i = 0; i < Mo && !d.has_big; ++i) {
+    double bx = (double)Wqi[i] / (double)d.BW, by = (double)Hqi[i] / (double)d.BH;
+    if (prm.stretch) {
+      bx = std::max(bx, 1.42);
+      by = std::max(by, 1.42);
+    }
+    d.has_big = (bx + 3.0) * (by + 3.0) > 32.0;
+  }
+
   // launch plan
   d.cell_blocks = std::max(1, std::min((Mo + kThreads - 1) / kThreads, kMaxCellBlocks));
   d.wa_blocks_total = 0;
@@ -1156,7 +1168,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || d.sms <= 0)
       d.sms = 152;
     // the cell-gradient kernel runs as one resident wave (grid-stride)
-    d.cg_blocks = std::max(1, std::min(d.cell_blocks, d.sms * cell_grad_blocks_per_sm(d.solve)));
+    d.cg_blocks = std::max(1, std::min(d.cell_blocks, d.sms * cell_grad_blocks_per_sm(d)));
   }
   // four blocks per SM: more bins per thread amortise the per-block exact
   // reductions of the density finish (measured on the 2.1M-cell design:

@@ -74,15 +74,102 @@ __device__ __forceinline__ unsigned long long warp_sum_u42(unsigned long long a)
 // change; always adding directly: 0.151 / 0.064, but 0.271 at iteration 55).
 constexpr int kMaxMergeGroups = 4;
 
+// A copy without a density pass behind it (a reset: n_eff = 0) has no such
+// measure.  Its blocks then look at their first 256 cells: how many of them
+// share the bin of their lower-left corner with a lower lane of their warp.
+// With N equally full bins that is 3968 / N on average, so 3 or fewer stand
+// for a spread copy, up to 86 (N = 32) for a concentrated one.  The
+// reset pass of a spread 2.1M-cell copy: 141 -> 112 us; of the 20k-cell design
+// with stretching (whose map merges 3 x 3 slots the same way): 105 -> 60.
+constexpr int kSampleDirect = 3, kSampleTable = 86;
+
+// Cells with more bins than this are left to the whole warp, a bin per lane.
+constexpr int kWarpBins = 32;
+
+// What the scatter adds for a cell: its rectangle, and with STRETCH (density
+// stretching, ePlace's local smoothing: the map that drives the field when it
+// is on) the stretched rectangle (create-time offsets and sizes in d.st) and
+// each term scaled to floor(ov R / 2^31), R = d.sR[i] <= 2^31: ov = q 2^31 + r
+// gives q R + floor(r R / 2^31), exact in 64 bits.
+template <bool STRETCH>
+struct ScatterCell {
+  QRect32 r;
+  unsigned int R;
+  __device__ __forceinline__ void load(const Dev &d, const float2 *xy, int i) {
+    const float2 v = xy[i];
+    if constexpr (STRETCH) {
+      const int4 st = d.st[i];  // {x shift, y shift, stretched W, stretched H}
+      R = d.sR[i];
+      r = qrect32(v.x, v.y, st.z, st.w, d.scale, d.XL + st.x, d.YL + st.y, d.BW32, d.BH32, d.nx,
+                  d.ny, d.ibw_q, d.ibh_q);
+    } else {
+      r = qrect32(v.x, v.y, d.Wq[i], d.Hq[i], d.scale, d.XL, d.YL, d.BW32, d.BH32, d.nx, d.ny,
+                  d.ibw_q, d.ibh_q);
+    }
+  }
+  __device__ __forceinline__ void none() {
+    r.x0 = r.x1 = r.y0 = r.y1 = 0;
+    r.ix0 = r.iy0 = 0;
+    r.ix1 = r.iy1 = -1;
+    R = 0u;
+  }
+  __device__ __forceinline__ int bins() const {
+    return r.ix0 <= r.ix1 && r.iy0 <= r.iy1 ? (r.ix1 - r.ix0 + 1) * (r.iy1 - r.iy0 + 1) : 0;
+  }
+  __device__ __forceinline__ unsigned long long term(const Dev &d, int ix, int iy) const {
+    const long long ov =
+        (long long)overlap32(r.x0, r.x1, ix, d.BW32) * overlap32(r.y0, r.y1, iy, d.BH32);
+    if constexpr (STRETCH) {
+      const unsigned long long o = (unsigned long long)ov;
+      return (o >> 31) * R + (((o & 0x7fffffffull) * R) >> 31);
+    } else {
+      return (unsigned long long)ov;
+    }
+  }
+};
+
+// The cells of a warp that cover more than kWarpBins bins (movable macros), one
+// after another by the whole warp: every lane takes every 32nd bin, straight
+// to the map (a cell's bins are distinct, so nothing contends).  Left to its
+// one lane, a macro of 17 x 17 bins held a pass of the 210k-cell mixed-size
+// design for 250 us instead of BIGMEASURE.
+template <bool STRETCH>
+__device__ __forceinline__ void scatter_big(const Dev &d, const ScatterCell<STRETCH> &cell, int mo,
+                                            unsigned long long *M, int lim) {
+  unsigned int big = __ballot_sync(0xffffffffu, cell.bins() > kWarpBins);
+  while (big) {
+    const int l = __ffs(big) - 1;
+    big &= big - 1;
+    ScatterCell<STRETCH> c;
+    c.r.x0 = __shfl_sync(0xffffffffu, cell.r.x0, l);
+    c.r.x1 = __shfl_sync(0xffffffffu, cell.r.x1, l);
+    c.r.y0 = __shfl_sync(0xffffffffu, cell.r.y0, l);
+    c.r.y1 = __shfl_sync(0xffffffffu, cell.r.y1, l);
+    c.r.ix0 = __shfl_sync(0xffffffffu, cell.r.ix0, l);
+    c.r.ix1 = __shfl_sync(0xffffffffu, cell.r.ix1, l);
+    c.r.iy0 = __shfl_sync(0xffffffffu, cell.r.iy0, l);
+    c.r.iy1 = __shfl_sync(0xffffffffu, cell.r.iy1, l);
+    c.R = __shfl_sync(0xffffffffu, cell.R, l);
+    const int m = __shfl_sync(0xffffffffu, mo, l);
+    const int h = c.r.iy1 - c.r.iy0 + 1, n = c.bins();
+    for (int k = threadIdx.x & 31; k < n; k += 32) {
+      const int ix = c.r.ix0 + k / h, iy = c.r.iy0 + k % h;
+      const unsigned long long t = c.term(d, ix, iy);
+      const int b = m + ix * d.ny + iy;
+      if (t && HP_IN(d.err, b, lim, BS_MAP_BIN)) atomicAdd(&M[b], t);
+    }
+  }
+}
+
 // Cells are processed grid-stride, a warp at a time, in one of three ways,
 // chosen per copy from how concentrated the previous density pass was:
 //  * SCAT_MERGED, very dense (the centred start of a placement, where
 //    millions of cells share a few bins): each cell touches at most 2 x 2
-//    bins when it is no larger than a bin; the warp visits those four slots
-//    in lock-step, lanes that hit the same bin are merged with a match/reduce
-//    (exact integer sums), and one lane per distinct bin adds the total to a
-//    shared-memory hash table that is flushed with one 64-bit atomic per
-//    distinct bin;
+//    bins when it is no larger than a bin (3 x 3 stretched); the warp visits
+//    those slots in lock-step, lanes that hit the same bin are merged with a
+//    match/reduce (exact integer sums), and one lane per distinct bin adds the
+//    total to a shared-memory hash table that is flushed with one 64-bit
+//    atomic per distinct bin;
 //  * SCAT_TABLE, concentrated (the middle of a placement, tens to a few
 //    thousand effective bins): every lane adds each term to the block's
 //    shared-memory table without the match, which costs more than the
@@ -90,182 +177,130 @@ constexpr int kMaxMergeGroups = 4;
 //    share a bin;
 //  * SCAT_DIRECT, spread: each lane adds its overlaps straight to the map.
 // Larger cells add their remaining bins through the table in the first two
-// ways.  Every way adds the same integers, so the map is the same.
-__global__ void __launch_bounds__(kThreads) k_scatter(Dev d, int copy0, int eval) {
+// ways, and from kWarpBins bins on go to the whole warp in all three.  Every
+// way adds the same integers, so the map is the same.
+// BIG: the design has cells of more bins.
+template <bool STRETCH, bool BIG>
+__global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int eval) {
   __shared__ int keys[kHash];
   __shared__ unsigned long long vals[kHash];
+  constexpr int SIDE = STRETCH ? 3 : 2;  // merged slots per axis
   pdl_wait();
   const int c = copy0 + blockIdx.y;
   if (!eval && d.cs[c].stopped) return;
-  for (int i = threadIdx.x; i < kHash; i += blockDim.x) {
-    keys[i] = -1;
-    vals[i] = 0ull;
-  }
-  __syncthreads();
   const float2 *xy = d.xy + (size_t)c * d.n_cells;
-  unsigned long long *M = d.M + (size_t)c * d.Gm;
-  const int stride = gridDim.x * blockDim.x;
+  // with fillers their map follows the movable one (bin b at G + b); the
+  // stretched map holds both
+  unsigned long long *M = STRETCH ? d.Ms + (size_t)c * d.G : d.M + (size_t)c * d.Gm;
+  const int lim = STRETCH ? d.G : d.Gm;
+  const int stride = gridDim.x * blockDim.x, lane = threadIdx.x & 31;
   const double n_eff = d.cs[c].n_eff;
-  // map index of cell i's bin b: b for a movable cell, G + b for a filler
-  // (the fillers' map follows the movable one)
-  const int mode = d.scat_force >= 0 ? d.scat_force
-                                     : (n_eff < d.scat_t1 ? SCAT_MERGED
-                                                          : (n_eff < d.scat_t2 ? SCAT_TABLE : SCAT_DIRECT));
+  int mode = d.scat_force >= 0 ? d.scat_force
+                               : (n_eff < d.scat_t1 ? SCAT_MERGED
+                                                    : (n_eff < d.scat_t2 ? SCAT_TABLE : SCAT_DIRECT));
+  if (d.scat_force < 0 && n_eff == 0.0) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int b = -1 - lane;  // distinct where there is no cell
+    if (i < d.n_mov) {
+      ScatterCell<STRETCH> cell;
+      cell.load(d, xy, i);
+      if (cell.bins()) b = cell.r.ix0 * d.ny + cell.r.iy0;
+    }
+    const int shared = __syncthreads_count(lane != __ffs(__match_any_sync(0xffffffffu, b)) - 1);
+    mode = shared <= kSampleDirect ? SCAT_DIRECT : (shared <= kSampleTable ? SCAT_TABLE : SCAT_MERGED);
+  }
   if (mode == SCAT_DIRECT) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n_mov; i += stride) {
-      const int mo = i < d.n_real ? 0 : d.G;
-      const float2 v = xy[i];
-      const QRect32 r = qrect32(v.x, v.y, d.Wq[i], d.Hq[i], d.scale, d.XL, d.YL, d.BW32, d.BH32,
-                                d.nx, d.ny, d.ibw_q, d.ibh_q);
-      for (int ix = r.ix0; ix <= r.ix1; ++ix) {
-        const int ox = overlap32(r.x0, r.x1, ix, d.BW32);
-        if (ox == 0) continue;
-        for (int iy = r.iy0; iy <= r.iy1; ++iy) {
-          const int oy = overlap32(r.y0, r.y1, iy, d.BH32);
-          if (oy == 0) continue;
-          const int b = mo + ix * d.ny + iy;
-          if (HP_IN(d.err, b, d.Gm, BS_MAP_BIN))
-            atomicAdd(&M[b], (unsigned long long)((long long)ox * oy));
+    // (warp-uniform trip count here and below)
+    for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < d.n_mov; i0 += stride) {
+      const int i = i0 + lane;
+      const int mo = (STRETCH || i < d.n_real) ? 0 : d.G;
+      ScatterCell<STRETCH> cell;
+      if (i < d.n_mov) cell.load(d, xy, i);
+      else cell.none();
+      if (!BIG || cell.bins() <= kWarpBins) {
+        for (int ix = cell.r.ix0; ix <= cell.r.ix1; ++ix) {
+          for (int iy = cell.r.iy0; iy <= cell.r.iy1; ++iy) {
+            const unsigned long long t = cell.term(d, ix, iy);
+            const int b = mo + ix * d.ny + iy;
+            if (t && HP_IN(d.err, b, lim, BS_MAP_BIN)) atomicAdd(&M[b], t);
+          }
         }
       }
+      if constexpr (BIG) scatter_big(d, cell, mo, M, lim);
     }
     return;
   }
-  if (mode == SCAT_TABLE) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n_mov; i += stride) {
-      const int mo = i < d.n_real ? 0 : d.G;
-      const float2 v = xy[i];
-      const QRect32 r = qrect32(v.x, v.y, d.Wq[i], d.Hq[i], d.scale, d.XL, d.YL, d.BW32, d.BH32,
-                                d.nx, d.ny, d.ibw_q, d.ibh_q);
-      for (int ix = r.ix0; ix <= r.ix1; ++ix) {
-        const int ox = overlap32(r.x0, r.x1, ix, d.BW32);
-        if (ox == 0) continue;
-        for (int iy = r.iy0; iy <= r.iy1; ++iy) {
-          const int oy = overlap32(r.y0, r.y1, iy, d.BH32);
-          if (oy == 0) continue;
-          hash_add(keys, vals, M, mo + ix * d.ny + iy, (unsigned long long)((long long)ox * oy),
-                   d.err, d.Gm);
-        }
-      }
-    }
-  } else {
-  // one cell's overlap with one bin is at most the bin area
-  const bool two_limbs = (double)d.BW * (double)d.BH < 4398046511104.0;  // 2^42
-  // warp-uniform trip count
-  for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < d.n_mov; i0 += stride) {
-    const int i = i0 + (threadIdx.x & 31);
-    const bool valid = i < d.n_mov;
-    const int mo = i < d.n_real ? 0 : d.G;
-    QRect32 r;
-    if (valid) {
-      const float2 v = xy[i];
-      r = qrect32(v.x, v.y, d.Wq[i], d.Hq[i], d.scale, d.XL, d.YL, d.BW32, d.BH32, d.nx, d.ny,
-                  d.ibw_q, d.ibh_q);
-    } else {
-      r.x0 = r.x1 = r.y0 = r.y1 = 0;
-      r.ix0 = r.iy0 = 0;
-      r.ix1 = r.iy1 = -1;
-    }
-#pragma unroll
-    for (int sl = 0; sl < 4; ++sl) {
-      const int ix = r.ix0 + (sl & 1), iy = r.iy0 + (sl >> 1);
-      int b = -1;
-      unsigned long long a = 0ull;
-      if (ix <= r.ix1 && iy <= r.iy1) {
-        const int ox = overlap32(r.x0, r.x1, ix, d.BW32);
-        const int oy = overlap32(r.y0, r.y1, iy, d.BH32);
-        a = (unsigned long long)((long long)ox * oy);
-        if (a != 0ull) b = mo + ix * d.ny + iy;
-      }
-      // one full-warp reduction per bin shared by several lanes (a per-group
-      // mask would serialise the groups inside every reduction); each
-      // group's lowest lane keeps the total, then all of them add at once:
-      // alone on its bin straight to the map, shared through the block table
-      const unsigned int mask = __match_any_sync(0xffffffffu, b);
-      const int lane = threadIdx.x & 31;
-      const bool lead = b >= 0 && lane == __ffs(mask) - 1;
-      const bool shared = __popc(mask) > 1;
-      unsigned int groups = __ballot_sync(0xffffffffu, lead && shared);
-      if (__popc(groups) > kMaxMergeGroups) {
-        // many small groups: one reduction per group would cost more than
-        // the few same-address conflicts of adding every term to the table
-        if (b >= 0) hash_add(keys, vals, M, b, a, d.err, d.Gm);
-        continue;
-      }
-      unsigned long long tot = a;
-      while (groups) {
-        const int l = __ffs(groups) - 1;
-        groups &= groups - 1;
-        const int key = __shfl_sync(0xffffffffu, b, l);
-        const unsigned long long mine = b == key ? a : 0ull;
-        const unsigned long long t =
-            two_limbs ? warp_sum_u42(mine) : group_sum_u64(0xffffffffu, mine);
-        if (lane == l) tot = t;
-      }
-      if (lead) {
-        if (shared)
-          hash_add(keys, vals, M, b, tot, d.err, d.Gm);
-        else if (HP_IN(d.err, b, d.Gm, BS_MAP_BIN))
-          atomicAdd(&M[b], tot);
-      }
-    }
-    // bins beyond the first 2 x 2 (cells larger than a bin)
-    if (valid && (r.ix1 - r.ix0 > 1 || r.iy1 - r.iy0 > 1)) {
-      for (int ix = r.ix0; ix <= r.ix1; ++ix) {
-        const int ox = overlap32(r.x0, r.x1, ix, d.BW32);
-        if (ox == 0) continue;
-        for (int iy = r.iy0; iy <= r.iy1; ++iy) {
-          if (ix - r.ix0 <= 1 && iy - r.iy0 <= 1) continue;  // done above
-          const int oy = overlap32(r.y0, r.y1, iy, d.BH32);
-          if (oy == 0) continue;
-          hash_add(keys, vals, M, mo + ix * d.ny + iy, (unsigned long long)((long long)ox * oy),
-                   d.err, d.Gm);
-        }
-      }
-    }
-  }
-  }  // SCAT_MERGED
-  __syncthreads();
-  for (int i = threadIdx.x; i < kHash; i += blockDim.x) {
-    int k = keys[i];
-    if (k >= 0) atomicAdd(&M[k], vals[i]);
-  }
-}
-
-// Density stretching (ePlace local smoothing): the map that drives the field
-// when it is on.  Every movable cell enters as its stretched rectangle
-// (create-time offsets and sizes in d.st) and each (cell, bin) term is
-// floor(ov R / 2^31) with the cell's fixed-point scale R = d.sR[i] <= 2^31:
-// ov = q 2^31 + r gives q R + floor(r R / 2^31), exact in 64 bits.  Terms go
-// through the block's shared-memory table (the centred start is dense).
-__global__ void __launch_bounds__(kThreads) k_scatter_stretch(Dev d, int copy0, int eval) {
-  __shared__ int keys[kHash];
-  __shared__ unsigned long long vals[kHash];
-  const int c = copy0 + blockIdx.y;
-  if (!eval && d.cs[c].stopped) return;
   for (int i = threadIdx.x; i < kHash; i += blockDim.x) {
     keys[i] = -1;
     vals[i] = 0ull;
   }
   __syncthreads();
-  const float2 *xy = d.xy + (size_t)c * d.n_cells;
-  unsigned long long *M = d.Ms + (size_t)c * d.G;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n_mov; i += gridDim.x * blockDim.x) {
-    const float2 v = xy[i];
-    const int4 st = d.st[i];  // {x shift, y shift, stretched W, stretched H}
-    const unsigned long long R = d.sR[i];
-    const QRect32 r = qrect32(v.x, v.y, st.z, st.w, d.scale, d.XL + st.x, d.YL + st.y, d.BW32,
-                              d.BH32, d.nx, d.ny, d.ibw_q, d.ibh_q);
-    for (int ix = r.ix0; ix <= r.ix1; ++ix) {
-      const int ox = overlap32(r.x0, r.x1, ix, d.BW32);
-      if (ox == 0) continue;
-      for (int iy = r.iy0; iy <= r.iy1; ++iy) {
-        const int oy = overlap32(r.y0, r.y1, iy, d.BH32);
-        if (oy == 0) continue;
-        const unsigned long long ov = (unsigned long long)((long long)ox * oy);
-        const unsigned long long t = (ov >> 31) * R + (((ov & 0x7fffffffull) * R) >> 31);
-        if (t) hash_add(keys, vals, M, ix * d.ny + iy, t, d.err, d.G);
+  // one cell's overlap with one bin is at most the bin area
+  const bool two_limbs = (double)d.BW * (double)d.BH < 4398046511104.0;  // 2^42
+  for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < d.n_mov; i0 += stride) {
+    const int i = i0 + lane;
+    const int mo = (STRETCH || i < d.n_real) ? 0 : d.G;
+    ScatterCell<STRETCH> cell;
+    if (i < d.n_mov) cell.load(d, xy, i);
+    else cell.none();
+    const bool lone = !BIG || cell.bins() <= kWarpBins;  // added by its own lane
+    int done = 0;  // slots per axis that the merge has added
+    if (mode == SCAT_MERGED) {
+      done = SIDE;
+#pragma unroll STRETCH ? 1 : 4
+      for (int sl = 0; sl < SIDE * SIDE; ++sl) {
+        const int ix = cell.r.ix0 + sl % SIDE, iy = cell.r.iy0 + sl / SIDE;
+        int b = -1;
+        unsigned long long a = 0ull;
+        if (lone && ix <= cell.r.ix1 && iy <= cell.r.iy1) {
+          a = cell.term(d, ix, iy);
+          if (a != 0ull) b = mo + ix * d.ny + iy;
+        }
+        // one full-warp reduction per bin shared by several lanes (a per-group
+        // mask would serialise the groups inside every reduction); each
+        // group's lowest lane keeps the total, then all of them add at once:
+        // alone on its bin straight to the map, shared through the block table
+        const unsigned int mask = __match_any_sync(0xffffffffu, b);
+        const bool lead = b >= 0 && lane == __ffs(mask) - 1;
+        const bool shared = __popc(mask) > 1;
+        unsigned int groups = __ballot_sync(0xffffffffu, lead && shared);
+        if (__popc(groups) > kMaxMergeGroups) {
+          // many small groups: one reduction per group would cost more than
+          // the few same-address conflicts of adding every term to the table
+          if (b >= 0) hash_add(keys, vals, M, b, a, d.err, lim);
+          continue;
+        }
+        unsigned long long tot = a;
+        while (groups) {
+          const int l = __ffs(groups) - 1;
+          groups &= groups - 1;
+          const int key = __shfl_sync(0xffffffffu, b, l);
+          const unsigned long long mine = b == key ? a : 0ull;
+          const unsigned long long t =
+              two_limbs ? warp_sum_u42(mine) : group_sum_u64(0xffffffffu, mine);
+          if (lane == l) tot = t;
+        }
+        if (lead) {
+          if (shared)
+            hash_add(keys, vals, M, b, tot, d.err, lim);
+          else if (HP_IN(d.err, b, lim, BS_MAP_BIN))
+            atomicAdd(&M[b], tot);
+        }
       }
+    }
+    // all bins through the table, or those beyond the merged slots
+    if (lone && (cell.r.ix1 - cell.r.ix0 >= done || cell.r.iy1 - cell.r.iy0 >= done)) {
+      for (int ix = cell.r.ix0; ix <= cell.r.ix1; ++ix) {
+        for (int iy = cell.r.iy0; iy <= cell.r.iy1; ++iy) {
+          if (ix - cell.r.ix0 < done && iy - cell.r.iy0 < done) continue;  // done above
+          const unsigned long long t = cell.term(d, ix, iy);
+          if (t) hash_add(keys, vals, M, mo + ix * d.ny + iy, t, d.err, lim);
+        }
+      }
+    }
+    if constexpr (BIG) {
+      __syncwarp();
+      scatter_big(d, cell, mo, M, lim);
     }
   }
   __syncthreads();
@@ -378,16 +413,24 @@ void launch_scatter_floor(const Dev &d, int copy0, int ncopy, cudaStream_t st) {
   k_scatter_floor<<<dim3(d.cell_blocks, ncopy), kThreads, 0, st>>>(d, copy0);
 }
 
+template <bool STRETCH>
+static void scatter(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
+  const dim3 grid(d.cell_blocks, ncopy);
+  if (d.has_big)
+    k_scatter<STRETCH, true><<<grid, kThreads, 0, st>>>(d, copy0, eval);
+  else
+    k_scatter<STRETCH, false><<<grid, kThreads, 0, st>>>(d, copy0, eval);
+}
+
 void launch_scatter_main(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
-  k_scatter<<<dim3(d.cell_blocks, ncopy), kThreads, 0, st>>>(d, copy0, eval);
+  scatter<false>(d, copy0, ncopy, eval, st);
 }
 
 void launch_scatter(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
-  dim3 grid(d.cell_blocks, ncopy);
-  k_scatter<<<grid, kThreads, 0, st>>>(d, copy0, eval);
+  scatter<false>(d, copy0, ncopy, eval, st);
   if (d.Ms) {
     cudaMemsetAsync(d.Ms + (size_t)copy0 * d.G, 0, sizeof(unsigned long long) * d.G * ncopy, st);
-    k_scatter_stretch<<<grid, kThreads, 0, st>>>(d, copy0, eval);
+    scatter<true>(d, copy0, ncopy, eval, st);
   }
 }
 

@@ -120,6 +120,7 @@ struct Dev {
   int *Wq, *Hq;      // [n_cells] quantised sizes
   float2 *pa;        // [n_mov] (pin count, charge area) per movable cell: the preconditioner's terms
   unsigned char *is_macro;  // [n_cells]
+  int has_big;       // some optimiser cell may cover more than 32 bins
   // density stretching (null when off): per movable cell {x shift, y shift,
   // stretched W, stretched H} in fixed point, the density scale R (2^31 = 1),
   // and the stretched map that drives the field
@@ -328,7 +329,7 @@ struct TuneHooks {
   void *ctx;
 };
 int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut *out);
-int cell_grad_blocks_per_sm(int solve);
+int cell_grad_blocks_per_sm(const Dev &d);
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st);
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st);

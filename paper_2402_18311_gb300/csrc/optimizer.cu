@@ -154,9 +154,16 @@ __device__ __forceinline__ void advance_scalars(CopyState *cs, bool first, doubl
 // norms are formed here too, and the last block advances the scalars.
 // STRETCH (density stretching on): the field is gathered over the cell's
 // stretched rectangle and scaled by its density scale R / 2^31.
+// Cells of more bins than kWarpGather (movable macros) are gathered by the
+// whole warp: left to one lane, a macro of 17 x 17 bins held the
+// stage for 110 us instead of 28 on the 210k-cell mixed-size design.
+constexpr float kWarpGather = 32.f;
+
 // PAIR: the field as (Ex, Ey) pairs (fused solves), one 8-byte load
 // per bin instead of two of 4 bytes from two planes.
-template <bool STRETCH, bool PAIR>
+// BIG: the design has such cells (the other designs' kernel is 15% faster
+// without the warp-wide step).
+template <bool STRETCH, bool PAIR, bool BIG>
 __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int eval) {
   __shared__ double smd[6 * (kThreads / 32) + 6];
   __shared__ float2 smc[3 * (kThreads / 32)];
@@ -221,7 +228,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
       s_pre[0] = h; s_pre[1] = w; s_pre[2] = v;
     }
   }
-  for (; i < d.n_mov; i += stride) {
+  // (BIG: a warp's lanes stay together to the last cell)
+  for (; i - (BIG ? (int)(threadIdx.x & 31) : 0) < d.n_mov; i += stride) {
+    const bool valid = BIG ? i < d.n_mov : true;
     const unsigned long long gs = gsn;
     const float2 vi = vnext;
     const float wi = whn.x, hi = whn.y;
@@ -235,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
         pan = pa[in]; gon = go[in];
       }
     }
-    ga[i] = 0ull;
+    if (valid) ga[i] = 0ull;
     const float2 sw = unpack_grad(d, gs);
     const float sx = sw.x, sy = sw.y;
     // density gradient: -sum_b |cell ∩ b| E_b over the bins the cell covers,
@@ -243,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
     // subtractions, so each overlap keeps FP32 relative precision)
     const float xi = vi.x, yi = vi.y;
     float xg = xi, yg = yi, wg = wi, hg = hi, scale_g = 1.f;
-    if constexpr (STRETCH) {
+    if (STRETCH && valid) {
       const int4 st = d.st[i];
       xg = xi - (float)st.x * d.inv_scale;
       yg = yi - (float)st.y * d.inv_scale;
@@ -256,7 +265,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
     const float rx = xg - (d.fxl + (float)ix0 * d.fbw), ry = yg - (d.fyl + (float)iy0 * d.fbh);
     const float rx1 = rx + wg, ry1 = ry + hg;
     float dx = 0.f, dy = 0.f;
-    if (wg <= d.fbw && hg <= d.fbh) {
+    const bool wide = valid && !(wg <= d.fbw && hg <= d.fbh);
+    // bins per axis, rounded up or one more (0 for a cell that is not on the grid)
+    float nbx = 0.f, nby = 0.f;
+    if constexpr (BIG) {
+      nbx = rx1 > 0.f ? fminf(rx1 * d.fibw, 8192.f) + 1.f : 0.f;
+      nby = ry1 > 0.f ? fminf(ry1 * d.fibh, 8192.f) + 1.f : 0.f;
+    }
+    const bool big = BIG && wide && nbx * nby > kWarpGather;
+    if (valid && !wide) {
       // no larger than a bin: at most the 2 x 2 bins from (ix0, iy0), the
       // far ones loaded only where the cell reaches them
       const float ox0 = fmaxf(fminf(rx1, d.fbw) - fmaxf(rx, 0.f), 0.f);
@@ -264,15 +281,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
       const float ox1 = ix0 + 1 < d.nx ? fmaxf(rx1 - d.fbw, 0.f) : 0.f;
       const float oy1 = iy0 + 1 < d.ny ? fmaxf(ry1 - d.fbh, 0.f) : 0.f;
       const size_t b0 = (size_t)ix0 * d.ny + iy0;
-      if (!HP_IN(d.err, (long long)b0 + (ox1 > 0.f ? d.ny : 0) + (oy1 > 0.f ? 1 : 0), d.G,
-                 BS_FIELD_BIN))
-        continue;
-      const bool far = ox1 > 0.f && oy1 > 0.f;
-      const float2 e00 = field(b0), e01 = oy1 > 0.f ? field(b0 + 1) : zero2;
-      const float2 e10 = ox1 > 0.f ? field(b0 + d.ny) : zero2, e11 = far ? field(b0 + d.ny + 1) : zero2;
-      dx = -(ox0 * fmaf(oy0, e00.x, oy1 * e01.x) + ox1 * fmaf(oy0, e10.x, oy1 * e11.x));
-      dy = -(ox0 * fmaf(oy0, e00.y, oy1 * e01.y) + ox1 * fmaf(oy0, e10.y, oy1 * e11.y));
-    } else {
+      if (HP_IN(d.err, (long long)b0 + (ox1 > 0.f ? d.ny : 0) + (oy1 > 0.f ? 1 : 0), d.G,
+                BS_FIELD_BIN)) {
+        const bool far = ox1 > 0.f && oy1 > 0.f;
+        const float2 e00 = field(b0), e01 = oy1 > 0.f ? field(b0 + 1) : zero2;
+        const float2 e10 = ox1 > 0.f ? field(b0 + d.ny) : zero2, e11 = far ? field(b0 + d.ny + 1) : zero2;
+        dx = -(ox0 * fmaf(oy0, e00.x, oy1 * e01.x) + ox1 * fmaf(oy0, e10.x, oy1 * e11.x));
+        dy = -(ox0 * fmaf(oy0, e00.y, oy1 * e01.y) + ox1 * fmaf(oy0, e10.y, oy1 * e11.y));
+      }
+    } else if (wide && !big) {
       for (int kx = 0, ix = ix0; ix < d.nx && (float)kx * d.fbw < rx1; ++kx, ++ix) {
         const float ox = fminf(rx1, (float)(kx + 1) * d.fbw) - fmaxf(rx, (float)kx * d.fbw);
         if (!(ox > 0.f)) continue;
@@ -286,6 +303,41 @@ __global__ void __launch_bounds__(kThreads, 3) k_cell_grad(Dev d, int copy0, int
           dy = fmaf(-a, e.y, dy);
         }
       }
+    }
+    if constexpr (BIG) {
+      // cells of more bins (movable macros) one after another by the whole warp,
+      // a bin per lane, in a fixed order
+      unsigned int bigs = __ballot_sync(0xffffffffu, big);
+      while (bigs) {
+        const int l = __ffs(bigs) - 1;
+        bigs &= bigs - 1;
+        const float bx = __shfl_sync(0xffffffffu, rx, l), by = __shfl_sync(0xffffffffu, ry, l);
+        const float bx1 = __shfl_sync(0xffffffffu, rx1, l), by1 = __shfl_sync(0xffffffffu, ry1, l);
+        const int jx = __shfl_sync(0xffffffffu, ix0, l), jy = __shfl_sync(0xffffffffu, iy0, l);
+        const int mx = min((int)__shfl_sync(0xffffffffu, nbx, l) + 1, d.nx - jx);
+        const int my = min((int)__shfl_sync(0xffffffffu, nby, l) + 1, d.ny - jy);
+        float sx = 0.f, sy = 0.f;
+        for (int q = threadIdx.x & 31; q < mx * my; q += 32) {
+          const int kx = q / my, ky = q - kx * my;
+          const float ox = fminf(bx1, (float)(kx + 1) * d.fbw) - fmaxf(bx, (float)kx * d.fbw);
+          const float oy = fminf(by1, (float)(ky + 1) * d.fbh) - fmaxf(by, (float)ky * d.fbh);
+          const size_t bin = (size_t)(jx + kx) * d.ny + jy + ky;
+          if (!(ox > 0.f) || !(oy > 0.f) || !HP_IN(d.err, bin, d.G, BS_FIELD_BIN)) continue;
+          const float2 e = field(bin);
+          sx = fmaf(-ox * oy, e.x, sx);
+          sy = fmaf(-ox * oy, e.y, sy);
+        }
+  #pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          sx += __shfl_xor_sync(0xffffffffu, sx, o);
+          sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        }
+        if ((threadIdx.x & 31) == l) {
+          dx = sx;
+          dy = sy;
+        }
+      }
+      if (!valid) break;  // the warp's last step
     }
     if constexpr (STRETCH) {
       dx *= scale_g;
@@ -566,16 +618,21 @@ void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t
   k_unpack_xy<<<b < 4096 ? b : 4096, kThreads, 0, st>>>(x, y, src, n);
 }
 
+namespace {
+using CellGrad = void (*)(Dev, int, int);
+CellGrad cell_grad_kernel(bool stretch, bool pair, bool big) {
+  static const CellGrad k[2][2][2] = {
+      {{k_cell_grad<false, false, false>, k_cell_grad<false, false, true>},
+       {k_cell_grad<false, true, false>, k_cell_grad<false, true, true>}},
+      {{k_cell_grad<true, false, false>, k_cell_grad<true, false, true>},
+       {k_cell_grad<true, true, false>, k_cell_grad<true, true, true>}}};
+  return k[stretch][pair][big];
+}
+}  // namespace
+
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
-  const dim3 grid(d.cg_blocks, ncopy), block(kThreads);
-  if (d.Ms && d.solve)
-    launch_pdl(k_cell_grad<true, true>, grid, block, 0, st, d, copy0, eval);
-  else if (d.Ms)
-    launch_pdl(k_cell_grad<true, false>, grid, block, 0, st, d, copy0, eval);
-  else if (d.solve)
-    launch_pdl(k_cell_grad<false, true>, grid, block, 0, st, d, copy0, eval);
-  else
-    launch_pdl(k_cell_grad<false, false>, grid, block, 0, st, d, copy0, eval);
+  launch_pdl(cell_grad_kernel(d.Ms != nullptr, d.solve != SOLVE_GEMM, d.has_big != 0),
+             dim3(d.cg_blocks, ncopy), dim3(kThreads), 0, st, d, copy0, eval);
 }
 // One failing index check and no access (place_test_bounds_check).
 __global__ void k_test_bounds(Dev d) {
@@ -586,12 +643,12 @@ __global__ void k_test_bounds(Dev d) {
 }
 void launch_test_bounds(const Dev &d, cudaStream_t st) { k_test_bounds<<<1, 32, 0, st>>>(d); }
 
-int cell_grad_blocks_per_sm(int solve) {
+int cell_grad_blocks_per_sm(const Dev &d) {
   int n = 0;
-  const cudaError_t e =
-      solve ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cell_grad<false, true>, kThreads, 0)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cell_grad<false, false>, kThreads, 0);
-  if (e != cudaSuccess || n < 1) n = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &n, cell_grad_kernel(d.prm.stretch != 0, d.solve != SOLVE_GEMM, d.has_big != 0), kThreads,
+          0) != cudaSuccess || n < 1)
+    n = 1;
   return n;
 }
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st) {
