@@ -225,8 +225,7 @@ struct place_t {
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
-  std::vector<int> wm_order, wm_ptr, wm_net, wm_obst;
-  int wm_max_nets = 1;
+  std::vector<int> wm_order, wm_ptr, wm_net, wm_pin_ptr, wm_pin, wm_obst;
   void *wm_mem = nullptr;
   WmDev wm{};
   // one captured graph per (first copy, copies) of a WireMask pass: the pass
@@ -659,22 +658,25 @@ int ensure_wiremask(place_t *h) {
   WmDev &w = h->wm;
   w.n_macros = (int)h->wm_order.size();
   w.n_fixed = d.n_cells - d.n_mov;
-  w.max_nets = h->wm_max_nets;
-  w.nblk = wm_select_blocks(d.G);
+  w.n_entries = (int)h->wm_net.size();
   const size_t K = d.K;
   Arena a;
-  int *order = nullptr, *mptr = nullptr, *mnet = nullptr, *obst = nullptr;
+  int *order = nullptr, *mptr = nullptr, *mnet = nullptr, *obst = nullptr, *pptr = nullptr, *pin = nullptr;
   auto lay = [&]() {
     order = a.take<int>(w.n_macros);
     mptr = a.take<int>(w.n_macros + 1);
     mnet = a.take<int>(std::max<size_t>(h->wm_net.size(), 1));
+    pptr = a.take<int>(h->wm_pin_ptr.size());
+    pin = a.take<int>(std::max<size_t>(h->wm_pin.size(), 1));
     obst = a.take<int>(h->wm_obst.size());
-    w.box = a.take<double>(K * w.max_nets * 8);
-    w.fx = a.take<double>(K * d.nx);
-    w.fy = a.take<double>(K * d.ny);
-    w.bobj = a.take<double>(K * w.nblk);
-    w.bdist = a.take<double>(K * w.nblk);
-    w.bidx = a.take<int>(K * w.nblk);
+    w.sbox = a.take<double>(K * std::max(w.n_entries, 1) * 4);
+    w.f = a.take<double>(K * (d.nx + d.ny));
+    w.dist = a.take<double>(K * (d.nx + d.ny));
+    w.range = a.take<int4>(K * (size_t)(w.n_fixed + w.n_macros));
+    w.bobj = a.take<unsigned long long>(K * d.ny);
+    w.bdist = a.take<unsigned long long>(K * d.ny);
+    w.bidx = a.take<int>(K * d.ny);
+    w.ctr = a.take<unsigned int>(K);
   };
   lay();
   void *mem = nullptr;
@@ -685,7 +687,7 @@ int ensure_wiremask(place_t *h) {
   a = Arena();
   a.base = (char *)mem;
   lay();
-  w.order = order; w.mptr = mptr; w.mnet = mnet; w.obst = obst;
+  w.order = order; w.mptr = mptr; w.mnet = mnet; w.obst = obst; w.mpin_ptr = pptr; w.mpin = pin;
   auto up = [&](int *dst, const std::vector<int> &src) -> int {
     if (!src.empty())
       CK(cudaMemcpyAsync(dst, src.data(), sizeof(int) * src.size(), cudaMemcpyHostToDevice, h->stream));
@@ -694,7 +696,11 @@ int ensure_wiremask(place_t *h) {
   int rc = up(order, h->wm_order);
   if (!rc) rc = up(mptr, h->wm_ptr);
   if (!rc) rc = up(mnet, h->wm_net);
+  if (!rc) rc = up(pptr, h->wm_pin_ptr);
+  if (!rc) rc = up(pin, h->wm_pin);
   if (!rc) rc = up(obst, h->wm_obst);
+  if (!rc && (e = cudaMemsetAsync(w.ctr, 0, sizeof(unsigned int) * K, h->stream)) != cudaSuccess)
+    rc = fail(PLACE_ECUDA, "WireMask scratch: %s", cudaGetErrorString(e));
   if (rc) {  // the next WireMask call starts over
     cudaFreeAsync(h->wm_mem, h->stream);
     h->wm_mem = nullptr;
@@ -1133,7 +1139,13 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     for (size_t t = 0; t < mo.size(); ++t) {
       h->wm_net.insert(h->wm_net.end(), nets[t].begin(), nets[t].end());
       h->wm_ptr.push_back((int)h->wm_net.size());
-      h->wm_max_nets = std::max(h->wm_max_nets, (int)nets[t].size());
+    }
+    // each entry's pins on movable macros (the only ones that move in a pass)
+    h->wm_pin_ptr.assign(1, 0);
+    for (int ne : h->wm_net) {
+      for (int j = net_ptr[ne]; j < net_ptr[ne + 1]; ++j)
+        if (pin_cell[j] < Mv && macro[pin_cell[j]]) h->wm_pin.push_back(j);
+      h->wm_pin_ptr.push_back((int)h->wm_pin.size());
     }
     for (int i = Mv; i < C; ++i) h->wm_obst.push_back(ci(i));
     h->wm_obst.insert(h->wm_obst.end(), mo.begin(), mo.end());
@@ -1925,7 +1937,7 @@ int place_perturb(place_t *h, int32_t op, float p, uint64_t seed, int32_t copy) 
         CK(cudaEventRecord(h->ev_fork, h->stream));
         CK(cudaStreamWaitEvent(h->cap, h->ev_fork, 0));
         CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-        launch_wiremask(h->d, h->wm, h->wm_ptr.data(), c0, n, h->cap);
+        launch_wiremask(h->d, h->wm, c0, n, h->cap);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(h->cap, &g);
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);

@@ -217,16 +217,19 @@ struct Dev {
 struct WmDev {
   int n_macros;         // movable macros
   int n_fixed;          // fixed cells: the obstacles every macro avoids
-  int max_nets;         // most nets on one macro (at least 1)
-  int nblk;             // candidate blocks per copy
+  int n_entries;        // nets over all macros: mptr[n_macros]
   const int *order;     // [n_macros] macros by decreasing area, ties by index
-  const int *mptr;      // [n_macros + 1] macro t's nets: mnet[mptr[t] .. mptr[t+1])
-  const int *mnet;      // library net indices, in netlist order per macro
+  const int *mptr;      // [n_macros + 1] macro t's nets: entries mptr[t] .. mptr[t+1]
+  const int *mnet;      // [n_entries] library net indices, in netlist order per macro
+  const int *mpin_ptr;  // [n_entries + 1] entry s's pins on movable macros:
+  const int *mpin;      // mpin[mpin_ptr[s] .. mpin_ptr[s+1]), library pin indices
   const int *obst;      // [n_fixed + n_macros] fixed cells, then `order`
-  double *box;          // [K][max_nets][8] per-net extents of the current macro
-  double *fx, *fy;      // [K][nx], [K][ny] wire-mask axes
-  double *bobj, *bdist; // [K][nblk] per-block winners
-  int *bidx;            // [K][nblk]
+  double *sbox;         // [K][n_entries][4] extents of the entries' other pins
+  double *f, *dist;     // [K][nx + ny] wire-mask axes (columns, rows) and distances
+  int4 *range;          // [K][n_fixed + n_macros] blocked columns and rows
+  unsigned long long *bobj, *bdist;  // [K][ny] the rows' winners
+  int *bidx;            // [K][ny]
+  unsigned int *ctr;    // [K] rows done
 };
 
 // WA gradient sums per movable cell.  Each pin adds its (gx, gy), rounded to
@@ -337,9 +340,7 @@ void launch_reset(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_reduce_slot(const Dev &d, int slot, int nvals, int copy0, int ncopy, cudaStream_t st);
 void shuffle_plan(Dev &d);
 void launch_shuffle(const Dev &d, int copy0, int ncopy, int op, int k, uint64_t seed, cudaStream_t st);
-int wm_select_blocks(int G);
-void launch_wiremask(const Dev &d, const WmDev &w, const int *mptr_host, int copy0, int ncopy,
-                     cudaStream_t st);
+void launch_wiremask(const Dev &d, const WmDev &w, int copy0, int ncopy, cudaStream_t st);
 
 // hooks for the job server (api.cu)
 int step_async(place_t *h, int n, int *stopped_host, cudaEvent_t ev);

@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "internal.cuh"
+#include "pairs.cuh"
 
 namespace hp {
 
@@ -473,55 +474,6 @@ __global__ void __launch_bounds__(kBigNet) k_wa_big(Dev d, int copy0, int cls, i
 // Coordinates are halved first (exact but for subnormals), so that no FP32 sum
 // overflows.  HPWL and
 // overflow of the 2.1M-cell design: 1.44 -> 0.27 ms.
-struct Pair {
-  float s, e;
-};
-__device__ __forceinline__ Pair pin_coord(float v, float o) {
-  Pair p;
-  two_sum(0.5f * v, 0.5f * o, p.s, p.e);
-  return p;
-}
-__device__ __forceinline__ void pair_max(Pair &m, Pair p) {
-  const bool up = p.s > m.s || (p.s == m.s && p.e > m.e);
-  m.s = up ? p.s : m.s;
-  m.e = up ? p.e : m.e;
-}
-__device__ __forceinline__ void pair_min(Pair &m, Pair p) {
-  const bool dn = p.s < m.s || (p.s == m.s && p.e < m.e);
-  m.s = dn ? p.s : m.s;
-  m.e = dn ? p.e : m.e;
-}
-struct PairBox {
-  Pair mx, nx, my, ny;  // maximum and minimum per axis
-};
-__device__ __forceinline__ PairBox empty_box() {
-  const Pair lo{-FLT_MAX, 0.f}, hi{FLT_MAX, 0.f};
-  return PairBox{lo, hi, lo, hi};
-}
-__device__ __forceinline__ void box_add(PairBox &b, float2 v, float2 o) {
-  const Pair x = pin_coord(v.x, o.x), y = pin_coord(v.y, o.y);
-  pair_max(b.mx, x); pair_min(b.nx, x);
-  pair_max(b.my, y); pair_min(b.ny, y);
-}
-__device__ __forceinline__ Pair pair_xor(Pair p, int o) {
-  return Pair{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.e, o)};
-}
-template <int G>
-__device__ __forceinline__ void box_reduce(PairBox &b) {
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) {
-    pair_max(b.mx, pair_xor(b.mx, o)); pair_min(b.nx, pair_xor(b.nx, o));
-    pair_max(b.my, pair_xor(b.my, o)); pair_min(b.ny, pair_xor(b.ny, o));
-  }
-}
-// An FP32 number as FP64 by moving its bits (normal numbers and zero; the
-// conversion instruction is on the FP64 pipe too).
-__device__ __forceinline__ double widen(float f) {
-  const unsigned int u = __float_as_uint(f), x = u & 0x7f800000u;
-  if (x == 0u || x == 0x7f800000u) return (u & 0x7fffffffu) ? (double)f : 0.0;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                          (int)(u << 29));
-}
 __device__ __forceinline__ double extent(Pair hi, Pair lo) {
   return (widen(hi.s) - widen(lo.s)) + (widen(hi.e) - widen(lo.e));
 }

@@ -20,24 +20,40 @@
 // Every value that decides a comparison is FP64 from a fixed sequence of
 // correctly rounded operations (explicit _rn intrinsics, so no contraction
 // into fused multiply-adds), so the result is bit-exact and
-// independent of the launch shape.  Per macro:
-//   - one warp per net computes the net's extents;
-//   - one thread per grid line sums a mask axis;
-//   - each block turns every obstacle into the exact range of candidate
-//     columns and rows it blocks (binary searches); each candidate then
-//     tests integer ranges and takes part in a block argmin;
-//   - a last kernel reduces the blocks' winners and moves the macro.
-// Copies run side by side (blockIdx.y).
+// independent of the launch shape.
+//
+// What bounds it: the chain over the macros, so everything that does not
+// depend on the macros moved before is done once, in parallel, and a macro
+// costs two launches:
+//   - k_wm_static, once per pass: per macro and net, the extent of the net's
+//     pins on other cells than movable macros (a block each; exact FP32 pairs,
+//     pairs.cuh, as FP64 minima and maxima are GB300's slowest instructions);
+//   - k_wm_mask per macro: each net's extent with the macros' pins added (a
+//     short list made at create), the two mask axes with the distances of
+//     their corners, and every obstacle as the exact range of candidate
+//     columns and rows that it blocks (binary searches);
+//   - k_wm_select per macro: a block per row of candidates turns the
+//     obstacles that cover the row into a bit mask, so that a candidate costs
+//     one bit test, one FP64 addition and one comparison; the last block
+//     reduces the rows' winners and moves the macro.
+// Copies run side by side (blockIdx.y).  One pass over 32 macros of a 210k-cell design on 512 x 512
+// bins, restored before and read back: 3.7 -> 0.6 ms against one warp per net in FP64
+// and four launches a macro.  (Launching each kernel early, by
+// griddepcontrol.launch_dependents at its start or before its last step, took
+// 28 us a macro instead of 15: measured, not taken.)
 #include <cmath>
 
 #include "common.cuh"
 #include "internal.cuh"
+#include "pairs.cuh"
 
 namespace hp {
 
 namespace {
 
-constexpr int kWmThreads = 256;
+constexpr int kWmThreads = 128;   // select: threads per row of candidates
+constexpr int kWmLines = 64;      // mask: grid lines (and nets in shared memory) per block
+constexpr int kWmNetThreads = 256;
 
 __device__ __forceinline__ double wm_step(double lo, double hi, int n) {
   return __ddiv_rn(__dsub_rn(hi, lo), (double)n);
@@ -51,261 +67,282 @@ __device__ __forceinline__ double wm_corner(double lo, double hi, int n, int i) 
 }
 
 // First k in [0, n] at which a predicate that is false and then true over
-// [0, n) holds (n when it never does).
+// [0, n) holds (n when it never does), stepping from a guess.
 template <typename P>
-__device__ __forceinline__ int first_true(int n, P pred) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (pred(mid)) hi = mid;
-    else lo = mid + 1;
-  }
-  return lo;
+__device__ __forceinline__ int first_true(int n, int guess, P pred) {
+  int k = min(max(guess, 0), n);
+  while (k > 0 && pred(k - 1)) --k;
+  while (k < n && !pred(k)) ++k;
+  return k;
 }
 
 // The corners i whose macro rectangle [X_i, X_i + w) overlaps [o0, o1) with
 // positive length: X_i < o1 and o0 < X_i + w.  The corners are
 // nondecreasing in i (rounding is monotone), so the first test holds for i
-// below some bound and the second from some bound on.  Two binary searches
-// over the same FP64 expressions give the range [i0, i1] exactly.
+// below some bound and the second from some bound on.  Two searches over the
+// same FP64 expressions, each from an estimate that is at most a corner or two
+// off, give the range [i0, i1] exactly.
 __device__ __forceinline__ int2 blocked_range(double lo, double b, int n, double w, double o0,
                                               double o1) {
-  const int i0 = first_true(n, [&](int i) { return o0 < __dadd_rn(wm_corner_b(lo, b, i), w); });
-  const int i1 = first_true(n, [&](int i) { return !(wm_corner_b(lo, b, i) < o1); }) - 1;
+  const float ib = 1.f / (float)b;
+  const int g0 = (int)floorf(fminf(fmaxf((float)(o0 - w - lo) * ib, -2.f), 16384.f));
+  const int g1 = (int)floorf(fminf(fmaxf((float)(o1 - lo) * ib, -2.f), 16384.f));
+  const int i0 = first_true(n, g0 + 1, [&](int i) { return o0 < __dadd_rn(wm_corner_b(lo, b, i), w); });
+  const int i1 = first_true(n, g1 + 1, [&](int i) { return !(wm_corner_b(lo, b, i) < o1); }) - 1;
   return make_int2(i0, i1);
 }
 
+// A candidate's key, compared as integers: the FP64 objective and distance in
+// an order-preserving form (neither is ever -0), then the candidate's index.
+// no_best() is after every candidate.
 struct Best {
-  double obj, dist;
-  int idx;  // flat candidate index j * nx + i; -1: none
+  unsigned long long obj, dist;
+  int idx;  // flat candidate index j * nx + i
 };
+constexpr int kNoIdx = 0x7fffffff;
+__device__ __forceinline__ Best no_best() { return Best{~0ull, ~0ull, kNoIdx}; }
+
+__device__ __forceinline__ unsigned long long ordered(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  return u ^ ((u >> 63) ? ~0ull : 0x8000000000000000ull);
+}
 
 __device__ __forceinline__ bool better(const Best &a, const Best &b) {
-  if (a.idx < 0) return false;
-  if (b.idx < 0) return true;
   if (a.obj != b.obj) return a.obj < b.obj;
   if (a.dist != b.dist) return a.dist < b.dist;
   return a.idx < b.idx;
 }
 
-__device__ __forceinline__ Best shfl_best(const Best &v, int o) {
-  Best r;
-  r.obj = __shfl_xor_sync(0xffffffffu, v.obj, o);
-  r.dist = __shfl_xor_sync(0xffffffffu, v.dist, o);
-  r.idx = __shfl_xor_sync(0xffffffffu, v.idx, o);
-  return r;
-}
-
-// Block-wide argmin (every thread of the block calls it); result in thread 0.
+// Block-wide minimum (every thread of the block calls it); result in thread 0.
 __device__ Best block_best(Best v) {
-  __shared__ double s_obj[kWmThreads / 32], s_dist[kWmThreads / 32];
-  __shared__ int s_idx[kWmThreads / 32];
+  __shared__ Best sb[kWmThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const Best w = shfl_best(v, o);
+    const Best w{__shfl_xor_sync(0xffffffffu, v.obj, o), __shfl_xor_sync(0xffffffffu, v.dist, o),
+                 __shfl_xor_sync(0xffffffffu, v.idx, o)};
     if (better(w, v)) v = w;
   }
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    s_obj[threadIdx.x >> 5] = v.obj;
-    s_dist[threadIdx.x >> 5] = v.dist;
-    s_idx[threadIdx.x >> 5] = v.idx;
-  }
+  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int k = 1; k < kWmThreads / 32; ++k) {
-      const Best w{s_obj[k], s_dist[k], s_idx[k]};
-      if (better(w, v)) v = w;
-    }
+#pragma unroll
+    for (int k = 1; k < kWmThreads / 32; ++k)
+      if (better(sb[k], v)) v = sb[k];
   }
   return v;
 }
 
-// Extents of every net of macro t: one warp per net.  box[8] =
-// {o-x, o+x, o-y, o+y, d-x, d+x, d-y, d+y}: other pins' coordinates and the
-// macro's own pin offsets (+-inf when empty).
-__global__ void __launch_bounds__(kWmThreads) k_wm_nets(Dev d, WmDev w, int t, int copy0) {
-  const int c = copy0 + blockIdx.y;
+// The extent {x-, x+, y-, y+} of entry s (a macro's net): its pins on other
+// cells than movable macros; +-inf when there are none.
+__global__ void __launch_bounds__(kWmNetThreads) k_wm_static(Dev d, WmDev w, int copy0) {
+  __shared__ PairBox sb[kWmNetThreads / 32];
+  const int c = copy0 + blockIdx.y, s = blockIdx.x;
   const float2 *xy = d.xy + (size_t)c * d.n_cells;
-  const int m = w.order[t];
-  const int nn = w.mptr[t + 1] - w.mptr[t];
-  const int s = blockIdx.x * (kWmThreads / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (s >= nn) return;  // the whole warp leaves together
-  if (!HP_IN(d.err, s, w.max_nets, BS_WM_NET)) return;
-  int e = w.mnet[w.mptr[t] + s];
+  int e = w.mnet[s];
   HP_FIX(d.err, e, d.n_nets, BS_WM_NET);
-  double v[8] = {INFINITY, -INFINITY, INFINITY, -INFINITY,
-                 INFINITY, -INFINITY, INFINITY, -INFINITY};
-  for (int j = d.net_ptr[e] + lane; j < d.net_ptr[e + 1]; j += 32) {
+  PairBox b = empty_box();
+  bool any = false;
+  for (int j = d.net_ptr[e] + threadIdx.x; j < d.net_ptr[e + 1]; j += kWmNetThreads) {
     if (!HP_IN(d.err, j, d.n_pins, BS_WM_NET)) break;
     int cj = d.pin_cell[j];
     HP_FIX(d.err, cj, d.n_cells, BS_WM_CELL);
-    const float2 o = d.pin_off[j];
-    if (cj == m) {
-      v[4] = fmin(v[4], (double)o.x); v[5] = fmax(v[5], (double)o.x);
-      v[6] = fmin(v[6], (double)o.y); v[7] = fmax(v[7], (double)o.y);
-    } else {
-      const float2 p = xy[cj];
-      const double px = __dadd_rn((double)p.x, (double)o.x);
-      const double py = __dadd_rn((double)p.y, (double)o.y);
-      v[0] = fmin(v[0], px); v[1] = fmax(v[1], px);
-      v[2] = fmin(v[2], py); v[3] = fmax(v[3], py);
-    }
+    if (cj < d.n_real && d.is_macro[cj]) continue;
+    box_add(b, xy[cj], d.pin_off[j]);
+    any = true;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-      v[k] = fmin(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-      v[k + 1] = fmax(v[k + 1], __shfl_xor_sync(0xffffffffu, v[k + 1], o));
+  box_reduce<32>(b);
+  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = b;
+  any = __syncthreads_or(any);
+  if (threadIdx.x < 32) {
+    b = sb[threadIdx.x % (kWmNetThreads / 32)];
+    box_reduce<kWmNetThreads / 32>(b);
+    if (threadIdx.x == 0) {
+      double *o = w.sbox + ((size_t)blockIdx.y * w.n_entries + s) * 4;
+      o[0] = any ? pair_value(b.nx) : INFINITY;
+      o[1] = any ? pair_value(b.mx) : -INFINITY;
+      o[2] = any ? pair_value(b.ny) : INFINITY;
+      o[3] = any ? pair_value(b.my) : -INFINITY;
     }
-  }
-  if (lane == 0) {
-    double *b = w.box + ((size_t)blockIdx.y * w.max_nets + s) * 8;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) b[k] = v[k];
   }
 }
 
-// The two axes of macro t's wire mask: thread q < nx sums Fx(X_q), the
-// next ny threads Fy(Y_q), over the macro's nets in order.
-__global__ void __launch_bounds__(kWmThreads) k_wm_profile(Dev d, WmDev w, int t) {
-  const int q = blockIdx.x * kWmThreads + threadIdx.x;
-  if (q >= d.nx + d.ny) return;
-  const bool isx = q < d.nx;
-  const int i = isx ? q : q - d.nx;
-  const double X = isx ? wm_corner(d.die_xl, d.die_xh, d.nx, i) : wm_corner(d.die_yl, d.die_yh, d.ny, i);
-  const int a = isx ? 0 : 2;
-  const int nn = w.mptr[t + 1] - w.mptr[t];
-  const double *box = w.box + (size_t)blockIdx.y * w.max_nets * 8;
-  double acc = 0.0;
-  for (int s = 0; s < nn; ++s) {
-    const double *b = box + (size_t)s * 8;
-    const double hi = fmax(b[a + 1], __dadd_rn(X, b[a + 5]));
-    const double lo = fmin(b[a], __dadd_rn(X, b[a + 4]));
-    const double wn = d.net_w ? (double)d.net_w[w.mnet[w.mptr[t] + s]] : 1.0;
-    acc = __dadd_rn(acc, __dmul_rn(wn, __dsub_rn(hi, lo)));
-  }
-  if (isx) w.fx[(size_t)blockIdx.y * d.nx + i] = acc;
-  else w.fy[(size_t)blockIdx.y * d.ny + i] = acc;
-}
-
-// One thread per candidate: inside the die, free of obstacles, key; the
-// block's best goes to its partial slot.  Each obstacle becomes the range of
-// candidate columns and rows it blocks (blocked_range, one thread per
-// obstacle, staged in shared memory), so a candidate's test is integer
-// compares; with up to one block's worth of obstacles the ranges are
-// formed once per block.
-__global__ void __launch_bounds__(kWmThreads) k_wm_select(Dev d, WmDev w, int t, int copy0) {
-  __shared__ int4 so[kWmThreads];  // blocked columns [x, y], rows [z, w]
+// Macro t.  Blocks [0, lines): kWmLines grid lines each, line q < nx the
+// column Fx(X_q), then the rows Fy(Y_q), summed over the macro's nets in
+// order, and the distance of the corner from the macro's old one (-1: the
+// macro would leave the die).  The other blocks: the obstacles' ranges.
+__global__ void __launch_bounds__(kWmLines) k_wm_mask(Dev d, WmDev w, int t, int copy0, int lines) {
+  __shared__ double box[8][kWmLines];
+  __shared__ double sw[kWmLines];
+  // the tables are the handle's constants: read before the wait
   const int c = copy0 + blockIdx.y;
   const float2 *xy = d.xy + (size_t)c * d.n_cells;
   int m = w.order[t];
   HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
   const double mw = (double)d.w[m], mh = (double)d.h[m];
-  const float2 pm = xy[m];
-  const int nob = w.n_fixed + t;
-  const int G = d.nx * d.ny;
   const double bx = wm_step(d.die_xl, d.die_xh, d.nx), by = wm_step(d.die_yl, d.die_yh, d.ny);
-  const double *fx = w.fx + (size_t)blockIdx.y * d.nx, *fy = w.fy + (size_t)blockIdx.y * d.ny;
-  auto stage = [&](int o0) {
-    if (o0 + (int)threadIdx.x < nob) {
-      int oc = w.obst[o0 + threadIdx.x];
-      HP_FIX(d.err, oc, d.n_cells, BS_WM_CELL);
-      const float2 p = xy[oc];
-      const int2 rx = blocked_range(d.die_xl, bx, d.nx, mw, (double)p.x,
-                                    __dadd_rn((double)p.x, (double)d.w[oc]));
-      const int2 ry = blocked_range(d.die_yl, by, d.ny, mh, (double)p.y,
-                                    __dadd_rn((double)p.y, (double)d.h[oc]));
-      so[threadIdx.x] = make_int4(rx.x, rx.y, ry.x, ry.y);
-    }
-  };
-  const bool once = nob <= kWmThreads;
-  if (once) {
-    stage(0);
-    __syncthreads();
+  if ((int)blockIdx.x >= lines) {
+    const int o = (blockIdx.x - lines) * kWmLines + threadIdx.x;
+    if (o >= w.n_fixed + t) return;
+    int oc = w.obst[o];
+    HP_FIX(d.err, oc, d.n_cells, BS_WM_CELL);
+    const double ow = (double)d.w[oc], oh = (double)d.h[oc];
+    pdl_wait();
+    const float2 p = xy[oc];
+    const int2 rx = blocked_range(d.die_xl, bx, d.nx, mw, (double)p.x, __dadd_rn((double)p.x, ow));
+    const int2 ry = blocked_range(d.die_yl, by, d.ny, mh, (double)p.y, __dadd_rn((double)p.y, oh));
+    w.range[(size_t)blockIdx.y * (w.n_fixed + w.n_macros) + o] = make_int4(rx.x, rx.y, ry.x, ry.y);
+    return;
   }
-  Best best{0.0, 0.0, -1};
-  for (int base = blockIdx.x * kWmThreads; base < G; base += gridDim.x * kWmThreads) {
-    const int q = base + threadIdx.x;
-    bool ok = q < G;
-    int i = 0, j = 0;
-    double X = 0.0, Y = 0.0;
-    if (ok) {
-      j = q / d.nx;
-      i = q - j * d.nx;
-      X = wm_corner_b(d.die_xl, bx, i);
-      Y = wm_corner_b(d.die_yl, by, j);
-      ok = __dadd_rn(X, mw) <= d.die_xh && __dadd_rn(Y, mh) <= d.die_yh;
-    }
-    for (int o0 = 0; o0 < nob; o0 += kWmThreads) {
-      if (!once) {
-        __syncthreads();  // the previous chunk has been read
-        stage(o0);
-        __syncthreads();
+  const int q = blockIdx.x * kWmLines + threadIdx.x;
+  const bool isx = q < d.nx, live = q < d.nx + d.ny;
+  const int i = isx ? q : q - d.nx;
+  const double X = isx ? wm_corner_b(d.die_xl, bx, i) : wm_corner_b(d.die_yl, by, i);
+  const int a = isx ? 0 : 2;
+  const int s0 = w.mptr[t], nn = w.mptr[t + 1] - s0;
+  double acc = 0.0;
+  bool waited = false;
+  for (int n0 = 0; n0 < nn; n0 += kWmLines) {
+    __syncthreads();
+    const int s = s0 + n0 + threadIdx.x;
+    const bool mine = n0 + (int)threadIdx.x < nn;
+    // box: other pins' extent {o-x, o+x, o-y, o+y}, then the macro's own pin
+    // offsets {d-x, d+x, d-y, d+y}
+    double v[8] = {INFINITY, -INFINITY, INFINITY, -INFINITY, INFINITY, -INFINITY, INFINITY, -INFINITY};
+    int k0 = 0, k1 = 0, others = 0;
+    if (mine) {
+      int e = w.mnet[s];
+      HP_FIX(d.err, e, d.n_nets, BS_WM_NET);
+      sw[threadIdx.x] = d.net_w ? (double)d.net_w[e] : 1.0;
+      k0 = w.mpin_ptr[s];
+      k1 = w.mpin_ptr[s + 1];
+      for (int k = k0; k < k1; ++k) {
+        int j = w.mpin[k];
+        HP_FIX(d.err, j, d.n_pins, BS_WM_NET);
+        if (d.pin_cell[j] != m) {
+          ++others;
+          continue;
+        }
+        const float2 of = d.pin_off[j];
+        v[4] = fmin(v[4], (double)of.x); v[5] = fmax(v[5], (double)of.x);
+        v[6] = fmin(v[6], (double)of.y); v[7] = fmax(v[7], (double)of.y);
       }
-      const int cnt = min(kWmThreads, nob - o0);
-      for (int k = 0; ok && k < cnt; ++k) {
-        const int4 r = so[k];
-        if (i >= r.x && i <= r.y && j >= r.z && j <= r.w) ok = false;
+    }
+    if (!waited) pdl_wait();
+    waited = true;
+    if (mine) {
+      const double *o = w.sbox + ((size_t)blockIdx.y * w.n_entries + s) * 4;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = o[k];
+      for (int k = k0; others > 0 && k < k1; ++k) {  // the other macros' pins
+        int j = w.mpin[k];
+        HP_FIX(d.err, j, d.n_pins, BS_WM_NET);
+        int cj = d.pin_cell[j];
+        HP_FIX(d.err, cj, d.n_cells, BS_WM_CELL);
+        if (cj == m) continue;
+        const float2 of = d.pin_off[j], p = xy[cj];
+        const double px = __dadd_rn((double)p.x, (double)of.x), py = __dadd_rn((double)p.y, (double)of.y);
+        v[0] = fmin(v[0], px); v[1] = fmax(v[1], px);
+        v[2] = fmin(v[2], py); v[3] = fmax(v[3], py);
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) box[k][threadIdx.x] = v[k];
+    }
+    __syncthreads();
+    if (live) {
+      const int cnt = min(kWmLines, nn - n0);
+      for (int k = 0; k < cnt; ++k) {
+        const double hi = fmax(box[a + 1][k], __dadd_rn(X, box[a + 5][k]));
+        const double lo = fmin(box[a][k], __dadd_rn(X, box[a + 4][k]));
+        acc = __dadd_rn(acc, __dmul_rn(sw[k], __dsub_rn(hi, lo)));
       }
     }
-    if (ok) {
-      const Best v{__dadd_rn(fx[i], fy[j]),
-                   __dadd_rn(fabs(__dsub_rn(X, (double)pm.x)), fabs(__dsub_rn(Y, (double)pm.y))), q};
+  }
+  if (!waited) pdl_wait();
+  if (live) {
+    const float2 pm = xy[m];
+    const bool in = isx ? __dadd_rn(X, mw) <= d.die_xh : __dadd_rn(X, mh) <= d.die_yh;
+    const double dist = in ? fabs(__dsub_rn(X, isx ? (double)pm.x : (double)pm.y)) : -1.0;
+    const size_t o = (size_t)blockIdx.y * (d.nx + d.ny) + q;
+    w.f[o] = acc;
+    w.dist[o] = dist;
+  }
+}
+
+// Macro t: row j = blockIdx.x of the candidates.
+__global__ void __launch_bounds__(kWmThreads) k_wm_select(Dev d, WmDev w, int t, int copy0) {
+  __shared__ unsigned int blocked[8192 / 32];
+  __shared__ int flag;
+  pdl_wait();
+  const int c = copy0 + blockIdx.y, j = blockIdx.x, nob = w.n_fixed + t;
+  const double *f = w.f + (size_t)blockIdx.y * (d.nx + d.ny);
+  const double *dist = w.dist + (size_t)blockIdx.y * (d.nx + d.ny);
+  const int4 *range = w.range + (size_t)blockIdx.y * (w.n_fixed + w.n_macros);
+  Best best = no_best();
+  const double fy = f[d.nx + j], dy = dist[d.nx + j];
+  if (dy >= 0.0) {  // (the whole block)
+    const int words = (d.nx + 31) / 32;
+    for (int i = threadIdx.x; i < words; i += kWmThreads) blocked[i] = 0u;
+    __syncthreads();
+    for (int o = threadIdx.x; o < nob; o += kWmThreads) {
+      const int4 r = range[o];  // columns [x, y], rows [z, w]
+      if (j < r.z || j > r.w) continue;
+      const int lo = max(r.x, 0), hi = min(r.y, d.nx - 1);
+      for (int k = lo >> 5; k <= hi >> 5 && lo <= hi; ++k) {
+        const unsigned int from = k == lo >> 5 ? 0xffffffffu << (lo & 31) : 0xffffffffu;
+        const unsigned int to = k == hi >> 5 ? 0xffffffffu >> (31 - (hi & 31)) : 0xffffffffu;
+        atomicOr(&blocked[k], from & to);
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < d.nx; i += kWmThreads) {
+      if (blocked[i >> 5] >> (i & 31) & 1u) continue;
+      const double dx = dist[i];
+      if (dx < 0.0) continue;
+      const unsigned long long obj = ordered(__dadd_rn(f[i], fy));
+      if (obj > best.obj) continue;
+      const Best v{obj, ordered(__dadd_rn(dx, dy)), j * d.nx + i};
       if (better(v, best)) best = v;
     }
   }
   best = block_best(best);
   if (threadIdx.x == 0) {
-    const size_t k = (size_t)blockIdx.y * w.nblk + blockIdx.x;
+    const size_t k = (size_t)blockIdx.y * d.ny + j;
     w.bobj[k] = best.obj;
     w.bdist[k] = best.dist;
     w.bidx[k] = best.idx;
   }
-}
-
-// One block per copy: the best of the partial winners moves the macro.
-__global__ void __launch_bounds__(kWmThreads) k_wm_apply(Dev d, WmDev w, int t, int copy0) {
-  const int c = copy0 + blockIdx.x;
-  Best best{0.0, 0.0, -1};
-  for (int k = threadIdx.x; k < w.nblk; k += kWmThreads) {
-    const size_t s = (size_t)blockIdx.x * w.nblk + k;
-    const Best v{w.bobj[s], w.bdist[s], w.bidx[s]};
+  if (!arrive_last_t0(w.ctr + blockIdx.y, &flag)) return;
+  best = no_best();
+  for (int k = threadIdx.x; k < d.ny; k += kWmThreads) {
+    const size_t s = (size_t)blockIdx.y * d.ny + k;
+    const Best v{__ldcg(w.bobj + s), __ldcg(w.bdist + s), __ldcg(w.bidx + s)};
     if (better(v, best)) best = v;
   }
   best = block_best(best);
-  if (threadIdx.x == 0 && best.idx >= 0 && HP_IN(d.err, best.idx, d.nx * d.ny, BS_WM_BIN)) {
-    const int j = best.idx / d.nx, i = best.idx - j * d.nx;
-    int m = w.order[t];
-    HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
-    d.xy[(size_t)c * d.n_cells + m] =
-        make_float2((float)wm_corner(d.die_xl, d.die_xh, d.nx, i),
-                    (float)wm_corner(d.die_yl, d.die_yh, d.ny, j));
+  if (threadIdx.x == 0) {
+    w.ctr[blockIdx.y] = 0u;
+    if (best.idx != kNoIdx && HP_IN(d.err, best.idx, d.nx * d.ny, BS_WM_BIN)) {
+      const int jj = best.idx / d.nx, i = best.idx - jj * d.nx;
+      int m = w.order[t];
+      HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
+      d.xy[(size_t)c * d.n_cells + m] =
+          make_float2((float)wm_corner(d.die_xl, d.die_xh, d.nx, i),
+                      (float)wm_corner(d.die_yl, d.die_yh, d.ny, jj));
+    }
   }
 }
 
 }  // namespace
 
-// Two blocks per SM: each block forms the obstacle ranges once and strides
-// over its candidates.
-int wm_select_blocks(int G) {
-  const int b = (G + kWmThreads - 1) / kWmThreads;
-  return b < 1 ? 1 : (b > 304 ? 304 : b);
-}
-
-void launch_wiremask(const Dev &d, const WmDev &w, const int *mptr_host, int copy0, int ncopy,
-                     cudaStream_t st) {
+void launch_wiremask(const Dev &d, const WmDev &w, int copy0, int ncopy, cudaStream_t st) {
+  if (w.n_entries > 0)
+    k_wm_static<<<dim3(w.n_entries, ncopy), kWmNetThreads, 0, st>>>(d, w, copy0);
+  const int lines = (d.nx + d.ny + kWmLines - 1) / kWmLines;
   for (int t = 0; t < w.n_macros; ++t) {
-    const int nn = mptr_host[t + 1] - mptr_host[t];
-    if (nn > 0)
-      k_wm_nets<<<dim3((nn + kWmThreads / 32 - 1) / (kWmThreads / 32), ncopy), kWmThreads, 0, st>>>(
-          d, w, t, copy0);
-    k_wm_profile<<<dim3((d.nx + d.ny + kWmThreads - 1) / kWmThreads, ncopy), kWmThreads, 0, st>>>(
-        d, w, t);
-    k_wm_select<<<dim3(w.nblk, ncopy), kWmThreads, 0, st>>>(d, w, t, copy0);
-    k_wm_apply<<<ncopy, kWmThreads, 0, st>>>(d, w, t, copy0);
+    const int ranges = (w.n_fixed + t + kWmLines - 1) / kWmLines;
+    launch_pdl(k_wm_mask, dim3(lines + ranges, ncopy), dim3(kWmLines), 0, st, d, w, t, copy0, lines);
+    launch_pdl(k_wm_select, dim3(d.ny, ncopy), dim3(kWmThreads), 0, st, d, w, t, copy0);
   }
 }
 
