@@ -1165,6 +1165,30 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
 
   // launch plan
   d.cell_blocks = std::max(1, std::min((Mo + kThreads - 1) / kThreads, kMaxCellBlocks));
+  {
+    // the scatter table's split: a block's cells (at most 2^lg) times the
+    // largest area that one of them has in one bin (below 2^bits) fit two
+    // 32-bit sums of the areas' low 32 - lg bits and of the rest when
+    // lg + bits - (32 - lg) <= 32
+    const long long step = (long long)d.cell_blocks * kThreads;
+    const long long most = ((Mo + step - 1) / step) * kThreads;
+    int lg = 0;
+    while ((1LL << lg) < most) ++lg;
+    unsigned long long area = 1;
+    for (int i = 0; i < Mo; ++i) {
+      long long w = Wqi[i], hh = Hqi[i];
+      if (prm.stretch) {
+        w = std::max<long long>(w, (long long)std::nearbyint(std::sqrt(2.0) * (double)d.BW));
+        hh = std::max<long long>(hh, (long long)std::nearbyint(std::sqrt(2.0) * (double)d.BH));
+      }
+      area = std::max(area, (unsigned long long)std::min<long long>(w, d.BW) *
+                                (unsigned long long)std::min<long long>(hh, d.BH));
+    }
+    int bits = 0;
+    while (bits < 64 && (area >> bits)) ++bits;
+    d.limb = lg < 32 && 2 * lg + bits <= 64 ? 32 - lg : 0;
+    if (d.limb > 31) d.limb = 31;  // (lg = 0 cannot be: a block is 256 threads)
+  }
   d.wa_blocks_total = 0;
   for (int c = 0; c < 5; ++c) {
     int n = d.cls_begin[c + 1] - d.cls_begin[c];

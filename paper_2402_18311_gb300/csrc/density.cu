@@ -20,10 +20,17 @@ constexpr int kHash = 2048;  // shared-memory aggregation table entries
 
 // Adds one (bin, area) contribution to the block's shared-memory table, or to
 // the global map when its slot is taken (bounded linear probing).  lim: the
-// map's length (checked in the bounds-checking build only).
+// map's length (checked in the bounds-checking build only).  A 64-bit addition
+// in shared memory is a compare-and-swap loop, which lanes on the same bin
+// repeat for one another; 32-bit additions are one instruction.  So an entry
+// holds two 32-bit sums, of the areas' low `limb` bits and of the rest, with
+// limb chosen at create such that a block's cells cannot overflow either
+// (d.limb; 0 where there is no such split: one 64-bit sum).  Density stage of
+// the 2.1M-cell design, the table way: 407 -> 107 us at the dense start; the
+// merged way there, where warps of many bins come here too: 93 -> 83 us.
 __device__ __forceinline__ void hash_add(int *keys, unsigned long long *vals,
                                          unsigned long long *M, int b,
-                                         unsigned long long a, int *err, int lim) {
+                                         unsigned long long a, int limb, int *err, int lim) {
   if (!HP_IN(err, b, lim, BS_MAP_BIN)) return;
   unsigned int hsh = ((unsigned int)b * 2654435761u) >> (32 - 11);
 #pragma unroll 1
@@ -31,7 +38,13 @@ __device__ __forceinline__ void hash_add(int *keys, unsigned long long *vals,
     int k = keys[hsh];  // plain read first: no atomic when the bin is already there
     if (k == -1) k = atomicCAS(&keys[hsh], -1, b);
     if (k == -1 || k == b) {
-      atomicAdd(&vals[hsh], a);
+      if (limb) {
+        unsigned int *v = reinterpret_cast<unsigned int *>(vals + hsh);
+        atomicAdd(v, (unsigned int)a & ((1u << limb) - 1u));
+        atomicAdd(v + 1, (unsigned int)(a >> limb));
+      } else {
+        atomicAdd(&vals[hsh], a);
+      }
       return;
     }
     hsh = (hsh + 1) & (kHash - 1);
@@ -68,11 +81,11 @@ __device__ __forceinline__ unsigned long long warp_sum_u42(unsigned long long a)
 // (set at create, by the autotuner when it runs).
 
 // In the merged path, a warp slot whose lanes form more shared-bin groups
-// than this adds every term to the block table instead.  Measured on the
-// 2.1M-cell design, density stage at iterations 5 / 155: 0.112 / 0.144 ms
-// with per-group reductions always, 0.100 / 0.126 with this cut-off (8: no
-// change; always adding directly: 0.151 / 0.064, but 0.271 at iteration 55).
-constexpr int kMaxMergeGroups = 4;
+// than this adds every term to the block table instead.  Density stage of the
+// 2.1M-cell design at iterations 10 / 170 with at most four groups merged:
+// 0.113 / 0.165 ms, with one: 0.086 / 0.132; every term to the table:
+// 0.111 / 0.107.
+constexpr int kMaxMergeGroups = 1;
 
 // A copy without a density pass behind it (a reset: n_eff = 0) has no such
 // measure.  Its blocks then look at their first 256 cells: how many of them
@@ -267,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int e
         if (__popc(groups) > kMaxMergeGroups) {
           // many small groups: one reduction per group would cost more than
           // the few same-address conflicts of adding every term to the table
-          if (b >= 0) hash_add(keys, vals, M, b, a, d.err, lim);
+          if (b >= 0) hash_add(keys, vals, M, b, a, d.limb, d.err, lim);
           continue;
         }
         unsigned long long tot = a;
@@ -282,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int e
         }
         if (lead) {
           if (shared)
-            hash_add(keys, vals, M, b, tot, d.err, lim);
+            hash_add(keys, vals, M, b, tot, d.limb, d.err, lim);
           else if (HP_IN(d.err, b, lim, BS_MAP_BIN))
             atomicAdd(&M[b], tot);
         }
@@ -294,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int e
         for (int iy = cell.r.iy0; iy <= cell.r.iy1; ++iy) {
           if (ix - cell.r.ix0 < done && iy - cell.r.iy0 < done) continue;  // done above
           const unsigned long long t = cell.term(d, ix, iy);
-          if (t) hash_add(keys, vals, M, mo + ix * d.ny + iy, t, d.err, lim);
+          if (t) hash_add(keys, vals, M, mo + ix * d.ny + iy, t, d.limb, d.err, lim);
         }
       }
     }
@@ -306,7 +319,10 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int e
   __syncthreads();
   for (int i = threadIdx.x; i < kHash; i += blockDim.x) {
     int k = keys[i];
-    if (k >= 0) atomicAdd(&M[k], vals[i]);
+    if (k >= 0) {
+      const unsigned long long v = vals[i];
+      atomicAdd(&M[k], d.limb ? (v & 0xffffffffull) + ((v >> 32) << d.limb) : v);
+    }
   }
 }
 

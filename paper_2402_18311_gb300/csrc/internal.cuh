@@ -120,6 +120,7 @@ struct Dev {
   int *Wq, *Hq;      // [n_cells] quantised sizes
   float2 *pa;        // [n_mov] (pin count, charge area) per movable cell: the preconditioner's terms
   unsigned char *is_macro;  // [n_cells]
+  int limb;          // bits of a scatter-table entry's low sum (density.cu; 0: one sum)
   int has_big;       // some optimiser cell may cover more than 32 bins
   // density stretching (null when off): per movable cell {x shift, y shift,
   // stretched W, stretched H} in fixed point, the density scale R (2^31 = 1),
