@@ -976,6 +976,8 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.Gm = nf ? 2 * d.G : d.G;
   d.fill_area_q = (double)nf * (double)fp.Wf * (double)fp.Hf;
   {
+    const double s1 = (d.mov_area_q + d.fill_area_q) / d.abin_q;
+    d.area2_bins = (float)(s1 * s1);
     double fixed_q = 0.0;
     for (int i = Mv; i < C; ++i) fixed_q += (double)Wq[i] * (double)Hq[i];
     d.rho_mean = (float)((d.mov_area_q + d.fill_area_q + d.t * fixed_q) / (d.abin_q * (double)d.G));
@@ -1470,7 +1472,7 @@ int place_step_timed(place_t *h, int32_t n_iters, float *stage_ms) {
     if (d.solve == SOLVE_FFT) launch_fft_rows(d, 0, K, FIN_ITER, st);
     if (d.solve == SOLVE_GEMM) launch_density_finish(d, 0, K, FIN_ITER, st);
     cudaEventRecord(ev[1], st);
-    if (d.solve == SOLVE_FFT) launch_fft_solve(d, 0, K, 0, 0, st);
+    if (d.solve == SOLVE_FFT) launch_fft_solve(d, 0, K, FIN_ITER, 0, st);
     if (d.solve == SOLVE_GEMM) launch_spectral(d, 0, K, 0, 0, st);
     if (d.solve == SOLVE_SMALL) launch_solve_small(d, 0, K, FIN_ITER, 0, st);
     cudaEventRecord(ev[2], st);

@@ -96,8 +96,8 @@ __device__ __forceinline__ float2 finish_pair(const Dev &d, const FinishArgs &a,
 __device__ __forceinline__ void finish_commit(const Dev &d, int c, int mode, u128 v, float q2) {
   CopyState *cs = d.cs + c;
   const double tau = ldexp(u128_to_double(v), -d.t_shift) / d.mov_area_q;
-  const double s1 = (d.mov_area_q + d.fill_area_q) / d.abin_q;
-  if (mode != FIN_EVAL) cs->n_eff = q2 > 0.f ? s1 * s1 / (double)q2 : 0.0;
+  // (q2 is an FP32 sum, and FP64 divisions are a microsecond each here)
+  if (mode != FIN_EVAL) cs->n_eff = q2 > 0.f ? (double)(d.area2_bins / q2) : 0.0;
   if (mode == FIN_ITER) {
     cs->tau = tau;
     if (tau <= (double)d.prm.tau_stop) cs->converged = cs->stopped = 1;
@@ -116,14 +116,12 @@ struct FinishShared {
   int flag;
 };
 
-// The block's sums to its partial slot; the last block of each copy reduces
-// them and records the overflow.
+// The block's sums to its partial slot.
 template <int NT>
-__device__ __forceinline__ void finish_reduce(const Dev &d, int c, int mode, const BinSums &s,
-                                              FinishShared *sh) {
+__device__ __forceinline__ void finish_partial(const Dev &d, int c, const BinSums &s, FinishShared *sh) {
   const u128 tA = ((u128)d.tA_hi << 64) | d.tA_lo;
   const u128 acc = s.acc + ((u128)s.m_over << d.t_shift) - (u128)s.n_over * tA;
-  float q2 = block_sum_f<NT>(s.q2, sh->smf);
+  const float q2 = block_sum_f<NT>(s.q2, sh->smf);
   const u128 r = block_sum_u128<NT>(acc, sh->sm);
   if (threadIdx.x == 0) {
     unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + blockIdx.x) * 2;
@@ -131,9 +129,36 @@ __device__ __forceinline__ void finish_reduce(const Dev &d, int c, int mode, con
     p[1] = (unsigned long long)(r >> 64);
     d.conc_part[(size_t)c * d.nb_red + blockIdx.x] = q2;
   }
+}
+
+// The copy's overflow from n partials, by one warp (an earlier kernel's
+// partials, or, behind a cluster barrier, this one's).
+__device__ __forceinline__ void finish_total(const Dev &d, int c, int mode, int n) {
+  u128 v = 0;
+  float q2 = 0.f;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 32) {
+    const unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + i) * 2;
+    v += ((u128)__ldcg(p + 1) << 64) | __ldcg(p);
+    q2 += __ldcg(d.conc_part + (size_t)c * d.nb_red + i);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v += shfl_xor_u128(v, o);
+    q2 += __shfl_xor_sync(0xffffffffu, q2, o);
+  }
+  if (threadIdx.x == 0) finish_commit(d, c, mode, v, q2);
+}
+
+// The block's sums to its partial slot; the last block of each copy reduces
+// them and records the overflow.
+template <int NT>
+__device__ __forceinline__ void finish_reduce(const Dev &d, int c, int mode, const BinSums &s,
+                                              FinishShared *sh) {
+  finish_partial<NT>(d, c, s, sh);
   if (!arrive_last_t0(d.ctr + (size_t)c * C_COUNT + C_FINISH, &sh->flag)) return;
   u128 v = 0;
-  q2 = 0.f;
+  float q2 = 0.f;
 #pragma unroll 4
   for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) {
     const unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + i) * 2;

@@ -95,6 +95,7 @@ struct Dev {
   double abin_q;              // BW * BH
   double mov_area_q;          // the design's movable area (units of 2^-2F): tau's denominator
   double fill_area_q;         // the fillers' area (units of 2^-2F)
+  float area2_bins;           // ((mov_area_q + fill_area_q) / abin_q)^2: the numerator of n_eff
   double die_xl, die_yl, die_xh, die_yh;
   float fxl, fyl, fxh, fyh;
   float fbw, fbh, fibw, fibh;  // bin width/height and their inverses (FP32)
@@ -286,11 +287,11 @@ void launch_pack_xy(float2 *dst, const float *x, const float *y, int n, cudaStre
 void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t st);
 void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st);
 void launch_spectral(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st);
-// Fast transforms: the sides they take; the first kernel (which is also the
-// density finish in mode), and the other two.
+// Fast transforms: the sides they take; the first kernel, and the other two
+// (the first two are the density finish in mode).
 bool fft_side(int n);
 void launch_fft_rows(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st);
-void launch_fft_solve(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st);
+void launch_fft_solve(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cudaStream_t st);
 // One cluster per copy: the grids it takes; finish and field in one kernel.
 bool small_grid(int nx, int ny);
 int small_prepare();

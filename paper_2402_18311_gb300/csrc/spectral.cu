@@ -254,7 +254,7 @@ void launch_field(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cu
     launch_solve_small(d, copy0, ncopy, mode, with_psi, st);
   } else if (d.solve == SOLVE_FFT) {
     launch_fft_rows(d, copy0, ncopy, mode, st);
-    launch_fft_solve(d, copy0, ncopy, with_psi, eval, st);
+    launch_fft_solve(d, copy0, ncopy, mode, with_psi, st);
   } else {
     launch_density_finish(d, copy0, ncopy, mode, st);
     launch_spectral(d, copy0, ncopy, with_psi, eval, st);

@@ -60,7 +60,7 @@ __device__ __forceinline__ float2 half_turn(float2 c, float a, float b) {
 
 template <int LOGN, bool STRETCH>
 __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
-    k_fft_rows(Dev d, int copy0, int mode) {
+    k_fft_rows(Dev d, int copy0, int mode) {  // (its overflow partials: k_fft_columns)
   constexpr int N = 1 << LOGN, T = N / 8, F = row_ffts(LOGN), NT = F * T;
   __shared__ float2 sm[F * padded(N)];
   __shared__ FinishShared fs;
@@ -124,17 +124,26 @@ __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
     Ta[k] = wa.x;
     Tb[k] = wb.x;
   }
-  finish_reduce<NT>(d, c, mode, sums, &fs);
+  finish_partial<NT>(d, c, sums, &fs);
 }
 
-// CP column pairs per block, M / 8 threads each.
+// CP column pairs per block, M / 8 threads each.  One more block per copy
+// reduces the overflow of the row kernel's partials: beside the transforms
+// instead of at the end of that kernel, whose last block held the next one up
+// for 4 us.  (A copy that its stop test ends here may still get a field, which
+// nothing reads.)
 template <int LOGM, int CP>
-__global__ void __launch_bounds__(CP * (1 << (LOGM - 3))) k_fft_columns(Dev d, int copy0, int eval) {
+__global__ void __launch_bounds__(CP * (1 << (LOGM - 3)))
+    k_fft_columns(Dev d, int copy0, int mode, int partials) {
   constexpr int M = 1 << LOGM, T = M / 8, NT = CP * T;
   __shared__ float2 sm[CP * padded(M)];
   pdl_wait();
   const int c = copy0 + blockIdx.y;
-  if (!eval && d.cs[c].stopped) return;
+  if (mode == FIN_ITER && d.cs[c].stopped) return;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x < 32) finish_total(d, c, mode, partials);
+    return;
+  }
   const int ny = d.ny, v0 = blockIdx.x * 2 * CP;
   const float *Tc = d.T + (size_t)c * 3 * d.G + v0;
   {
@@ -198,6 +207,9 @@ __global__ void __launch_bounds__(CP * (1 << (LOGM - 3))) k_fft_columns(Dev d, i
   __syncthreads();
   transform<LOGM, true>(z, t, s, d.fft_wx);
   transform<LOGM, true>(w, t, s, d.fft_wx);
+  // (16-byte stores of every second row; collected in shared memory first, so
+  // that a row's columns leave together, the two kernels take 37 us instead of
+  // 32 at 1024^2 bins)
   float4 *PQ = reinterpret_cast<float4 *>(d.SB + (size_t)c * 3 * d.G) + (va >> 1);
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
@@ -274,6 +286,12 @@ __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
   }
 }
 
+int log2i(int n) {
+  int l = 0;
+  while ((1 << l) < n) ++l;
+  return l;
+}
+
 template <int LOGN>
 void rows(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st) {
   const dim3 grid(d.nx / 2 / row_ffts(LOGN), ncopy), block(row_ffts(LOGN) << (LOGN - 3));
@@ -283,11 +301,19 @@ void rows(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st) {
     launch_pdl(k_fft_rows<LOGN, false>, grid, block, 0, st, d, copy0, mode);
 }
 
+// Four pairs of columns per block (whole 32-byte sectors; fewer of the longest
+// columns), half of that where it would leave SMs without a block.  A column's result does not depend on it.
 template <int LOGM>
-void columns(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st) {
-  constexpr int CP = LOGM >= 12 ? 1 : (LOGM == 11 ? 2 : 4);
-  launch_pdl(k_fft_columns<LOGM, CP>, dim3(d.ny / 2 / CP, ncopy), dim3(CP << (LOGM - 3)), 0, st, d,
-             copy0, eval);
+void columns(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st) {
+  constexpr int MOST = LOGM >= 12 ? 1 : (LOGM == 11 ? 2 : 4);
+  constexpr int HALF = MOST > 1 && LOGM > 6 ? MOST / 2 : MOST;  // (at least a warp)
+  const int partials = d.nx / 2 / row_ffts(log2i(d.ny));
+  if (d.ny / 2 / MOST * ncopy < d.sms)
+    launch_pdl(k_fft_columns<LOGM, HALF>, dim3(d.ny / 2 / HALF + 1, ncopy), dim3(HALF << (LOGM - 3)), 0,
+               st, d, copy0, mode, partials);
+  else
+    launch_pdl(k_fft_columns<LOGM, MOST>, dim3(d.ny / 2 / MOST + 1, ncopy), dim3(MOST << (LOGM - 3)), 0,
+               st, d, copy0, mode, partials);
 }
 
 template <int LOGN>
@@ -297,12 +323,6 @@ void fields(const Dev &d, int copy0, int ncopy, int psi, int eval, cudaStream_t 
     launch_pdl(k_fft_fields<LOGN, true>, grid, block, 0, st, d, copy0, eval);
   else
     launch_pdl(k_fft_fields<LOGN, false>, grid, block, 0, st, d, copy0, eval);
-}
-
-int log2i(int n) {
-  int l = 0;
-  while ((1 << l) < n) ++l;
-  return l;
 }
 
 }  // namespace
@@ -324,9 +344,9 @@ void launch_fft_rows(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t 
   HP_BY_LENGTH(d.ny, rows, d, copy0, ncopy, mode, st)
 }
 
-void launch_fft_solve(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st) {
-  HP_BY_LENGTH(d.nx, columns, d, copy0, ncopy, eval, st)
-  HP_BY_LENGTH(d.ny, fields, d, copy0, ncopy, with_psi, eval, st)
+void launch_fft_solve(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cudaStream_t st) {
+  HP_BY_LENGTH(d.nx, columns, d, copy0, ncopy, mode, st)
+  HP_BY_LENGTH(d.ny, fields, d, copy0, ncopy, with_psi, mode != FIN_ITER, st)
 }
 
 }  // namespace hp

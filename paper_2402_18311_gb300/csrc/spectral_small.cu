@@ -82,8 +82,7 @@ template <bool STRETCH, bool PSI>
 __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallNT)
     k_solve_small(Dev d, int copy0, int mode) {
   extern __shared__ __align__(16) float dyn_small[];
-  __shared__ u128 sm[32];
-  __shared__ float smf[32];
+  __shared__ FinishShared fs;
   float *const sb[2] = {dyn_small, dyn_small + kSmallB};
   // a stage's outputs run along its B operand's rows, so this block has side /
   // 8 rows of each transform matrix; they are constants of the handle, loaded
@@ -128,18 +127,7 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallNT)
     const int v = i / nx, x = i - v * nx;
     T[i] = dot(a1 + (v - ry) * ny, &sb[0][x * (ny + 4)], ny);
   }
-  {
-    const u128 tA = ((u128)d.tA_hi << 64) | d.tA_lo;
-    const u128 acc = sums.acc + ((u128)sums.m_over << d.t_shift) - (u128)sums.n_over * tA;
-    const float q2 = block_sum_f<kSmallNT>(sums.q2, smf);
-    const u128 r = block_sum_u128<kSmallNT>(acc, sm);
-    if (threadIdx.x == 0) {
-      unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + blockIdx.x) * 2;
-      p[0] = (unsigned long long)r;
-      p[1] = (unsigned long long)(r >> 64);
-      d.conc_part[(size_t)c * d.nb_red + blockIdx.x] = q2;
-    }
-  }
+  finish_partial<kSmallNT>(d, c, sums, &fs);
   cluster_arrive();
   cluster_wait();
   // every block has read the map: zero it for the next pass (an evaluation
@@ -165,20 +153,7 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallNT)
   cluster_arrive();
   // the copy's overflow, while the others arrive
   if (blockIdx.x == 0 && threadIdx.x < 32) {
-    const int l = threadIdx.x;
-    u128 v = 0;
-    float q2 = 0.f;
-    if (l < kSmallBlocks) {
-      const unsigned long long *p = d.tau_part + ((size_t)c * d.nb_red + l) * 2;
-      v = ((u128)__ldcg(p + 1) << 64) | __ldcg(p);
-      q2 = __ldcg(d.conc_part + (size_t)c * d.nb_red + l);
-    }
-#pragma unroll
-    for (int o = kSmallBlocks / 2; o > 0; o >>= 1) {
-      v += shfl_xor_u128(v, o);
-      q2 += __shfl_xor_sync(0xffffffffu, q2, o);
-    }
-    if (l == 0) finish_commit(d, c, mode, v, q2);
+    finish_total(d, c, mode, kSmallBlocks);
     __syncwarp();
   }
   cluster_wait();
