@@ -226,9 +226,6 @@ struct place_t {
   cudaGraph_t graph0 = nullptr;
   cudaGraphExec_t exec0 = nullptr;
   bool k0_pending = true;
-  // handles with a fused solve: M may hold an evaluation's map and has to be zero
-  // before the next iteration (which leaves it zero itself)
-  bool m_dirty = true;
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
@@ -488,7 +485,7 @@ void drop_graph(place_t *h) {
   h->graph = h->graph0 = nullptr;
 }
 
-int enqueue_reset(place_t *h, int c0, int n);
+int enqueue_reset(place_t *h, int c0, int n, const NewXy &src = NewXy());
 int ensure_graph(place_t *h);
 cudaError_t launch_iter(place_t *h);
 
@@ -558,16 +555,25 @@ int check_dev_err(place_t *h) {
   return PLACE_OK;
 }
 
-// Optimiser reset of copies [c0, c0+n): clamp, u = v, scalars, tau_{-1}.
-int enqueue_reset(place_t *h, int c0, int n) {
+// The map of copies [c0, c0+n) zero for a scatter: handles with a fused solve
+// keep it so, every pass clearing what it has read.
+int clear_map(place_t *h, int c0, int n) {
+  const Dev &d = h->d;
+  if (d.solve == SOLVE_GEMM)
+    CK(cudaMemsetAsync(d.M + (size_t)c0 * d.Gm, 0, sizeof(unsigned long long) * d.Gm * n, h->stream));
+  return PLACE_OK;
+}
+
+// Optimiser reset of copies [c0, c0+n): new positions (src), clamp, u = v,
+// scalars, tau_{-1}.
+int enqueue_reset(place_t *h, int c0, int n, const NewXy &src) {
   Dev &d = h->d;
   cudaStream_t st = h->stream;
   h->k0_pending = true;  // the next iteration preconditions these copies' first step
-  h->m_dirty = true;
-  launch_reset(d, c0, n, st);
-  CK(cudaMemsetAsync(d.M + (size_t)c0 * d.Gm, 0, sizeof(unsigned long long) * d.Gm * n, st));
+  launch_reset(d, c0, n, src, st);
+  if (int rc = clear_map(h, c0, n)) return rc;
   launch_scatter(d, c0, n, 1, st);
-  launch_density_finish(d, c0, n, FIN_RESET, st);
+  launch_density_finish(d, c0, n, FIN_RESET, 1, st);
   CKL();
   return PLACE_OK;
 }
@@ -585,8 +591,7 @@ void enqueue_iteration(const Dev &d, cudaStream_t st, const cudaStream_t *wst, c
   for (int b = 0; b < nb; ++b) cudaStreamWaitEvent(wst[b], fork, 0);
   launch_wa_branches(d, 0, K, wst);
   for (int b = 0; b < nb; ++b) cudaEventRecord(join[b], wst[b]);
-  // a fused solve zeroes the map that it has read; the GEMM handles clear it
-  // here (clear_map has the other half of that rule)
+  // a fused solve zeroes the map that it has read; the GEMM handles clear it here
   if (!d.solve) cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
   launch_scatter(d, 0, K, 0, st);
   launch_field(d, 0, K, FIN_ITER, 0, st);
@@ -613,22 +618,11 @@ int ensure_graph(place_t *h) {
   return PLACE_OK;
 }
 
-// On a handle with a fused solve the map is zero before an iteration: cleared here
-// after a call that left one in it, by the iteration itself otherwise.
-cudaError_t clear_map(place_t *h) {
-  const Dev &d = h->d;
-  if (!d.solve || !h->m_dirty) return cudaSuccess;
-  h->m_dirty = false;
-  return cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * d.K, h->stream);
-}
-
 // One iteration of every copy: the graph with the k = 0 preconditioning pass
 // when a reset since the last iteration may have left a copy at k = 0, the
 // one without it otherwise (the two compute the same: the pass does nothing
 // for a copy past k = 0).  ensure_graph must have succeeded.
 cudaError_t launch_iter(place_t *h) {
-  const cudaError_t e = clear_map(h);
-  if (e != cudaSuccess) return e;
   if (h->k0_pending) {
     h->k0_pending = false;
     return cudaGraphLaunch(h->exec0, h->stream);
@@ -636,18 +630,70 @@ cudaError_t launch_iter(place_t *h) {
   return cudaGraphLaunch(h->exec, h->stream);
 }
 
-// Interleaved device positions -> caller's x, y (host or device) through the
-// handle's scratch; synchronises.
+// Whether a kernel on the handle's device may read or write bytes bytes at p
+// itself: plain device memory of that device, the whole range inside one
+// allocation, and none of the handle's own (host, managed and peer memory go
+// through a copy, as does a range that a copy would refuse).
+bool direct(const place_t *h, const void *p, size_t bytes) {
+  typedef CUresult (*Fn)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+  static const Fn fn = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return (Fn)f;
+  }();
+  int dev = -1, on = -1;
+  unsigned int type = 0, managed = 0;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute at[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                               CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                               CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void *out[5] = {&type, &on, &managed, &start, &size};
+  if (!fn || ((uintptr_t)p & 3) || cudaGetDevice(&dev) != cudaSuccess ||
+      fn(5, at, out, (CUdeviceptr)p) != CUDA_SUCCESS)
+    return false;
+  const CUdeviceptr a = (CUdeviceptr)p, own = (CUdeviceptr)h->mem;
+  return type == CU_MEMORYTYPE_DEVICE && !managed && on == dev && a >= start && a + bytes <= start + size &&
+         (a + bytes <= own || a >= own + h->mem_bytes);
+}
+
+// Interleaved device positions -> caller's x, y (host or device), through the
+// handle's scratch where the caller's memory is not the device's own;
+// synchronises.
 int copy_out_xy(place_t *h, const float2 *src, float *x, float *y) {
   const Dev &d = h->d;
   const int C = d.n_cells - d.n_fill;  // the design's cells: movable, then fixed
-  launch_unpack_xy(d.px_tmp, d.py_tmp, src, d.n_real, h->stream);
-  launch_unpack_xy(d.px_tmp + d.n_real, d.py_tmp + d.n_real, src + d.n_mov, C - d.n_real, h->stream);
-  CKL();
-  if (x) CK(cudaMemcpyAsync(x, h->d.px_tmp, sizeof(float) * C, cudaMemcpyDefault, h->stream));
-  if (y) CK(cudaMemcpyAsync(y, h->d.py_tmp, sizeof(float) * C, cudaMemcpyDefault, h->stream));
+  const size_t bytes = sizeof(float) * C;
+  const bool apart = !x || !y || (const char *)x + bytes <= (const char *)y || (const char *)y + bytes <= (const char *)x;
+  if (apart && (!x || direct(h, x, bytes)) && (!y || direct(h, y, bytes))) {
+    if (x || y) launch_unpack_xy(x, y, src, d.n_real, C, d.n_fill, h->stream);
+    CKL();
+  } else {
+    launch_unpack_xy(d.px_tmp, d.py_tmp, src, d.n_real, C, d.n_fill, h->stream);
+    CKL();
+    if (x) CK(cudaMemcpyAsync(x, d.px_tmp, bytes, cudaMemcpyDefault, h->stream));
+    if (y) CK(cudaMemcpyAsync(y, d.py_tmp, bytes, cudaMemcpyDefault, h->stream));
+  }
   CK(cudaStreamSynchronize(h->stream));
   return PLACE_OK;
+}
+
+// Optimiser reset of copies [c0, c0 + n) with new positions of cells [lo, lo +
+// m) from the caller's arrays (host or device).
+int reset_to(place_t *h, int c0, int n, const float *x, const float *y, int lo, int m) {
+  const Dev &d = h->d;
+  const size_t bytes = sizeof(float) * m;
+  NewXy src{x, y, lo, lo + m};
+  if (m > 0 && !(direct(h, x, bytes) && direct(h, y, bytes))) {
+    CK(cudaMemcpyAsync(d.px_tmp, x, bytes, cudaMemcpyDefault, h->stream));
+    CK(cudaMemcpyAsync(d.py_tmp, y, bytes, cudaMemcpyDefault, h->stream));
+    src.x = d.px_tmp;
+    src.y = d.py_tmp;
+  }
+  return enqueue_reset(h, c0, n, src);
 }
 
 int check_copy(const place_t *h, int copy, bool allow_all) {
@@ -1326,6 +1372,8 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   ce = cudaMemsetAsync(d.E, 0, sizeof(float) * (size_t)d.K * 3 * d.G, h->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(d.Fmap, 0, sizeof(long long) * d.G, h->stream);
   if (ce == cudaSuccess)
+    ce = cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * d.K, h->stream);
+  if (ce == cudaSuccess)
     ce = cudaMemsetAsync(d.gacc, 0, sizeof(unsigned long long) * (size_t)d.K * std::max(Mo, 1), h->stream);
   if (ce == cudaSuccess && wa_prepare(d.wa_big_cap)) ce = cudaErrorInvalidValue;
   if (ce == cudaSuccess && d.solve == SOLVE_SMALL && small_prepare()) ce = cudaErrorInvalidValue;
@@ -1361,6 +1409,9 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
       h->autotuned = 1;
       h->autotune_ms = to.ms;
       for (int c = 0; c < d.K && rc == PLACE_OK; ++c) up(d.xy + (size_t)c * Ci, xy0.data(), sizeof(float2) * Ci);
+      if (rc == PLACE_OK && cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * d.K,
+                                            h->stream) != cudaSuccess)
+        rc = fail(PLACE_ECUDA, "memset of the density map failed");
       if (rc == PLACE_OK) rc = enqueue_reset(h, 0, d.K);
       if (rc == PLACE_OK) {
         ce = cudaStreamSynchronize(h->stream);
@@ -1470,14 +1521,13 @@ int place_step_timed(place_t *h, int32_t n_iters, float *stage_ms) {
   std::vector<double> acc(PLACE_N_STAGES, 0.0);
   int rc = PLACE_OK;
   for (int it = 0; it < n_iters && rc == PLACE_OK; ++it) {
-    clear_map(h);
     cudaEventRecord(ev[0], st);
     if (!d.solve) cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
     launch_scatter(d, 0, K, 0, st);
     // the stages' line within a fused solve: behind the first transform with
     // the fast transforms, before the one kernel of a small grid
     if (d.solve == SOLVE_FFT) launch_fft_rows(d, 0, K, FIN_ITER, st);
-    if (d.solve == SOLVE_GEMM) launch_density_finish(d, 0, K, FIN_ITER, st);
+    if (d.solve == SOLVE_GEMM) launch_density_finish(d, 0, K, FIN_ITER, 0, st);
     cudaEventRecord(ev[1], st);
     if (d.solve == SOLVE_FFT) launch_fft_solve(d, 0, K, FIN_ITER, 0, st);
     if (d.solve == SOLVE_GEMM) launch_spectral(d, 0, K, 0, 0, st);
@@ -1791,7 +1841,7 @@ int place_get_fillers(place_t *h, int32_t copy, float *x, float *y, int32_t cap,
   if (n) *n = d.n_fill;
   const int m = std::min(cap, d.n_fill);
   if (m > 0 && (x || y)) {
-    launch_unpack_xy(d.px_tmp, d.py_tmp, d.xy + (size_t)copy * d.n_cells + d.n_real, m, h->stream);
+    launch_unpack_xy(d.px_tmp, d.py_tmp, d.xy + (size_t)copy * d.n_cells + d.n_real, m, m, 0, h->stream);
     CKL();
     if (x) CK(cudaMemcpyAsync(x, d.px_tmp, sizeof(float) * m, cudaMemcpyDefault, h->stream));
     if (y) CK(cudaMemcpyAsync(y, d.py_tmp, sizeof(float) * m, cudaMemcpyDefault, h->stream));
@@ -1807,11 +1857,7 @@ int place_set_fillers(place_t *h, int32_t copy, const float *x, const float *y) 
   if (d.n_fill == 0) return PLACE_OK;
   if (!x || !y) return fail(PLACE_EINVAL, "null positions");
   const int c0 = copy < 0 ? 0 : copy, n = copy < 0 ? d.K : 1;
-  CK(cudaMemcpyAsync(d.px_tmp, x, sizeof(float) * d.n_fill, cudaMemcpyDefault, h->stream));
-  CK(cudaMemcpyAsync(d.py_tmp, y, sizeof(float) * d.n_fill, cudaMemcpyDefault, h->stream));
-  for (int c = c0; c < c0 + n; ++c)
-    launch_pack_xy(d.xy + (size_t)c * d.n_cells + d.n_real, d.px_tmp, d.py_tmp, d.n_fill, h->stream);
-  return enqueue_reset(h, c0, n);
+  return reset_to(h, c0, n, x, y, d.n_real, d.n_fill);
 }
 
 int place_device_views(place_t *h, int32_t copy, float **x, float **y) {
@@ -1828,12 +1874,8 @@ int place_set_positions(place_t *h, int32_t copy, const float *x, const float *y
   int rc = check_copy(h, copy, true);
   if (rc) return rc;
   if (!x || !y) return fail(PLACE_EINVAL, "null positions");
-  const size_t C = h->d.n_cells, Mv = h->d.n_real;
-  int c0 = copy < 0 ? 0 : copy, n = copy < 0 ? h->d.K : 1;
-  CK(cudaMemcpyAsync(h->d.px_tmp, x, sizeof(float) * Mv, cudaMemcpyDefault, h->stream));
-  CK(cudaMemcpyAsync(h->d.py_tmp, y, sizeof(float) * Mv, cudaMemcpyDefault, h->stream));
-  for (int c = c0; c < c0 + n; ++c) launch_pack_xy(h->d.xy + c * C, h->d.px_tmp, h->d.py_tmp, (int)Mv, h->stream);
-  return enqueue_reset(h, c0, n);
+  const int c0 = copy < 0 ? 0 : copy, n = copy < 0 ? h->d.K : 1;
+  return reset_to(h, c0, n, x, y, 0, h->d.n_real);
 }
 
 int place_eval_wirelength(place_t *h, int32_t copy, float gamma, double *wl, float *gx, float *gy) {
@@ -1866,10 +1908,8 @@ int place_eval_wirelength(place_t *h, int32_t copy, float gamma, double *wl, flo
 namespace {
 
 int scatter_at(place_t *h, int copy) {
-  Dev &d = h->d;
-  h->m_dirty = true;
-  CK(cudaMemsetAsync(d.M + (size_t)copy * d.Gm, 0, sizeof(unsigned long long) * d.Gm, h->stream));
-  launch_scatter(d, copy, 1, 1, h->stream);
+  if (int rc = clear_map(h, copy, 1)) return rc;
+  launch_scatter(h->d, copy, 1, 1, h->stream);
   return PLACE_OK;
 }
 
@@ -1883,9 +1923,16 @@ int place_eval_density(place_t *h, int32_t copy, int64_t *map, double *overflow)
   if (rc) return rc;
   Dev &d = h->d;
   if ((rc = scatter_at(h, copy))) return rc;
-  launch_density_finish(d, copy, 1, FIN_EVAL, h->stream);
+  launch_density_finish(d, copy, 1, FIN_EVAL, map == nullptr, h->stream);
   CKL();
-  if (map) CK(cudaMemcpyAsync(map, d.M + (size_t)copy * d.Gm, sizeof(int64_t) * d.G, cudaMemcpyDefault, h->stream));
+  if (map) {
+    // the map that is handed out is cleared after the copy (whether or not it
+    // could be made)
+    unsigned long long *M = d.M + (size_t)copy * d.Gm;
+    const cudaError_t e = cudaMemcpyAsync(map, M, sizeof(int64_t) * d.G, cudaMemcpyDefault, h->stream);
+    CK(cudaMemsetAsync(M, 0, sizeof(unsigned long long) * d.Gm, h->stream));
+    CK(e);
+  }
   double s = 0;
   CK(cudaMemcpyAsync(&s, d.scal + (size_t)copy * S_COUNT + S_TAU, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -1938,12 +1985,18 @@ int place_eval_hpwl_overflow(place_t *h, double *hpwl, double *overflow) {
   if (!h) return fail(PLACE_EINVAL, "null handle");
   Dev &d = h->d;
   const int K = d.K;
+  // the density pass beside the HPWL's kernels
+  CK(cudaEventRecord(h->ev_fork, h->stream));
+  CK(cudaStreamWaitEvent(h->cap, h->ev_fork, 0));
+  if (d.solve == SOLVE_GEMM)
+    CK(cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, h->cap));
+  launch_scatter(d, 0, K, 1, h->cap);
+  launch_density_finish(d, 0, K, FIN_EVAL, 1, h->cap);
+  const cudaError_t e = cudaEventRecord(h->ev_join, h->cap);
   launch_hpwl64(d, 0, K, h->stream);
   launch_reduce_slot(d, S_HP64, d.wa_blocks_total, 0, K, h->stream);
-  h->m_dirty = true;
-  CK(cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, h->stream));
-  launch_scatter(d, 0, K, 1, h->stream);
-  launch_density_finish(d, 0, K, FIN_EVAL, h->stream);
+  CK(e);
+  CK(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
   CKL();
   std::vector<double> sc((size_t)K * S_COUNT);
   CK(cudaMemcpyAsync(sc.data(), d.scal, sizeof(double) * sc.size(), cudaMemcpyDeviceToHost, h->stream));

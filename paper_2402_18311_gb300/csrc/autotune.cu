@@ -269,7 +269,7 @@ int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut 
       cudaMemsetAsync(d.M, 0, mbytes, st);
       d.scat_force = SCAT_MERGED;
       launch_scatter_main(d, 0, 1, 1, st);
-      launch_density_finish(d, 0, 1, FIN_RESET, st);
+      launch_density_finish(d, 0, 1, FIN_RESET, 0, st);
       CopyState cs;
       if (cudaMemcpyAsync(&cs, d.cs, sizeof cs, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
           cudaStreamSynchronize(st) != cudaSuccess)

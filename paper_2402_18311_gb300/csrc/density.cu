@@ -363,9 +363,10 @@ __device__ __forceinline__ void store_bf16_pair(__nv_bfloat16 *hp, __nv_bfloat16
 // solve): four bins per step, (x, y), (x, y+1) and their mirrors
 // (x, ny-1-y), (x, ny-2-y), and rho leaves as the sums rho_y + rho_{ny-1-y}
 // at y and the differences at ny/2 + y (y < ny/2).  Handles with a fused
-// solve form rho there and come here for the overflow alone.
+// solve form rho there and come here for the overflow alone;
+// clear: they leave the map zero.
 template <bool STRETCH, bool FOLD>
-__global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, int mode) {
+__global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, int mode, int clear) {
   __shared__ FinishShared fs;
   pdl_wait();
   const int c = copy0 + blockIdx.y;
@@ -389,7 +390,10 @@ __global__ void __launch_bounds__(kThreads) k_density_finish(Dev d, int copy0, i
     const int G2 = d.G >> 1;
     for (int b2 = blockIdx.x * blockDim.x + threadIdx.x; b2 < G2; b2 += gridDim.x * blockDim.x) {
       const float2 rv = finish_pair<STRETCH>(d, fa, b2, sums);
-      if (d.solve) continue;
+      if (d.solve != SOLVE_GEMM) {
+        if (clear) clear_pair(d, c, b2);
+        continue;
+      }
       if (d.tc)
         store_bf16_pair(d.rho_h + (size_t)c * d.G, d.rho_l + (size_t)c * d.G, b2, rv.x, rv.y);
       else
@@ -458,17 +462,12 @@ void launch_scatter_fixed(const Dev &d, const float2 *xy, int n0, int n1,
   k_scatter_range<<<blocks, kThreads, 0, st>>>(d, xy, n0, n1, out);
 }
 
-void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st) {
+void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, int clear, cudaStream_t st) {
   dim3 grid(d.bin_blocks, ncopy);
-  const bool fold = d.bfly && !d.solve;
-  if (d.Ms && fold)
-    launch_pdl(k_density_finish<true, true>, grid, dim3(kThreads), 0, st, d, copy0, mode);
-  else if (d.Ms)
-    launch_pdl(k_density_finish<true, false>, grid, dim3(kThreads), 0, st, d, copy0, mode);
-  else if (fold)
-    launch_pdl(k_density_finish<false, true>, grid, dim3(kThreads), 0, st, d, copy0, mode);
-  else
-    launch_pdl(k_density_finish<false, false>, grid, dim3(kThreads), 0, st, d, copy0, mode);
+  const bool fold = d.bfly && d.solve == SOLVE_GEMM;
+  auto *k = d.Ms ? (fold ? k_density_finish<true, true> : k_density_finish<true, false>)
+                 : (fold ? k_density_finish<false, true> : k_density_finish<false, false>);
+  launch_pdl(k, grid, dim3(kThreads), 0, st, d, copy0, mode, clear);
 }
 
 }  // namespace hp

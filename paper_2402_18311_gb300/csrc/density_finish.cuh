@@ -110,6 +110,13 @@ __device__ __forceinline__ void finish_commit(const Dev &d, int c, int mode, u12
   }
 }
 
+// The map (and the fillers') zero again at bins 2 b2 and 2 b2 + 1.
+__device__ __forceinline__ void clear_pair(const Dev &d, int c, int b2) {
+  ulonglong2 *M = reinterpret_cast<ulonglong2 *>(d.M + (size_t)c * d.Gm);
+  M[b2] = make_ulonglong2(0ull, 0ull);
+  if (d.n_fill) M[(d.G >> 1) + b2] = make_ulonglong2(0ull, 0ull);
+}
+
 struct FinishShared {
   u128 sm[32];
   float smf[32];

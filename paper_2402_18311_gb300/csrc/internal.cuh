@@ -160,8 +160,8 @@ struct Dev {
   float *cu, *cv;                          // c_k / n factors
 
   // the Poisson solve the handle runs.  The fused ones (not SOLVE_GEMM) finish
-  // the density pass themselves, keep M zero between density passes and hold
-  // the field as (Ex, Ey) pairs
+  // the density pass themselves, keep M zero between density passes (whoever
+  // scatters also clears) and hold the field as (Ex, Ey) pairs
   int solve;
   float rho_mean;           // the mean bin density, up to cells beyond the die
   float2 *fft_wx, *fft_wy;  // [nx], [ny] exp(-2 pi i k / n)
@@ -283,9 +283,8 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 void launch_scatter(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st);
 void launch_scatter_fixed(const Dev &d, const float2 *xy, int n0, int n1,
                           unsigned long long *out, cudaStream_t st);
-void launch_pack_xy(float2 *dst, const float *x, const float *y, int n, cudaStream_t st);
-void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t st);
-void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, cudaStream_t st);
+void launch_unpack_xy(float *x, float *y, const float2 *src, int n0, int n, int skip, cudaStream_t st);
+void launch_density_finish(const Dev &d, int copy0, int ncopy, int mode, int clear, cudaStream_t st);
 void launch_spectral(const Dev &d, int copy0, int ncopy, int with_psi, int eval, cudaStream_t st);
 // Fast transforms: the sides they take; the first kernel, and the other two
 // (the first two are the density finish in mode).
@@ -338,7 +337,12 @@ int cell_grad_blocks_per_sm(const Dev &d);
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st);
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st);
-void launch_reset(const Dev &d, int copy0, int ncopy, cudaStream_t st);
+// src: new positions of cells [lo, hi) (device arrays of hi - lo; none: null).
+struct NewXy {
+  const float *x = nullptr, *y = nullptr;
+  int lo = 0, hi = 0;
+};
+void launch_reset(const Dev &d, int copy0, int ncopy, const NewXy &src, cudaStream_t st);
 void launch_reduce_slot(const Dev &d, int slot, int nvals, int copy0, int ncopy, cudaStream_t st);
 void shuffle_plan(Dev &d);
 void launch_shuffle(const Dev &d, int copy0, int ncopy, int op, int k, uint64_t seed, cudaStream_t st);

@@ -564,15 +564,18 @@ __global__ void __launch_bounds__(kThreads) k_redo_step(Dev d, int copy0) {
   }
 }
 
-// Optimiser reset: clamp the movable positions into the die, u = v, and
-// initial scalars (tau_{-1} and gamma_0 follow from the density pass).
-__global__ void __launch_bounds__(kThreads) k_reset(Dev d, int copy0) {
+// Optimiser reset: new positions where there are any, the movable ones clamped
+// into the die, u = v, and initial scalars (tau_{-1} and gamma_0 follow from
+// the density pass).
+__global__ void __launch_bounds__(kThreads) k_reset(Dev d, int copy0, NewXy src) {
   const int c = copy0 + blockIdx.y;
   const size_t cn = (size_t)c * d.n_cells, cm = (size_t)c * d.n_mov;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n_mov; i += gridDim.x * blockDim.x) {
-    const float2 v = d.xy[cn + i];
-    float vx = fmaxf(d.fxl, fminf(v.x, d.fxh - d.w[i]));
-    float vy = fmaxf(d.fyl, fminf(v.y, d.fyh - d.h[i]));
+    const float2 v = i >= src.lo && i < src.hi ? make_float2(src.x[i - src.lo], src.y[i - src.lo])
+                                               : d.xy[cn + i];
+    const float2 s = d.wh[i];
+    float vx = fmaxf(d.fxl, fminf(v.x, d.fxh - s.x));
+    float vy = fmaxf(d.fyl, fminf(v.y, d.fyh - s.y));
     d.xy[cn + i] = make_float2(vx, vy);
     d.u[cm + i] = make_float2(vx, vy);
     d.gacc[cm + i] = 0ull;
@@ -593,29 +596,20 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_slot(Dev d, int slot, in
   if (threadIdx.x == 0) d.scal[(size_t)c * S_COUNT + slot] = s;
 }
 
-__global__ void k_pack_xy(float2 *dst, const float *x, const float *y, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    dst[i] = make_float2(x[i], y[i]);
-}
-
-__global__ void k_unpack_xy(float *x, float *y, const float2 *src, int n) {
+// Cells [0, n0) and, past `skip` others, the rest of n cells: x and y (either
+// may be null) from interleaved positions.
+__global__ void k_unpack_xy(float *x, float *y, const float2 *src, int n0, int n, int skip) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float2 v = src[i];
-    x[i] = v.x;
-    y[i] = v.y;
+    const float2 v = src[i < n0 ? i : i + skip];
+    if (x) x[i] = v.x;
+    if (y) y[i] = v.y;
   }
 }
 
-void launch_pack_xy(float2 *dst, const float *x, const float *y, int n, cudaStream_t st) {
+void launch_unpack_xy(float *x, float *y, const float2 *src, int n0, int n, int skip, cudaStream_t st) {
   if (n <= 0) return;
   int b = (n + kThreads - 1) / kThreads;
-  k_pack_xy<<<b < 4096 ? b : 4096, kThreads, 0, st>>>(dst, x, y, n);
-}
-
-void launch_unpack_xy(float *x, float *y, const float2 *src, int n, cudaStream_t st) {
-  if (n <= 0) return;
-  int b = (n + kThreads - 1) / kThreads;
-  k_unpack_xy<<<b < 4096 ? b : 4096, kThreads, 0, st>>>(x, y, src, n);
+  k_unpack_xy<<<b < 4096 ? b : 4096, kThreads, 0, st>>>(x, y, src, n0, n, skip);
 }
 
 namespace {
@@ -663,8 +657,8 @@ void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st) {
     launch_pdl(k_update<false>, grid, dim3(kThreads), 0, st, d, copy0);
   }
 }
-void launch_reset(const Dev &d, int copy0, int ncopy, cudaStream_t st) {
-  k_reset<<<dim3(d.cell_blocks, ncopy), kThreads, 0, st>>>(d, copy0);
+void launch_reset(const Dev &d, int copy0, int ncopy, const NewXy &src, cudaStream_t st) {
+  k_reset<<<dim3(d.cell_blocks, ncopy), kThreads, 0, st>>>(d, copy0, src);
 }
 void launch_reduce_slot(const Dev &d, int slot, int nvals, int copy0, int ncopy,
                         cudaStream_t st) {

@@ -256,7 +256,7 @@ void launch_field(const Dev &d, int copy0, int ncopy, int mode, int with_psi, cu
     launch_fft_rows(d, copy0, ncopy, mode, st);
     launch_fft_solve(d, copy0, ncopy, mode, with_psi, st);
   } else {
-    launch_density_finish(d, copy0, ncopy, mode, st);
+    launch_density_finish(d, copy0, ncopy, mode, 0, st);
     launch_spectral(d, copy0, ncopy, with_psi, eval, st);
   }
 }

@@ -91,20 +91,12 @@ __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
       s[pad(N - 1 - q)] = make_float2(ra[m].y - d.rho_mean, rb[m].y - d.rho_mean);
     }
   }
-  // the map is zero again for the next pass (an evaluation still hands it out)
-  if (mode == FIN_ITER) {
-    ulonglong2 *Mz = reinterpret_cast<ulonglong2 *>(d.M + (size_t)c * d.Gm);
+  // the map is zero again for the next pass
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int q = t + m * T;
-      const ulonglong2 z = make_ulonglong2(0ull, 0ull);
-      Mz[xa * (N / 2) + q] = z;
-      Mz[(xa + 1) * (N / 2) + q] = z;
-      if (d.n_fill) {
-        Mz[(d.G >> 1) + xa * (N / 2) + q] = z;
-        Mz[(d.G >> 1) + (xa + 1) * (N / 2) + q] = z;
-      }
-    }
+  for (int m = 0; m < 4; ++m) {
+    const int q = t + m * T;
+    clear_pair(d, c, xa * (N / 2) + q);
+    clear_pair(d, c, (xa + 1) * (N / 2) + q);
   }
   __syncthreads();
   float2 v[8];

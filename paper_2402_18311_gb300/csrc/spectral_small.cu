@@ -130,9 +130,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallNT)
   finish_partial<kSmallNT>(d, c, sums, &fs);
   cluster_arrive();
   cluster_wait();
-  // every block has read the map: zero it for the next pass (an evaluation
-  // still hands it out)
-  if (mode == FIN_ITER && own) {
+  // every block has read the map: zero it for the next pass
+  if (own) {
     unsigned long long *M = d.M + (size_t)c * d.Gm;
     M[i] = 0ull;
     if (d.n_fill) M[G + i] = 0ull;

@@ -68,7 +68,7 @@ def test_field_and_gradient_match_oracle(nx, ny, mode):
         place.place_destroy(h)
 
 
-@pytest.mark.parametrize("nx", [32, 64])  # one cluster; fast transforms
+@pytest.mark.parametrize("nx", [32, 64, 48])  # one cluster; fast transforms; GEMMs
 @pytest.mark.parametrize("opts", [{}, {"fillers": 1}, {"stretch": 1}, {"max_backtracks": 5}])
 def test_evaluations_between_iterations_change_nothing(nx, opts):
     # an iteration leaves the map zero and an evaluation does not: iterations
