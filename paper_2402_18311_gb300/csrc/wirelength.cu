@@ -511,18 +511,19 @@ __global__ void __launch_bounds__(kThreads) k_hpwl_thread(Dev d, int copy0, int 
     int p0, p1;
     if (!hpwl_net(d, e, p0, p1) || p1 <= p0) continue;
     PairBox b = empty_box();
-    float2 o[4], v[4];
+    // (the class is ordered by degree: a warp's nets nearly always agree)
+    int cj[4];
+    float2 o[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      // a short net repeats its first pin, which changes no extent
-      const int j = p0 + k < p1 ? p0 + k : p0;
-      int cj = d.pin_cell[j];
-      HP_FIX(d.err, cj, d.n_cells, BS_HPWL_CELL);
-      o[k] = d.pin_off[j];
-      v[k] = xy[cj];
+      if (p0 + k >= p1) break;
+      cj[k] = d.pin_cell[p0 + k];
+      HP_FIX(d.err, cj[k], d.n_cells, BS_HPWL_CELL);
+      o[k] = d.pin_off[p0 + k];
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) box_add(b, v[k], o[k]);
+    for (int k = 0; k < 4; ++k)
+      if (p0 + k < p1) box_add(b, xy[cj[k]], o[k]);
     acc = box_hpwl(b, d.net_w ? d.net_w[e] : 1.0f, acc);
   }
   hpwl_store<kThreads>(d, c, cls, acc, sm);
