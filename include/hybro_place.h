@@ -485,8 +485,8 @@ int place_test_bounds_check(place_t *h);
  * whose quantised size falls outside [1, 2^31), or a total area of 2^62 units
  * or more, makes *overflow NaN (the map is then not meaningful).
  *
- * Sharing: all calls use the one scratch array and each call clears it
- * first; calls whose work overlaps on the GPU (different streams or host
+ * Sharing: all calls use the one scratch array and each call leaves it
+ * clear; calls whose work overlaps on the GPU (different streams or host
  * threads) race on it and must be serialised.  The first call with a given
  * device current looks up the array's device address
  * (cudaGetSymbolAddress); make that first call before any stream capture.

@@ -204,6 +204,37 @@ int use_fold(int tc, int fold, int nx, int ny) {
 }  // namespace
 
 namespace hp {
+bool set_target(Dev &d, float target_density) {
+  // t = mant * 2^-shift exactly (24-bit mantissa of the float)
+  d.t = (double)target_density;
+  int e = 0;
+  const double f = std::frexp(d.t, &e);
+  d.t_mant = (long long)std::ldexp(f, 24);
+  d.t_shift = 24 - e;
+  if (d.t_shift < 0 || d.t_shift > 60) return false;
+  const unsigned __int128 tA = (unsigned __int128)(unsigned long long)d.t_mant *
+                               (unsigned __int128)(unsigned long long)(d.BW * d.BH);
+  d.tA_lo = (unsigned long long)tA;
+  d.tA_hi = (unsigned long long)(tA >> 64);
+  const unsigned __int128 fl = tA >> d.t_shift;
+  d.tA_floor = fl > (unsigned __int128)0x7fffffffffffffffull ? 0x7fffffffffffffffull
+                                                               : (unsigned long long)fl;
+  return true;
+}
+
+// A block's cells (at most 2^lg) times the largest area that one of them has
+// in one bin (below 2^bits) fit two 32-bit sums, of the areas' low 32 - lg bits
+// and of the rest, when lg + bits - (32 - lg) <= 32.
+int table_limb(long long n, int blocks, unsigned long long area) {
+  const long long step = (long long)std::max(blocks, 1) * kThreads;
+  const long long most = ((n + step - 1) / step) * kThreads;
+  int lg = 0, bits = 0;
+  while ((1LL << lg) < most) ++lg;
+  while (bits < 64 && (area >> bits)) ++bits;
+  // (a block is 256 threads, so the low sum has at most 24 bits)
+  return lg >= 8 && lg < 32 && 2 * lg + bits <= 64 ? 32 - lg : 0;
+}
+
 // Lets other translation units report through place_last_error().
 void set_last_error(const char *msg) { g_err = msg; }
 }  // namespace hp
@@ -964,28 +995,11 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.inv_area_q = (float)std::ldexp(1.0, -2 * F);
   d.XL = (long long)(die->xl * s); d.YL = (long long)(die->yl * s);
   d.BW = (long long)(bw * s); d.BH = (long long)(bh * s);
-  d.t = (double)bins->target_density;
-  {
-    // t = mant * 2^-shift exactly (24-bit mantissa of the float)
-    int e = 0;
-    double f = std::frexp((double)bins->target_density, &e);
-    d.t_mant = (long long)std::ldexp(f, 24);
-    d.t_shift = 24 - e;
-    if (d.t_shift < 0 || d.t_shift > 60) {
-      delete h;
-      return fail(PLACE_EINVAL, "target density out of range");
-    }
+  if (!set_target(d, bins->target_density)) {
+    delete h;
+    return fail(PLACE_EINVAL, "target density out of range");
   }
   d.abin_q = (double)d.BW * (double)d.BH;
-  {
-    const unsigned __int128 tA = (unsigned __int128)(unsigned long long)d.t_mant *
-                                 (unsigned __int128)(unsigned long long)(d.BW * d.BH);
-    d.tA_lo = (unsigned long long)tA;
-    d.tA_hi = (unsigned long long)(tA >> 64);
-    const unsigned __int128 fl = tA >> d.t_shift;
-    d.tA_floor = fl > (unsigned __int128)0x7fffffffffffffffull ? 0x7fffffffffffffffull
-                                                                 : (unsigned long long)fl;
-  }
   d.BW32 = (int)d.BW; d.BH32 = (int)d.BH;
   d.ibw_q = (float)(1.0 / (double)d.BW); d.ibh_q = (float)(1.0 / (double)d.BH);
   d.die_xl = die->xl; d.die_yl = die->yl; d.die_xh = die->xh; d.die_yh = die->yh;
@@ -1221,14 +1235,6 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   // launch plan
   d.cell_blocks = std::max(1, std::min((Mo + kThreads - 1) / kThreads, kMaxCellBlocks));
   {
-    // the scatter table's split: a block's cells (at most 2^lg) times the
-    // largest area that one of them has in one bin (below 2^bits) fit two
-    // 32-bit sums of the areas' low 32 - lg bits and of the rest when
-    // lg + bits - (32 - lg) <= 32
-    const long long step = (long long)d.cell_blocks * kThreads;
-    const long long most = ((Mo + step - 1) / step) * kThreads;
-    int lg = 0;
-    while ((1LL << lg) < most) ++lg;
     unsigned long long area = 1;
     for (int i = 0; i < Mo; ++i) {
       long long w = Wqi[i], hh = Hqi[i];
@@ -1239,10 +1245,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
       area = std::max(area, (unsigned long long)std::min<long long>(w, d.BW) *
                                 (unsigned long long)std::min<long long>(hh, d.BH));
     }
-    int bits = 0;
-    while (bits < 64 && (area >> bits)) ++bits;
-    d.limb = lg < 32 && 2 * lg + bits <= 64 ? 32 - lg : 0;
-    if (d.limb > 31) d.limb = 31;  // (lg = 0 cannot be: a block is 256 threads)
+    d.limb = table_limb(Mo, d.cell_blocks, area);
   }
   d.wa_blocks_total = 0;
   for (int c = 0; c < 5; ++c) {

@@ -348,6 +348,13 @@ void shuffle_plan(Dev &d);
 void launch_shuffle(const Dev &d, int copy0, int ncopy, int op, int k, uint64_t seed, cudaStream_t st);
 void launch_wiremask(const Dev &d, const WmDev &w, int copy0, int ncopy, cudaStream_t st);
 
+// The target density t = t_mant 2^-t_shift and what follows from it and the
+// bin size; false when it is out of range (api.cu).
+bool set_target(Dev &d, float target_density);
+// Bits of a scatter-table entry's low sum for n cells over `blocks` blocks,
+// each of at most `area` per bin (0: no split; api.cu).
+int table_limb(long long n, int blocks, unsigned long long area);
+
 // hooks for the job server (api.cu)
 int step_async(place_t *h, int n, int *stopped_host, cudaEvent_t ev);
 int copy_positions(place_t *dst, place_t *src, cudaEvent_t src_done);
