@@ -14,8 +14,8 @@
 //   G4  E[w][x][y] = sum_u Am_w[x][u] T[w][y][u] Am = (S_M, C_M^T, C_M^T)
 // so no transpose pass is needed between steps.
 //
-// This file holds the FP32 CUDA-core GEMM (64x64x16 tiles, 4x4 register
-// micro-tiles); the tensor-core BF16x3 path lives in spectral_tc.cu.
+// This file holds the FP32 CUDA-core GEMM; the tensor-core BF16x3 path lives in
+// spectral_tc.cu, the fast transforms in spectral_fft.cu.
 #include "common.cuh"
 #include "internal.cuh"
 #include "spectral_tc.cuh"
@@ -37,50 +37,82 @@ struct GemmArgs {
   int eval;
 };
 
-constexpr int BM = 64, BN = 64, BK = 16;
-
+// One TILE x TILE output tile per block of 256 threads, R x R outputs each, in
+// chains of fused multiply-adds over ascending k whatever the tile.  What
+// bounds it at these sizes is the latency of a step's loads, so the next step's
+// are in flight (in registers) while a step is computed, and grids of few
+// tiles take 32 x 32 ones.  A 30k-cell design's field on 368 x 176 bins:
+// 136 -> 98 us.
+template <int TILE>
 __global__ void __launch_bounds__(256) k_gemm_nt(GemmArgs g) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
+  // contraction per step (K is a multiple of 16), loader rows and loads per step
+  constexpr int BK = TILE == 32 ? 32 : 16, ROWS = 256 / (BK / 4), NL = TILE / ROWS;
+  constexpr int R = TILE / 16, LD = TILE + R;
+  __shared__ __align__(16) float As[2][BK][LD];
+  __shared__ __align__(16) float Bs[2][BK][LD];
   const int z = blockIdx.z;
   const int which = z % g.nwhich;
   const int c = g.copy0 + z / g.nwhich;
   if (!g.eval && g.cs[c].stopped) return;
   const float *A = g.A[which];
   const float *B = g.B + which * g.sBw + c * g.sBc;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int m0 = blockIdx.y * TILE, n0 = blockIdx.x * TILE;
   const int tid = threadIdx.x;
-  const int lr = tid >> 2, lk = (tid & 3) * 4;  // loader: row, k offset
+  const int lr = tid / (BK / 4), lk = tid % (BK / 4) * 4;  // loader: first row, k offset
   const int tx = tid & 15, ty = tid >> 4;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
-    float4 av = make_float4(0.f, 0.f, 0.f, 0.f), bv = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (m0 + lr < g.M) av = *reinterpret_cast<const float4 *>(A + (size_t)(m0 + lr) * g.K + k0 + lk);
-    if (n0 + lr < g.N) bv = *reinterpret_cast<const float4 *>(B + (size_t)(n0 + lr) * g.K + k0 + lk);
-    As[lk + 0][lr] = av.x; As[lk + 1][lr] = av.y; As[lk + 2][lr] = av.z; As[lk + 3][lr] = av.w;
-    Bs[lk + 0][lr] = bv.x; Bs[lk + 1][lr] = bv.y; Bs[lk + 2][lr] = bv.z; Bs[lk + 3][lr] = bv.w;
-    __syncthreads();
+  float acc[R][R] = {};
+  float4 av[NL], bv[NL];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
-      float4 b4 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
-      float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int l = 0; l < NL; ++l) {
+      const int r = lr + ROWS * l;
+      const bool in = k0 + lk < g.K;
+      av[l] = bv[l] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in && m0 + r < g.M) av[l] = *reinterpret_cast<const float4 *>(A + (size_t)(m0 + r) * g.K + k0 + lk);
+      if (in && n0 + r < g.N) bv[l] = *reinterpret_cast<const float4 *>(B + (size_t)(n0 + r) * g.K + k0 + lk);
     }
-    __syncthreads();
+  };
+  fetch(0);
+  for (int k0 = 0, p = 0; k0 < g.K; k0 += BK, p ^= 1) {
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      const int r = lr + ROWS * l;
+      As[p][lk + 0][r] = av[l].x; As[p][lk + 1][r] = av[l].y;
+      As[p][lk + 2][r] = av[l].z; As[p][lk + 3][r] = av[l].w;
+      Bs[p][lk + 0][r] = bv[l].x; Bs[p][lk + 1][r] = bv[l].y;
+      Bs[p][lk + 2][r] = bv[l].z; Bs[p][lk + 3][r] = bv[l].w;
+    }
+    __syncthreads();  // (the other buffer's readers passed the last one)
+    if (k0 + BK < g.K) fetch(k0 + BK);
+    const int parts = (min(BK, g.K - k0)) / 16;
+    for (int h = 0; h < parts; ++h) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int kk = 16 * h + q;
+        float a[R], b[R];
+        if constexpr (R == 4) {
+          *reinterpret_cast<float4 *>(a) = *reinterpret_cast<const float4 *>(&As[p][kk][ty * R]);
+          *reinterpret_cast<float4 *>(b) = *reinterpret_cast<const float4 *>(&Bs[p][kk][tx * R]);
+        } else {
+          *reinterpret_cast<float2 *>(a) = *reinterpret_cast<const float2 *>(&As[p][kk][ty * R]);
+          *reinterpret_cast<float2 *>(b) = *reinterpret_cast<const float2 *>(&Bs[p][kk][tx * R]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < R; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      }
+    }
   }
   float *D = g.D + which * g.sDw + c * g.sDc;
   const size_t GN = (size_t)g.M * g.N;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
+  for (int i = 0; i < R; ++i) {
+    const int m = m0 + ty * R + i;
     if (m >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
+    for (int j = 0; j < R; ++j) {
+      const int n = n0 + tx * R + j;
       if (n >= g.N) continue;
       const size_t o = (size_t)m * g.N + n;
       if (!g.spectral) {
@@ -99,9 +131,15 @@ __global__ void __launch_bounds__(256) k_gemm_nt(GemmArgs g) {
   }
 }
 
-static void gemm(const GemmArgs &g, int ncopy, cudaStream_t st) {
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.nwhich * ncopy);
-  k_gemm_nt<<<grid, 256, 0, st>>>(g);
+static void gemm(const GemmArgs &g, int ncopy, int sms, cudaStream_t st) {
+  const int z = g.nwhich * ncopy;
+  const dim3 wide((g.N + 63) / 64, (g.M + 63) / 64, z), small((g.N + 31) / 32, (g.M + 31) / 32, z);
+  // fewer than two 64-wide tiles per SM: the small tiles' four times as many
+  // blocks are the faster
+  if ((int)(wide.x * wide.y) * z < 2 * sms)
+    k_gemm_nt<32><<<small, 256, 0, st>>>(g);
+  else
+    k_gemm_nt<64><<<wide, 256, 0, st>>>(g);
 }
 
 void launch_spectral_fp32(const Dev &d, int copy0, int ncopy, int with_psi, int eval,
@@ -118,25 +156,25 @@ void launch_spectral_fp32(const Dev &d, int copy0, int ncopy, int with_psi, int 
   g.B = d.rho; g.sBw = 0; g.sBc = G;
   g.D = d.T; g.sDw = 0; g.sDc = 3 * G;
   g.M = N; g.N = M; g.K = N; g.nwhich = 1; g.spectral = 0;
-  gemm(g, ncopy, st);
+  gemm(g, ncopy, d.sms, st);
   // G2: A^ = Cm * T1^T   (M x N, K = M), spectral epilogue into SB
   g.A[0] = d.Cm;
   g.B = d.T; g.sBw = 0; g.sBc = 3 * G;
   g.D = d.SB; g.sDw = 0; g.sDc = 3 * G;
   g.M = M; g.N = N; g.K = M; g.spectral = 1; g.with_psi = with_psi;
-  gemm(g, ncopy, st);
+  gemm(g, ncopy, d.sms, st);
   // G3: T[w] = An_w * B_w^T   (N x M, K = N)
   g.A[0] = d.CTn; g.A[1] = d.STn; g.A[2] = d.CTn;
   g.B = d.SB; g.sBw = G; g.sBc = 3 * G;
   g.D = d.T; g.sDw = G; g.sDc = 3 * G;
   g.M = N; g.N = M; g.K = N; g.spectral = 0; g.nwhich = with_psi ? 3 : 2;
-  gemm(g, ncopy, st);
+  gemm(g, ncopy, d.sms, st);
   // G4: E[w] = Am_w * T[w]^T   (M x N, K = M)
   g.A[0] = d.STm; g.A[1] = d.CTm; g.A[2] = d.CTm;
   g.B = d.T; g.sBw = G; g.sBc = 3 * G;
   g.D = d.E; g.sDw = G; g.sDc = 3 * G;
   g.M = M; g.N = N; g.K = M;
-  gemm(g, ncopy, st);
+  gemm(g, ncopy, d.sms, st);
 }
 
 // Tensor-core chain (BF16x3): rho_hl -> T_hl[0] -> SB_hl -> T_hl[w] -> E[w].
