@@ -620,7 +620,7 @@ void enqueue_iteration(const Dev &d, cudaStream_t st, const cudaStream_t *wst, c
   const int nb = std::max(1, std::min(d.wa_streams, kMaxWaStreams));
   cudaEventRecord(fork, st);
   for (int b = 0; b < nb; ++b) cudaStreamWaitEvent(wst[b], fork, 0);
-  launch_wa_branches(d, 0, K, wst);
+  launch_wa_branches(d, 0, K, 0, nullptr, wst);
   for (int b = 0; b < nb; ++b) cudaEventRecord(join[b], wst[b]);
   // a fused solve zeroes the map that it has read; the GEMM handles clear it here
   if (!d.solve) cudaMemsetAsync(d.M, 0, sizeof(unsigned long long) * (size_t)d.Gm * K, st);
@@ -691,6 +691,10 @@ bool direct(const place_t *h, const void *p, size_t bytes) {
          (a + bytes <= own || a >= own + h->mem_bytes);
 }
 
+bool apart(const void *a, const void *b, size_t bytes) {
+  return (const char *)a + bytes <= (const char *)b || (const char *)b + bytes <= (const char *)a;
+}
+
 // Interleaved device positions -> caller's x, y (host or device), through the
 // handle's scratch where the caller's memory is not the device's own;
 // synchronises.
@@ -698,8 +702,7 @@ int copy_out_xy(place_t *h, const float2 *src, float *x, float *y) {
   const Dev &d = h->d;
   const int C = d.n_cells - d.n_fill;  // the design's cells: movable, then fixed
   const size_t bytes = sizeof(float) * C;
-  const bool apart = !x || !y || (const char *)x + bytes <= (const char *)y || (const char *)y + bytes <= (const char *)x;
-  if (apart && (!x || direct(h, x, bytes)) && (!y || direct(h, y, bytes))) {
+  if ((!x || !y || apart(x, y, bytes)) && (!x || direct(h, x, bytes)) && (!y || direct(h, y, bytes))) {
     if (x || y) launch_unpack_xy(x, y, src, d.n_real, C, d.n_fill, h->stream);
     CKL();
   } else {
@@ -1891,13 +1894,26 @@ int place_eval_wirelength(place_t *h, int32_t copy, float gamma, double *wl, flo
   CK(cudaMemcpyAsync(gdev, &gamma, sizeof(float), cudaMemcpyHostToDevice, h->stream));
   // the sums of a stopped copy's last WA pass may not have been consumed
   CK(cudaMemsetAsync(d.gacc + (size_t)copy * d.n_mov, 0, sizeof(unsigned long long) * d.n_mov, h->stream));
-  launch_wa(d, copy, 1, 1, gdev, h->stream);
-  launch_cell_grad(d, copy, 1, 1, h->stream);
+  // the classes on the iteration's branches
+  const cudaStream_t wst[kMaxWaStreams] = {h->stream, h->cap2, h->cap3};
+  const cudaEvent_t joins[kMaxWaStreams] = {h->ev_join, h->ev_join2, h->ev_join3};
+  const int nb = std::max(1, std::min(d.wa_streams, kMaxWaStreams));
+  if (nb > 1) CK(cudaEventRecord(h->ev_fork, h->stream));
+  for (int b = 1; b < nb; ++b) CK(cudaStreamWaitEvent(wst[b], h->ev_fork, 0));
+  launch_wa_branches(d, copy, 1, 1, gdev, wst);
+  for (int b = 1; b < nb; ++b) {
+    CK(cudaEventRecord(joins[b], wst[b]));
+    CK(cudaStreamWaitEvent(h->stream, joins[b], 0));
+  }
+  const size_t Mo = d.n_mov, Mv = d.n_real;  // per-copy stride, the design's movable cells
+  float *ox = d.gwx + copy * Mo, *oy = d.gwy + copy * Mo;
+  const size_t bytes = sizeof(float) * Mv;
+  const bool in_place = gx && gy && direct(h, gx, bytes) && direct(h, gy, bytes) && apart(gx, gy, bytes);
+  launch_wa_unpack(d, copy, in_place ? gx : ox, in_place ? gy : oy, h->stream);
   launch_reduce_slot(d, S_WL, d.wa_blocks_total, copy, 1, h->stream);
   CKL();
-  const size_t Mo = d.n_mov, Mv = d.n_real;  // per-copy stride, the design's movable cells
-  if (gx) CK(cudaMemcpyAsync(gx, d.gwx + copy * Mo, sizeof(float) * Mv, cudaMemcpyDefault, h->stream));
-  if (gy) CK(cudaMemcpyAsync(gy, d.gwy + copy * Mo, sizeof(float) * Mv, cudaMemcpyDefault, h->stream));
+  if (gx && !in_place) CK(cudaMemcpyAsync(gx, ox, bytes, cudaMemcpyDefault, h->stream));
+  if (gy && !in_place) CK(cudaMemcpyAsync(gy, oy, bytes, cudaMemcpyDefault, h->stream));
   double v = 0;
   CK(cudaMemcpyAsync(&v, d.scal + (size_t)copy * S_COUNT + S_WL, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));

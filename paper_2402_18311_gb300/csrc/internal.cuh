@@ -301,10 +301,11 @@ void launch_spectral_tc_stalled(const Dev &d, cudaStream_t st);
 void launch_test_bounds(const Dev &d, cudaStream_t st);
 void launch_wa(const Dev &d, int copy0, int ncopy, int eval, const float *gamma_override,
                cudaStream_t st);
-// The WA classes of an iteration on d.wa_streams branches: branch b's classes
+// The WA classes on d.wa_streams branches: branch b's classes
 // run in sequence on st[b] (st[0..wa_streams-1]); every branch must already
 // follow the positions' producer.
-void launch_wa_branches(const Dev &d, int copy0, int ncopy, const cudaStream_t *st);
+void launch_wa_branches(const Dev &d, int copy0, int ncopy, int eval, const float *gamma_override,
+                        const cudaStream_t *st);
 constexpr int kMaxWaStreams = 3;
 void launch_hpwl64(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 int wa_prepare(int cap);
@@ -335,6 +336,7 @@ struct TuneHooks {
 int autotune(Dev &d, int max_deg, cudaStream_t st, const TuneHooks &hk, TuneOut *out);
 int cell_grad_blocks_per_sm(const Dev &d);
 void launch_cell_grad(const Dev &d, int copy0, int ncopy, int eval, cudaStream_t st);
+void launch_wa_unpack(const Dev &d, int copy, float *gx, float *gy, cudaStream_t st);
 void launch_precond0(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 void launch_update(const Dev &d, int copy0, int ncopy, cudaStream_t st);
 // src: new positions of cells [lo, hi) (device arrays of hi - lo; none: null).

@@ -612,6 +612,24 @@ void launch_unpack_xy(float *x, float *y, const float2 *src, int n0, int n, int 
   k_unpack_xy<<<b < 4096 ? b : 4096, kThreads, 0, st>>>(x, y, src, n0, n, skip);
 }
 
+// A copy's WA gradient sums as floats (the design's movable cells), and cleared
+// for the next pass: place_eval_wirelength, which needs nothing else of the
+// cell-gradient pass.
+__global__ void __launch_bounds__(kThreads) k_wa_unpack(Dev d, int copy, float *gx, float *gy) {
+  unsigned long long *ga = d.gacc + (size_t)copy * d.n_mov;
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < d.n_mov; i += gridDim.x * kThreads) {
+    const float2 g = unpack_grad(d, ga[i]);
+    ga[i] = 0ull;
+    if (i < d.n_real) {
+      gx[i] = g.x;
+      gy[i] = g.y;
+    }
+  }
+}
+void launch_wa_unpack(const Dev &d, int copy, float *gx, float *gy, cudaStream_t st) {
+  k_wa_unpack<<<d.cell_blocks, kThreads, 0, st>>>(d, copy, gx, gy);
+}
+
 namespace {
 using CellGrad = void (*)(Dev, int, int);
 CellGrad cell_grad_kernel(bool stretch, bool pair, bool big) {

@@ -613,7 +613,8 @@ void launch_wa(const Dev &d, int copy0, int ncopy, int eval, const float *gamma_
 // few long blocks then overlap the others' many short ones).
 constexpr int kWaBranch[3][5] = {{0, 0, 0, 0, 0}, {0, 0, 1, 1, 1}, {0, 1, 1, 2, 2}};
 
-void launch_wa_branches(const Dev &d, int copy0, int ncopy, const cudaStream_t *st) {
+void launch_wa_branches(const Dev &d, int copy0, int ncopy, int eval, const float *gamma_ovr,
+                        const cudaStream_t *st) {
   const int nb = d.wa_streams < 1 ? 1 : (d.wa_streams > kMaxWaStreams ? kMaxWaStreams : d.wa_streams);
   int launched[kMaxWaStreams] = {0, 0, 0};
   for (int cls = 0; cls < d.n_cls; ++cls) {
@@ -621,7 +622,7 @@ void launch_wa_branches(const Dev &d, int copy0, int ncopy, const cudaStream_t *
     const int b = kWaBranch[nb - 1][cls < 5 ? cls : 4];
     // the first class of a branch follows the branch's fork; the others
     // follow a WA kernel and launch programmatically
-    launch_wa_one(d, cls, copy0, ncopy, 0, nullptr, launched[b]++ > 0, st[b]);
+    launch_wa_one(d, cls, copy0, ncopy, eval, gamma_ovr, launched[b]++ > 0, st[b]);
   }
 }
 
