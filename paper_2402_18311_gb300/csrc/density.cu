@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter(Dev d, int copy0, int e
   unsigned long long *M = STRETCH ? d.Ms + (size_t)c * d.G : d.M + (size_t)c * d.Gm;
   scatter_block<STRETCH, BIG>(
       d, d.n_mov, d.cs[c].n_eff, M, STRETCH ? d.G : d.Gm, keys, vals,
-      [&](ScatterCell<STRETCH> &cell, int i, bool) { cell.load(d, xy, i); },
+      [&](ScatterCell<STRETCH> &cell, int i) { cell.load(d, xy, i); },
       [&](int i) { return (STRETCH || i < d.n_real) ? 0 : d.G; });
 }
 

@@ -107,10 +107,10 @@ __global__ void __launch_bounds__(kNaThreads)
   bool bad = false;
   scatter_block<false, true>(
       d, n, 0.0, s->map, d.G, keys, vals,
-      [&](ScatterCell<false> &cell, int i, bool real) {
+      [&](ScatterCell<false> &cell, int i) {
         long long W = 0, H = 0;
         if (na_size(w[i], h[i], d.scale, W, H)) {
-          if (real) area += (u128)(unsigned long long)(W * H);
+          area += (u128)(unsigned long long)(W * H);
           cell.R = 0u;
           cell.r = qrect32(x[i], y[i], (int)W, (int)H, d.scale, d.XL, d.YL, d.BW32, d.BH32, d.nx,
                            d.ny, d.ibw_q, d.ibh_q);

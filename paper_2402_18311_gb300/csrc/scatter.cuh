@@ -137,7 +137,7 @@ struct ScatterCell {
 // after another by the whole warp: every lane takes every 32nd bin, straight
 // to the map (a cell's bins are distinct, so nothing contends).  Left to its
 // one lane, a macro of 17 x 17 bins held a pass of the 210k-cell mixed-size
-// design for 250 us instead of BIGMEASURE.
+// design for 250 us; the whole scatter and finish there now take 26.
 template <bool STRETCH>
 __device__ __forceinline__ void scatter_big(const Dev &d, const ScatterCell<STRETCH> &cell, int mo,
                                             unsigned long long *M, int lim) {
@@ -185,9 +185,9 @@ __device__ __forceinline__ void scatter_big(const Dev &d, const ScatterCell<STRE
 // ways, and from kWarpBins bins on go to the whole warp in all three.  Every
 // way adds the same integers, so the map is the same.
 // One block's part of a scatter of n cells into the map M of lim entries:
-// load(cell, i, real) reads cell i (real: false for the sample), offset(i) is
-// added to its bins.  keys, vals: the block's table (kHash entries).  BIG:
-// there may be cells of more than kWarpBins bins.
+// load(cell, i) reads cell i (each once), offset(i) is added to its bins.  keys,
+// vals: the block's table (kHash entries).  BIG: there may be cells of more
+// than kWarpBins bins.
 template <bool STRETCH, bool BIG, typename Load, typename Offset>
 __device__ __forceinline__ void scatter_block(const Dev &d, int n, double n_eff, unsigned long long *M,
                                               int lim, int *keys, unsigned long long *vals, Load load,
@@ -197,25 +197,23 @@ __device__ __forceinline__ void scatter_block(const Dev &d, int n, double n_eff,
   int mode = d.scat_force >= 0 ? d.scat_force
                                : (n_eff < d.scat_t1 ? SCAT_MERGED
                                                     : (n_eff < d.scat_t2 ? SCAT_TABLE : SCAT_DIRECT));
+  // (a warp's lanes stay together: i0 is its first cell)
+  int i0 = blockIdx.x * kThreads + (threadIdx.x & ~31);
+  ScatterCell<STRETCH> cell;
+  auto fetch = [&]() {
+    if (i0 + lane < n) load(cell, i0 + lane);
+    else cell.none();
+  };
+  fetch();
   if (d.scat_force < 0 && n_eff == 0.0) {
-    const int i = blockIdx.x * kThreads + threadIdx.x;
-    int b = -1 - lane;  // distinct where there is no cell
-    if (i < n) {
-      ScatterCell<STRETCH> cell;
-      load(cell, i, false);
-      if (cell.bins()) b = cell.r.ix0 * d.ny + cell.r.iy0;
-    }
+    // (distinct where there is no cell)
+    const int b = cell.bins() ? cell.r.ix0 * d.ny + cell.r.iy0 : -1 - lane;
     const int shared = __syncthreads_count(lane != __ffs(__match_any_sync(0xffffffffu, b)) - 1);
     mode = shared <= kSampleDirect ? SCAT_DIRECT : (shared <= kSampleTable ? SCAT_TABLE : SCAT_MERGED);
   }
   if (mode == SCAT_DIRECT) {
-    // (warp-uniform trip count here and below)
-    for (int i0 = blockIdx.x * kThreads + (threadIdx.x & ~31); i0 < n; i0 += stride) {
-      const int i = i0 + lane;
-      const int mo = offset(i);
-      ScatterCell<STRETCH> cell;
-      if (i < n) load(cell, i, true);
-      else cell.none();
+    while (i0 < n) {
+      const int mo = offset(i0 + lane);
       if (!BIG || cell.bins() <= kWarpBins) {
         for (int ix = cell.r.ix0; ix <= cell.r.ix1; ++ix) {
           for (int iy = cell.r.iy0; iy <= cell.r.iy1; ++iy) {
@@ -226,6 +224,8 @@ __device__ __forceinline__ void scatter_block(const Dev &d, int n, double n_eff,
         }
       }
       if constexpr (BIG) scatter_big(d, cell, mo, M, lim);
+      i0 += stride;
+      fetch();
     }
     return;
   }
@@ -236,12 +236,8 @@ __device__ __forceinline__ void scatter_block(const Dev &d, int n, double n_eff,
   __syncthreads();
   // one cell's overlap with one bin is at most the bin area
   const bool two_limbs = (double)d.BW * (double)d.BH < 4398046511104.0;  // 2^42
-  for (int i0 = blockIdx.x * kThreads + (threadIdx.x & ~31); i0 < n; i0 += stride) {
-    const int i = i0 + lane;
-    const int mo = offset(i);
-    ScatterCell<STRETCH> cell;
-    if (i < n) load(cell, i, true);
-    else cell.none();
+  while (i0 < n) {
+    const int mo = offset(i0 + lane);
     const bool lone = !BIG || cell.bins() <= kWarpBins;  // added by its own lane
     int done = 0;  // slots per axis that the merge has added
     if (mode == SCAT_MERGED) {
@@ -301,6 +297,8 @@ __device__ __forceinline__ void scatter_block(const Dev &d, int n, double n_eff,
       __syncwarp();
       scatter_big(d, cell, mo, M, lim);
     }
+    i0 += stride;
+    fetch();
   }
   __syncthreads();
   for (int i = threadIdx.x; i < kHash; i += blockDim.x) {
