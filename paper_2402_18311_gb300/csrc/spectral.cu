@@ -134,9 +134,12 @@ __global__ void __launch_bounds__(256) k_gemm_nt(GemmArgs g) {
 static void gemm(const GemmArgs &g, int ncopy, int sms, cudaStream_t st) {
   const int z = g.nwhich * ncopy;
   const dim3 wide((g.N + 63) / 64, (g.M + 63) / 64, z), small((g.N + 31) / 32, (g.M + 31) / 32, z);
-  // fewer than two 64-wide tiles per SM: the small tiles' four times as many
-  // blocks are the faster
-  if ((int)(wide.x * wide.y) * z < 2 * sms)
+  // Fewer 64-wide tiles than half the SMs: the small tiles' four times as many
+  // blocks are the faster.  Small / wide, a field on 368 x 176 bins (18 tiles a
+  // field) 97 / 113 us, 496 x 496 (64) 176 / 184; 496 x 752 (96) 231 / 222,
+  // 496 x 1008 (128) 328 / 294, 1008 x 1008 (256) 710 / 635 (712 before the
+  // loads were in flight).
+  if ((int)(wide.x * wide.y) * z < (sms + 1) / 2)
     k_gemm_nt<32><<<small, 256, 0, st>>>(g);
   else
     k_gemm_nt<64><<<wide, 256, 0, st>>>(g);

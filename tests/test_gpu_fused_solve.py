@@ -101,3 +101,27 @@ def test_evaluations_between_iterations_change_nothing(nx, opts):
         finally:
             place.place_destroy(h)
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nx,ny", [(144, 112), (48, 176)])  # sides of 32 k + 16
+def test_gemm_tiles_agree(nx, ny):
+    # one copy takes the GEMMs' small tiles, forty the wide ones: the same
+    # chain of multiply-adds per element, so the same bits
+    d = _design(nx, ny, seed=12)
+    got = []
+    for copies in (1, 40):
+        h = place.place_create(d, place.place_default_params(
+            tau_stop=-1.0, autotune=0, n_copies=copies, dct_mode=place.PLACE_DCT_FP32))
+        try:
+            place.place_step(h, 15)
+            for c in {0, copies - 1}:
+                x, y = np.empty(d.n_cells, np.float32), np.empty(d.n_cells, np.float32)
+                place.place_get_positions(h, c, x, y)
+                e = np.empty((2, nx * ny), np.float32)
+                place.place_eval_field(h, c, None, e[0], e[1])
+                got.append((x, y, e))
+        finally:
+            place.place_destroy(h)
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            np.testing.assert_array_equal(a, b)
