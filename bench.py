@@ -152,6 +152,17 @@ def dist_env():
     return rank, world, local
 
 
+def fast_transforms(dct, d):
+    """Whether the handle solves by fast transforms: power-of-two sides (a
+    64 x 64 grid is one cluster's), and the mode left to the library or FP32."""
+    return (dct != 1 and d.nx * d.ny > 4096
+            and all(64 <= n <= 4096 and n & (n - 1) == 0 for n in (d.nx, d.ny)))
+
+
+def solve_name(dct, d, info):
+    return "fast transforms, fp32" if fast_transforms(dct, d) else ["fp32", "bf16x3"][info.dct_mode]
+
+
 def algorithmic(d, info):
     """Algorithmic bytes / flops of one iteration per stage (one copy)."""
     C, P, E, G = d.n_movable, d.n_pins, d.n_nets, d.nx * d.ny
@@ -279,6 +290,10 @@ def run_ours(args):
     e2e_v = world * n_e2e / e2e_s
 
     alg = algorithmic(d, info)
+    if fast_transforms(args.dct, d):
+        # one forward and two inverse 2-D transforms (the first half of the
+        # forward one is timed with the density stage)
+        alg["spectral"] = {"flops": 7.5 * d.nx * d.ny * float(np.log2(d.nx * d.ny))}
     pk, pk_kind = peaks()
     names = ["density", "spectral", "wirelength", "cellgrad", "update"]
     dom = int(np.argmax(stage_ms))
@@ -288,7 +303,7 @@ def run_ours(args):
         sec = float(stage_ms[i]) / 1e3
         if "flops" in a:
             per[n] = {"ms": float(stage_ms[i]), "TFLOP/s": a["flops"] / sec / 1e12 if sec > 0 else None}
-            if info.dct_mode == 1 and sec > 0:
+            if "flops_pipe" in a and info.dct_mode == 1 and sec > 0:
                 # what the tensor pipe executed, against the measured bf16 peak
                 per[n]["pipe_TFLOP/s"] = a["flops_pipe"] / sec / 1e12
                 per[n]["pipe_frac_of_bf16"] = a["flops_pipe"] / sec / 1e12 / pk["bf16_tflops"]
@@ -334,12 +349,12 @@ def run_ours(args):
         "metric": METRIC, "value": value, "unit": "iters/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f32" if args.dct == 0 else "f32+bf16x3", "data": "synthetic",
+        "dtype": "f32+bf16x3" if "bf16" in solve_name(args.dct, d, info) else "f32", "data": "synthetic",
         "config": {"workload": args.workload, "desc": desc, "copies_per_gpu": prm.n_copies,
                    "parallelism": f"replicas{world}", "l2": "inputs larger than L2 "
                    "(per-iteration working set > 129 MB)" if args.workload == "large_2m"
                    else "working set fits L2 (no flush)",
-                   "dct_mode": ["fp32", "bf16x3"][args.dct], "tuning": tuning(info),
+                   "dct_mode": solve_name(args.dct, d, info), "tuning": tuning(info),
                    "timed_iterations": [args.advance + args.warmup + 1,
                                         args.advance + args.warmup + args.steps]},
         "e2e": {"value": e2e_v, "unit": "iters/s",
@@ -466,7 +481,7 @@ def run_configs(args, place, torch):
     rh, rt = place.place_get_hybro_rounds(h, 0)
     place.place_destroy(h)
     out["tiny_1k"] = {"desc": WORKLOADS["tiny_1k"][1], "iterations": 600, "seconds": el,
-                      "iters_per_s": 600 / el, "spectral": ["fp32", "bf16x3"][info.dct_mode],
+                      "iters_per_s": 600 / el, "spectral": solve_name(place.PLACE_DCT_AUTO, d, info),
                       "round_hpwl": rh.tolist(), "round_overflow": rt.tolist(),
                       "best_round": int(br[0]), "best_hpwl": float(bh[0]),
                       "note": "300 iterations, Shuffle (all) p = 0.5 seed 0, 300 more; host "
@@ -494,7 +509,7 @@ def run_configs(args, place, torch):
                           "converged": bool(st.converged), "seconds": ms / 1e3,
                           "iters_per_s": 1e3 * st.iter / ms, "final_overflow": float(tv[0]),
                           "final_hpwl": float(hp[0]),
-                          "spectral": ["fp32", "bf16x3"][info.dct_mode],
+                          "spectral": solve_name(args.dct, d, info),
                           "note": "to overflow <= 0.07 or 1,000 iterations, CUDA events around "
                                   "the whole run (50-iteration launches, stop flags read back)"}
     return out
@@ -831,8 +846,9 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default="large_2m", choices=sorted(WORKLOADS))
-    ap.add_argument("--dct", type=int, default=1, choices=[0, 1],
-                    help="spectral solve: 1 = BF16x3 on tcgen05 tensor cores, 0 = FP32 CUDA cores")
+    ap.add_argument("--dct", type=int, default=-1, choices=[-1, 0, 1],
+                    help="spectral solve: -1 = the library's choice, 1 = BF16x3 on tcgen05 tensor "
+                         "cores, 0 = FP32 CUDA cores")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-restarts", action="store_true",
                     help="skip the batched-vs-serial restarts measurement")

@@ -49,8 +49,14 @@ extern "C" {
 
 /* Spectral-solve arithmetic. */
 #define PLACE_DCT_AUTO (-1) /* the default: PLACE_DCT_BF16X3 when nx and ny are
-                               multiples of 128, else PLACE_DCT_FP32 */
-#define PLACE_DCT_FP32 0   /* FP32 CUDA-core GEMMs (any grid, multiples of 16) */
+                               multiples of 128, else PLACE_DCT_FP32; but where both
+                               sides are powers of two (64 .. 4096) and dct_fold is 1,
+                               FP32 fast transforms do the solve (faster, and closer to
+                               the exact field) and the resolved mode's resources are
+                               kept beside them */
+#define PLACE_DCT_FP32 0   /* FP32 CUDA cores (any grid, multiples of 16): fast
+                              transforms where both sides are powers of two (64 ..
+                              4096), one kernel up to 4096 bins, GEMMs otherwise */
 #define PLACE_DCT_BF16X3 1 /* split-BF16 (3 products, FP32 accumulation) on the
                               tcgen05 tensor cores; grids must be multiples of 128 */
 
@@ -164,8 +170,9 @@ typedef struct place_params {
                              classes run as a chain on one graph branch, or
                              split over two or three branches that run side by
                              side (integer gradient sums: the same bits) */
-  int32_t dct_fold;       /* 1 (default): on the BF16x3 path with both grid sides
-                             multiples of 256, every transform is split into its
+  int32_t dct_fold;       /* 1 (default): with PLACE_DCT_AUTO, fast transforms where the
+                             grid allows them (above); on the BF16x3 path with both grid
+                             sides multiples of 256, every transform is split into its
                              even and odd frequencies (the first step of a fast
                              cosine transform), which halves the tensor-core
                              work of the solve; 0: the plain GEMMs.  Both solve
@@ -181,7 +188,9 @@ typedef struct place_info {
   int64_t device_bytes;   /* device memory the handle holds */
   int32_t kernels_per_iter; /* this library's kernel launches in one iteration (the first
                               iteration after a reset adds one: k_precond0) */
-  int32_t dct_mode;       /* the spectral path in use: PLACE_DCT_FP32 or _BF16X3 */
+  int32_t dct_mode;       /* the resolved mode, PLACE_DCT_FP32 or _BF16X3 (with
+                             PLACE_DCT_AUTO on power-of-two sides the fast transforms
+                             solve in either, see there) */
   int32_t n_fillers;      /* filler cells (0 unless params.fillers) */
   int32_t bounds_checked; /* 1: the library was built with index checks
                            * (-DPLACE_DEBUG_BOUNDS): a failed check makes the
@@ -193,7 +202,7 @@ typedef struct place_info {
   double scatter_t1, scatter_t2; /* effective-bin thresholds of the scatter's ways */
   double autotune_ms;     /* host time the tuning took at create (0 on a cache hit) */
   int32_t wa_streams;     /* graph branches the WA classes run on (1..3) */
-  int32_t dct_fold;       /* 1: the solve runs the even/odd split (params.dct_fold) */
+  int32_t dct_fold;       /* 1: the BF16x3 path has the even/odd split (params.dct_fold) */
 } place_info;
 
 /* Optimiser scalars of one copy after its last iteration. */
