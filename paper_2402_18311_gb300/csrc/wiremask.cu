@@ -31,7 +31,7 @@
 //   - k_wm_mask per macro: each net's extent with the macros' pins added (a
 //     short list made at create), the two mask axes with the distances of
 //     their corners, and every obstacle as the exact range of candidate
-//     columns and rows that it blocks (binary searches);
+//     columns and rows that it blocks (stepping from a guess);
 //   - k_wm_select per macro: a block per row of candidates turns the
 //     obstacles that cover the row into a bit mask, so that a candidate costs
 //     one bit test, one FP64 addition and one comparison; the last block
