@@ -635,7 +635,7 @@ def run_wiremask(args, place, torch, rounds=3, reps=5):
     place.place_eval_hpwl_overflow(h, hp1, tau1)
     out = {"workload": "medium_mixed_210k: medium_210k with 32 movable macros of 16-64 units",
            "macros": int(d.is_macro[:d.n_movable].sum()), "grid": f"{d.nx}x{d.ny}",
-           "wiremask_pass_ms": 1e3 * t_wm, "launches_per_pass": 4 * 32,
+           "wiremask_pass_ms": 1e3 * t_wm, "launches_per_pass": 1 + 2 * 32,
            "converged_hpwl": float(hp0[0]), "converged_overflow": float(tau0[0]),
            "hpwl_after_wiremask": float(hp1[0]), "rounds": rounds}
     for name, op, p in (("wiremask", place.PLACE_WIREMASK, 0.0),
