@@ -261,6 +261,7 @@ struct place_t {
   // run kUnrollAfter iterations
   cudaGraphExec_t exec_n = nullptr;
   long long n_iters = 0;
+  bool no_runs = false;  // there was no memory for that graph: one at a time
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
@@ -749,7 +750,7 @@ int launch_iters(place_t *h, int n) {
   if (int rc = ensure_graph(h)) return rc;
   int i = 0;
   while (i < n) {
-    const bool run = !h->k0_pending && n - i >= kUnroll;
+    const bool run = !h->k0_pending && !h->no_runs && n - i >= kUnroll;
     if (run && !h->exec_n && h->n_iters >= kUnrollAfter) {
       const cudaStream_t wst[kMaxWaStreams] = {h->cap2, h->cap3, h->cap4};
       const cudaEvent_t joins[kMaxWaStreams] = {h->ev_join, h->ev_join2, h->ev_join3};
@@ -759,8 +760,11 @@ int launch_iters(place_t *h, int n) {
       cudaError_t e = cudaStreamEndCapture(h->cap, &g);
       if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec_n, g, 0);
       if (g) cudaGraphDestroy(g);
-      if (e != cudaSuccess) {
-        h->exec_n = nullptr;
+      if (e != cudaSuccess) h->exec_n = nullptr;
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        h->no_runs = true;
+      } else if (e != cudaSuccess) {
         return fail(PLACE_ECUDA, "graph of %d iterations: %s", kUnroll, cudaGetErrorString(e));
       }
     }
