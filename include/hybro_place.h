@@ -285,8 +285,9 @@ int place_step_multi(place_t *const *hs, int32_t n, int32_t n_iters, int32_t *co
  * L1 distance from the macro's old corner, then the lowest bin row, then the
  * lowest column.  A macro with no free corner stays where it is.  The first
  * WireMask call allocates device scratch of about
- * K (16 (nx + ny) + 20 ny + 32 nets_of_macros + 16 (fixed cells + macros))
- * bytes, freed by place_destroy.  It runs two small kernels per macro, captured
+ * K (16 (nx + ny) + 20 ny + 32 (E + S) + 16 (fixed cells + macros)) bytes, E the
+ * nets of every macro added up, S the nets that several macros share, freed by
+ * place_destroy.  It runs two small kernels per macro, captured
  * into a CUDA graph on the first call for each copy selection and replayed
  * by later calls (the graph is freed by place_destroy).  A design
  * without movable macros only resets the optimiser.  EINVAL on an unknown

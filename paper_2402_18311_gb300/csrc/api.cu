@@ -265,11 +265,13 @@ struct place_t {
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
-  std::vector<int> wm_order, wm_ptr, wm_net, wm_pin_ptr, wm_pin, wm_obst;
+  std::vector<int> wm_order, wm_ptr, wm_more, wm_net, wm_cell, wm_slot, wm_dptr, wm_dent, wm_obst;
+  std::vector<float4> wm_own;
+  int wm_shared = 0;
   void *wm_mem = nullptr;
   WmDev wm{};
   // one captured graph per (first copy, copies) of a WireMask pass: the pass
-  // is four small kernels per macro, so its launches dominate otherwise
+  // is two small kernels per macro, so its launches dominate otherwise
   std::map<std::pair<int, int>, cudaGraphExec_t> wm_graphs;
   // Hybro bookkeeping (host)
   std::vector<double> best_hpwl, best_tau;
@@ -797,17 +799,26 @@ int ensure_wiremask(place_t *h) {
   w.n_macros = (int)h->wm_order.size();
   w.n_fixed = d.n_cells - d.n_mov;
   w.n_entries = (int)h->wm_net.size();
-  const size_t K = d.K;
+  w.n_dnets = (int)h->wm_dptr.size() - 1;
+  w.n_shared = h->wm_shared;
+  const size_t K = d.K, n = std::max(w.n_entries, 1);
   Arena a;
-  int *order = nullptr, *mptr = nullptr, *mnet = nullptr, *obst = nullptr, *pptr = nullptr, *pin = nullptr;
+  int *order = nullptr, *mptr = nullptr, *more = nullptr, *mnet = nullptr, *mcell = nullptr, *slot = nullptr,
+      *dptr = nullptr, *dent = nullptr, *obst = nullptr;
+  float4 *own = nullptr;
   auto lay = [&]() {
     order = a.take<int>(w.n_macros);
     mptr = a.take<int>(w.n_macros + 1);
-    mnet = a.take<int>(std::max<size_t>(h->wm_net.size(), 1));
-    pptr = a.take<int>(h->wm_pin_ptr.size());
-    pin = a.take<int>(std::max<size_t>(h->wm_pin.size(), 1));
+    more = a.take<int>(w.n_macros);
+    mnet = a.take<int>(n);
+    mcell = a.take<int>(n);
+    slot = a.take<int>(n);
+    own = a.take<float4>(n);
+    dptr = a.take<int>(w.n_dnets + 1);
+    dent = a.take<int>(n);
     obst = a.take<int>(h->wm_obst.size());
-    w.sbox = a.take<double>(K * std::max(w.n_entries, 1) * 4);
+    w.sbox = a.take<double>(K * n * 4);
+    w.moved = a.take<double>(K * std::max(w.n_shared, 1) * 4);
     w.f = a.take<double>(K * (d.nx + d.ny));
     w.dist = a.take<double>(K * (d.nx + d.ny));
     w.range = a.take<int4>(K * (size_t)(w.n_fixed + w.n_macros));
@@ -825,17 +836,22 @@ int ensure_wiremask(place_t *h) {
   a = Arena();
   a.base = (char *)mem;
   lay();
-  w.order = order; w.mptr = mptr; w.mnet = mnet; w.obst = obst; w.mpin_ptr = pptr; w.mpin = pin;
-  auto up = [&](int *dst, const std::vector<int> &src) -> int {
+  w.order = order; w.mptr = mptr; w.more = more; w.mnet = mnet; w.mcell = mcell; w.slot = slot;
+  w.own = own; w.dptr = dptr; w.dent = dent; w.obst = obst;
+  auto up = [&](auto *dst, const auto &src) -> int {
     if (!src.empty())
-      CK(cudaMemcpyAsync(dst, src.data(), sizeof(int) * src.size(), cudaMemcpyHostToDevice, h->stream));
+      CK(cudaMemcpyAsync(dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice, h->stream));
     return PLACE_OK;
   };
   int rc = up(order, h->wm_order);
   if (!rc) rc = up(mptr, h->wm_ptr);
+  if (!rc) rc = up(more, h->wm_more);
   if (!rc) rc = up(mnet, h->wm_net);
-  if (!rc) rc = up(pptr, h->wm_pin_ptr);
-  if (!rc) rc = up(pin, h->wm_pin);
+  if (!rc) rc = up(mcell, h->wm_cell);
+  if (!rc) rc = up(slot, h->wm_slot);
+  if (!rc) rc = up(own, h->wm_own);
+  if (!rc) rc = up(dptr, h->wm_dptr);
+  if (!rc) rc = up(dent, h->wm_dent);
   if (!rc) rc = up(obst, h->wm_obst);
   if (!rc && (e = cudaMemsetAsync(w.ctr, 0, sizeof(unsigned int) * K, h->stream)) != cudaSuccess)
     rc = fail(PLACE_ECUDA, "WireMask scratch: %s", cudaGetErrorString(e));
@@ -1252,24 +1268,53 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
     });
     std::vector<int> slot(C, -1);
     for (size_t t = 0; t < mo.size(); ++t) slot[mo[t]] = (int)t;
-    std::vector<std::vector<int>> nets(mo.size());
+    // an entry per (macro, net), and with it the extent of the macro's pin
+    // offsets on the net; all tables are linear in the pins
+    struct Entry {
+      int net;
+      float4 own;
+    };
+    std::vector<std::vector<Entry>> nets(mo.size());
     for (int e = 0; e < E; ++e)
       for (int j = nl->net_ptr[e]; j < nl->net_ptr[e + 1]; ++j) {
         const int t = slot[nl->pin_cell[j]];
-        if (t >= 0 && (nets[t].empty() || nets[t].back() != lib_of[e])) nets[t].push_back(lib_of[e]);
+        if (t < 0) continue;
+        if (nets[t].empty() || nets[t].back().net != lib_of[e])
+          nets[t].push_back({lib_of[e], make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY)});
+        float4 &o = nets[t].back().own;
+        const float ox = nl->pin_dx[j], oy = nl->pin_dy[j];
+        o = make_float4(std::fmin(o.x, ox), std::fmax(o.y, ox), std::fmin(o.z, oy), std::fmax(o.w, oy));
       }
     h->wm_ptr.assign(1, 0);
+    std::vector<int> count(E, 0), at(E, -1);  // a net's entries; its number among the distinct nets
     for (size_t t = 0; t < mo.size(); ++t) {
-      h->wm_net.insert(h->wm_net.end(), nets[t].begin(), nets[t].end());
+      for (const Entry &en : nets[t]) {
+        h->wm_net.push_back(en.net);
+        h->wm_cell.push_back(mo[t]);
+        h->wm_own.push_back(en.own);
+        ++count[en.net];
+      }
       h->wm_ptr.push_back((int)h->wm_net.size());
     }
-    // each entry's pins on movable macros (the only ones that move in a pass)
-    h->wm_pin_ptr.assign(1, 0);
+    // the entries of each distinct net, ascending (the macros' order)
+    h->wm_dptr.assign(1, 0);
+    std::vector<int> shared(E, -1), left(count);
     for (int ne : h->wm_net) {
-      for (int j = net_ptr[ne]; j < net_ptr[ne + 1]; ++j)
-        if (pin_cell[j] < Mv && macro[pin_cell[j]]) h->wm_pin.push_back(j);
-      h->wm_pin_ptr.push_back((int)h->wm_pin.size());
+      if (at[ne] >= 0) continue;
+      at[ne] = (int)h->wm_dptr.size() - 1;
+      h->wm_dptr.push_back(h->wm_dptr.back() + count[ne]);
+      if (count[ne] > 1) shared[ne] = h->wm_shared++;
     }
+    const int n_ent = (int)h->wm_net.size();
+    h->wm_dent.resize(n_ent);
+    h->wm_more.assign(mo.size(), 0);
+    for (size_t t = 0; t < mo.size(); ++t)
+      for (int s = h->wm_ptr[t]; s < h->wm_ptr[t + 1]; ++s) {
+        const int ne = h->wm_net[s];
+        h->wm_dent[h->wm_dptr[at[ne]] + count[ne] - left[ne]] = s;
+        if (--left[ne] > 0) h->wm_more[t] = 1;
+        h->wm_slot.push_back(shared[ne]);
+      }
     for (int i = Mv; i < C; ++i) h->wm_obst.push_back(ci(i));
     h->wm_obst.insert(h->wm_obst.end(), mo.begin(), mo.end());
   }

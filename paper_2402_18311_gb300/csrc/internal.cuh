@@ -220,13 +220,20 @@ struct WmDev {
   int n_macros;         // movable macros
   int n_fixed;          // fixed cells: the obstacles every macro avoids
   int n_entries;        // nets over all macros: mptr[n_macros]
+  int n_dnets;          // the distinct ones, and those with several macros
+  int n_shared;
   const int *order;     // [n_macros] macros by decreasing area, ties by index
   const int *mptr;      // [n_macros + 1] macro t's nets: entries mptr[t] .. mptr[t+1]
+  const int *more;      // [n_macros] some later macro is on one of macro t's nets
   const int *mnet;      // [n_entries] library net indices, in netlist order per macro
-  const int *mpin_ptr;  // [n_entries + 1] entry s's pins on movable macros:
-  const int *mpin;      // mpin[mpin_ptr[s] .. mpin_ptr[s+1]), library pin indices
+  const int *mcell;     // [n_entries] the entry's macro
+  const int *slot;      // [n_entries] its net among those with several macros, or -1
+  const float4 *own;    // [n_entries] extent of its pin offsets {x-, x+, y-, y+}
+  const int *dptr;      // [n_dnets + 1] each net's entries: dent[dptr[n] .. dptr[n+1]),
+  const int *dent;      // [n_entries] ascending
   const int *obst;      // [n_fixed + n_macros] fixed cells, then `order`
-  double *sbox;         // [K][n_entries][4] extents of the entries' other pins
+  double *sbox;         // [K][n_entries][4] extents of the entries' other pins, without
+  double *moved;        // [K][n_shared][4] the macros that have moved: those here
   double *f, *dist;     // [K][nx + ny] wire-mask axes (columns, rows) and distances
   int4 *range;          // [K][n_fixed + n_macros] blocked columns and rows
   unsigned long long *bobj, *bdist;  // [K][ny] the rows' winners

@@ -25,19 +25,26 @@
 // What bounds it: the chain over the macros, so everything that does not
 // depend on the macros moved before is done once, in parallel, and a macro
 // costs two launches:
-//   - k_wm_static, once per pass: per macro and net, the extent of the net's
-//     pins on other cells than movable macros (a block each; exact FP32 pairs,
-//     pairs.cuh, as FP64 minima and maxima are GB300's slowest instructions);
-//   - k_wm_mask per macro: each net's extent with the macros' pins added (a
-//     short list made at create), the two mask axes with the distances of
-//     their corners, and every obstacle as the exact range of candidate
-//     columns and rows that it blocks (stepping from a guess);
+//   - k_wm_static, once per pass, a block per net with macros on it: the extent
+//     of the net's pins on other cells than movable macros (exact FP32 pairs,
+//     pairs.cuh, as FP64 minima and maxima are GB300's slowest instructions),
+//     and from it, adding the net's macros from the last one to move back to
+//     the first, for each of them the extent of those pins and of the
+//     macros that still stand where they were;
+//   - k_wm_mask per macro: each net's extent with that of the macros that have
+//     moved (kept per net, one step of minimum and maximum a macro), the two
+//     mask axes with the distances of their corners, and every obstacle as the
+//     exact range of candidate columns and rows that it blocks (stepping from a
+//     guess);
 //   - k_wm_select per macro: a block per row of candidates turns the
 //     obstacles that cover the row into a bit mask, so that a candidate costs
 //     one bit test, one FP64 addition and one comparison; the last block
-//     reduces the rows' winners and moves the macro.
+//     reduces the rows' winners, moves the macro and adds it to its nets'
+//     moved extents.
+// So the tables hold one entry per macro and net, and a macro's cost depends on
+// the number of its nets, not on how many macros share them.
 // Copies run side by side (blockIdx.y).  One pass over 32 macros of a 210k-cell design on 512 x 512
-// bins, restored before and read back: 3.7 -> 0.6 ms against one warp per net in FP64
+// bins, restored before and read back: 3.7 -> 0.54 ms against one warp per net in FP64
 // and four launches a macro.  (Launching each kernel early, by
 // griddepcontrol.launch_dependents at its start or before its last step, took
 // 28 us a macro instead of 15: measured, not taken.)
@@ -133,13 +140,45 @@ __device__ Best block_best(Best v) {
   return v;
 }
 
-// The extent {x-, x+, y-, y+} of entry s (a macro's net): its pins on other
-// cells than movable macros; +-inf when there are none.
+// An extent {x-, x+, y-, y+}; empty: +-inf.
+struct Extent {
+  double v[4];
+};
+__device__ __forceinline__ Extent no_extent() { return Extent{{INFINITY, -INFINITY, INFINITY, -INFINITY}}; }
+__device__ __forceinline__ void extent_add(Extent &a, const Extent &b) {
+  a.v[0] = fmin(a.v[0], b.v[0]); a.v[1] = fmax(a.v[1], b.v[1]);
+  a.v[2] = fmin(a.v[2], b.v[2]); a.v[3] = fmax(a.v[3], b.v[3]);
+}
+// A macro's pins on one net, with its corner at p and their offsets' extent o.
+// (Rounding is monotone: the extent of the rounded sums is the rounded sum of
+// the extent.)
+__device__ __forceinline__ Extent extent_at(float2 p, float4 o) {
+  return Extent{{__dadd_rn((double)p.x, (double)o.x), __dadd_rn((double)p.x, (double)o.y),
+                 __dadd_rn((double)p.y, (double)o.z), __dadd_rn((double)p.y, (double)o.w)}};
+}
+__device__ __forceinline__ Extent load_extent(const double *p, size_t k) {
+  Extent e;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) e.v[i] = p[4 * k + i];
+  return e;
+}
+__device__ __forceinline__ void store_extent(double *p, size_t k, const Extent &e) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[4 * k + i] = e.v[i];
+}
+
+// Net blockIdx.x of those with macros on them, its entries (a macro and the net)
+// in the macros' order: the extent of its pins on other cells than movable
+// macros, and for each entry that extent with the macros after it added, at
+// their places before the pass.
 __global__ void __launch_bounds__(kWmNetThreads) k_wm_static(Dev d, WmDev w, int copy0) {
-  __shared__ PairBox sb[kWmNetThreads / 32];
-  const int c = copy0 + blockIdx.y, s = blockIdx.x;
+  constexpr int kWarps = kWmNetThreads / 32;
+  __shared__ PairBox sb[kWarps];
+  __shared__ Extent se[kWarps], carry;
+  const int c = copy0 + blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float2 *xy = d.xy + (size_t)c * d.n_cells;
-  int e = w.mnet[s];
+  const int q0 = w.dptr[blockIdx.x], q1 = w.dptr[blockIdx.x + 1];
+  int e = w.mnet[w.dent[q0]];
   HP_FIX(d.err, e, d.n_nets, BS_WM_NET);
   PairBox b = empty_box();
   bool any = false;
@@ -152,17 +191,56 @@ __global__ void __launch_bounds__(kWmNetThreads) k_wm_static(Dev d, WmDev w, int
     any = true;
   }
   box_reduce<32>(b);
-  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = b;
+  if (lane == 0) sb[warp] = b;
   any = __syncthreads_or(any);
+  double *sbox = w.sbox + (size_t)blockIdx.y * w.n_entries * 4;
   if (threadIdx.x < 32) {
-    b = sb[threadIdx.x % (kWmNetThreads / 32)];
-    box_reduce<kWmNetThreads / 32>(b);
+    b = sb[threadIdx.x % kWarps];
+    box_reduce<kWarps>(b);
     if (threadIdx.x == 0) {
-      double *o = w.sbox + ((size_t)blockIdx.y * w.n_entries + s) * 4;
-      o[0] = any ? pair_value(b.nx) : INFINITY;
-      o[1] = any ? pair_value(b.mx) : -INFINITY;
-      o[2] = any ? pair_value(b.ny) : INFINITY;
-      o[3] = any ? pair_value(b.my) : -INFINITY;
+      const Extent s = any ? Extent{{pair_value(b.nx), pair_value(b.mx), pair_value(b.ny), pair_value(b.my)}}
+                           : no_extent();
+      if (q1 - q0 == 1) {
+        store_extent(sbox, w.dent[q0], s);
+      } else {
+        carry = s;
+        store_extent(w.moved, (size_t)blockIdx.y * w.n_shared + w.slot[w.dent[q0]], no_extent());
+      }
+    }
+  }
+  if (q1 - q0 == 1) return;
+  // a net of several macros: a scan from its last entry, in steps of a block
+  for (int end = q1; end > q0; end -= kWmNetThreads) {
+    const int q = end - 1 - (int)threadIdx.x;  // thread 0 has the last one
+    int s = 0;
+    Extent v = no_extent();
+    if (q >= q0) {
+      s = w.dent[q];
+      int m = w.mcell[s];
+      HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
+      v = extent_at(xy[m], w.own[s]);
+    }
+    // inclusive over the warp, then the warps before and the steps before
+    Extent in = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      Extent x;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x.v[i] = __shfl_up_sync(0xffffffffu, in.v[i], o);
+      if (lane >= o) extent_add(in, x);
+    }
+    Extent out;  // exclusive
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out.v[i] = __shfl_up_sync(0xffffffffu, in.v[i], 1);
+    if (lane == 0) out = no_extent();
+    if (lane == 31) se[warp] = in;
+    __syncthreads();
+    for (int k = 0; k < warp; ++k) extent_add(out, se[k]);
+    extent_add(out, carry);
+    if (q >= q0) store_extent(sbox, s, out);
+    __syncthreads();  // (carry and se have been read)
+    if (threadIdx.x == kWmNetThreads - 1) {
+      extent_add(out, v);
+      carry = out;
     }
   }
 }
@@ -208,45 +286,25 @@ __global__ void __launch_bounds__(kWmLines) k_wm_mask(Dev d, WmDev w, int t, int
     const bool mine = n0 + (int)threadIdx.x < nn;
     // box: other pins' extent {o-x, o+x, o-y, o+y}, then the macro's own pin
     // offsets {d-x, d+x, d-y, d+y}
-    double v[8] = {INFINITY, -INFINITY, INFINITY, -INFINITY, INFINITY, -INFINITY, INFINITY, -INFINITY};
-    int k0 = 0, k1 = 0, others = 0;
+    float4 own;
+    int shared = -1;
     if (mine) {
       int e = w.mnet[s];
       HP_FIX(d.err, e, d.n_nets, BS_WM_NET);
       sw[threadIdx.x] = d.net_w ? (double)d.net_w[e] : 1.0;
-      k0 = w.mpin_ptr[s];
-      k1 = w.mpin_ptr[s + 1];
-      for (int k = k0; k < k1; ++k) {
-        int j = w.mpin[k];
-        HP_FIX(d.err, j, d.n_pins, BS_WM_NET);
-        if (d.pin_cell[j] != m) {
-          ++others;
-          continue;
-        }
-        const float2 of = d.pin_off[j];
-        v[4] = fmin(v[4], (double)of.x); v[5] = fmax(v[5], (double)of.x);
-        v[6] = fmin(v[6], (double)of.y); v[7] = fmax(v[7], (double)of.y);
-      }
+      own = w.own[s];
+      shared = w.slot[s];
     }
     if (!waited) pdl_wait();
     waited = true;
     if (mine) {
-      const double *o = w.sbox + ((size_t)blockIdx.y * w.n_entries + s) * 4;
+      Extent o = load_extent(w.sbox + (size_t)blockIdx.y * w.n_entries * 4, s);
+      if (shared >= 0)  // the net's macros that have moved
+        extent_add(o, load_extent(w.moved + (size_t)blockIdx.y * w.n_shared * 4, shared));
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = o[k];
-      for (int k = k0; others > 0 && k < k1; ++k) {  // the other macros' pins
-        int j = w.mpin[k];
-        HP_FIX(d.err, j, d.n_pins, BS_WM_NET);
-        int cj = d.pin_cell[j];
-        HP_FIX(d.err, cj, d.n_cells, BS_WM_CELL);
-        if (cj == m) continue;
-        const float2 of = d.pin_off[j], p = xy[cj];
-        const double px = __dadd_rn((double)p.x, (double)of.x), py = __dadd_rn((double)p.y, (double)of.y);
-        v[0] = fmin(v[0], px); v[1] = fmax(v[1], px);
-        v[2] = fmin(v[2], py); v[3] = fmax(v[3], py);
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) box[k][threadIdx.x] = v[k];
+      for (int k = 0; k < 4; ++k) box[k][threadIdx.x] = o.v[k];
+      box[4][threadIdx.x] = (double)own.x; box[5][threadIdx.x] = (double)own.y;
+      box[6][threadIdx.x] = (double)own.z; box[7][threadIdx.x] = (double)own.w;
     }
     __syncthreads();
     if (live) {
@@ -273,6 +331,10 @@ __global__ void __launch_bounds__(kWmLines) k_wm_mask(Dev d, WmDev w, int t, int
 __global__ void __launch_bounds__(kWmThreads) k_wm_select(Dev d, WmDev w, int t, int copy0) {
   __shared__ unsigned int blocked[8192 / 32];
   __shared__ int flag;
+  __shared__ float2 place;
+  int m = w.order[t];
+  HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
+  const int s0 = w.mptr[t], s1 = w.more[t] ? w.mptr[t + 1] : s0;
   pdl_wait();
   const int c = copy0 + blockIdx.y, j = blockIdx.x, nob = w.n_fixed + t;
   const double *f = w.f + (size_t)blockIdx.y * (d.nx + d.ny);
@@ -322,22 +384,33 @@ __global__ void __launch_bounds__(kWmThreads) k_wm_select(Dev d, WmDev w, int t,
   best = block_best(best);
   if (threadIdx.x == 0) {
     w.ctr[blockIdx.y] = 0u;
+    float2 *at = d.xy + (size_t)c * d.n_cells + m;
+    float2 p = *at;
     if (best.idx != kNoIdx && HP_IN(d.err, best.idx, d.nx * d.ny, BS_WM_BIN)) {
       const int jj = best.idx / d.nx, i = best.idx - jj * d.nx;
-      int m = w.order[t];
-      HP_FIX(d.err, m, d.n_cells, BS_WM_CELL);
-      d.xy[(size_t)c * d.n_cells + m] =
-          make_float2((float)wm_corner(d.die_xl, d.die_xh, d.nx, i),
+      p = make_float2((float)wm_corner(d.die_xl, d.die_xh, d.nx, i),
                       (float)wm_corner(d.die_yl, d.die_yh, d.ny, jj));
+      *at = p;
     }
+    place = p;
+  }
+  if (s1 == s0) return;  // no later macro shares a net with this one
+  __syncthreads();
+  for (int s = s0 + threadIdx.x; s < s1; s += kWmThreads) {
+    const int k = w.slot[s];
+    if (k < 0) continue;
+    const size_t at = (size_t)blockIdx.y * w.n_shared + k;
+    Extent e = load_extent(w.moved, at);
+    extent_add(e, extent_at(place, w.own[s]));
+    store_extent(w.moved, at, e);
   }
 }
 
 }  // namespace
 
 void launch_wiremask(const Dev &d, const WmDev &w, int copy0, int ncopy, cudaStream_t st) {
-  if (w.n_entries > 0)
-    k_wm_static<<<dim3(w.n_entries, ncopy), kWmNetThreads, 0, st>>>(d, w, copy0);
+  if (w.n_dnets > 0)
+    k_wm_static<<<dim3(w.n_dnets, ncopy), kWmNetThreads, 0, st>>>(d, w, copy0);
   const int lines = (d.nx + d.ny + kWmLines - 1) / kWmLines;
   for (int t = 0; t < w.n_macros; ++t) {
     const int ranges = (w.n_fixed + t + kWmLines - 1) / kWmLines;
