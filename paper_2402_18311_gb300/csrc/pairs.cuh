@@ -58,7 +58,10 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
                           (int)(u << 29));
 }
+// What the rounding of a pair dropped: nothing of an infinite sum (whose e is not
+// a number).
+__device__ __forceinline__ double pair_rest(Pair p) { return widen(p.e == p.e ? p.e : 0.f); }
 // A pair's number, not halved any more: the exact sum rounded once to FP64.
-__device__ __forceinline__ double pair_value(Pair p) { return 2.0 * (widen(p.s) + widen(p.e)); }
+__device__ __forceinline__ double pair_value(Pair p) { return 2.0 * (widen(p.s) + pair_rest(p)); }
 
 }  // namespace hp

@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kBigNet) k_wa_big(Dev d, int copy0, int cls, i
 // overflows.  HPWL and
 // overflow of the 2.1M-cell design: 1.44 -> 0.27 ms.
 __device__ __forceinline__ double extent(Pair hi, Pair lo) {
-  return (widen(hi.s) - widen(lo.s)) + (widen(hi.e) - widen(lo.e));
+  return (widen(hi.s) - widen(lo.s)) + (pair_rest(hi) - pair_rest(lo));
 }
 // acc + w times the net's half perimeter, halved like its coordinates
 __device__ __forceinline__ double box_hpwl(const PairBox &b, float w, double acc) {
