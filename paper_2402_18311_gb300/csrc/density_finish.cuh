@@ -57,11 +57,11 @@ __device__ __forceinline__ void bin_excess(const Dev &d, unsigned long long m, l
       ++s.n_over;
     }
   } else {
-    // excess * 2^s = m 2^s + t_mant F - t_mant A: exact in unsigned 128
-    // bits (below 2^124, and valid when overlapping fixed cells make F > A)
-    u128 lhs = (u128)m << d.t_shift;
-    lhs += (u128)(unsigned long long)d.t_mant * (u128)(unsigned long long)f;
-    if (lhs > tA) s.acc += lhs - tA;
+    // excess * 2^s = m 2^s + t_mant F - t_mant A: exact in signed 128 bits
+    // (below 2^124; F > A where fixed cells overlap, F < 0 only in a map that a
+    // caller of place_overflow_noalloc brings)
+    const __int128 e = (__int128)((u128)m << d.t_shift) + (__int128)d.t_mant * (__int128)f - (__int128)tA;
+    if (e > 0) s.acc += (u128)e;
   }
 }
 
