@@ -1114,7 +1114,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.fill_area_q = (double)nf * (double)fp.Wf * (double)fp.Hf;
   {
     const double s1 = (d.mov_area_q + d.fill_area_q) / d.abin_q;
-    d.area2_bins = (float)(s1 * s1);
+    d.area2_bins = s1 * s1;
     double fixed_q = 0.0;
     for (int i = Mv; i < C; ++i) fixed_q += (double)Wq[i] * (double)Hq[i];
     d.rho_mean = (float)((d.mov_area_q + d.fill_area_q + d.t * fixed_q) / (d.abin_q * (double)d.G));

@@ -90,23 +90,27 @@ __device__ __forceinline__ float2 finish_pair(const Dev &d, const FinishArgs &a,
                      fmaf(a.tf, u64_to_float((unsigned long long)f.y) * a.inv_a, mf1));
 }
 
-// The copy's overflow from its bins' excess v (times 2^s) and concentration
-// q2, recorded by mode: the iteration's tau (with the stop test), an
+// The copy's overflow from its bins' excess v (times 2^s) and its concentration
+// from q2, recorded by mode: the iteration's tau (with the stop test), an
 // evaluation's result, or the reset value tau_{-1} that sets the first gamma.
+// Called by a warp whose lane 0 has v and q2: its FP64 division, a microsecond
+// here, is shared with lane 1's (n_eff).
 __device__ __forceinline__ void finish_commit(const Dev &d, int c, int mode, u128 v, float q2) {
   CopyState *cs = d.cs + c;
-  const double tau = ldexp(u128_to_double(v), -d.t_shift) / d.mov_area_q;
-  // (q2 is an FP32 sum, and FP64 divisions are a microsecond each here)
-  if (mode != FIN_EVAL) cs->n_eff = q2 > 0.f ? (double)(d.area2_bins / q2) : 0.0;
+  q2 = __shfl_sync(0xffffffffu, q2, 0);
+  const bool first = threadIdx.x == 0;
+  const double r = (first ? ldexp(u128_to_double(v), -d.t_shift) : d.area2_bins) / (first ? d.mov_area_q : (double)q2);
+  if (threadIdx.x == 1 && mode != FIN_EVAL) cs->n_eff = q2 > 0.f ? r : 0.0;
+  if (!first) return;
   if (mode == FIN_ITER) {
-    cs->tau = tau;
-    if (tau <= (double)d.prm.tau_stop) cs->converged = cs->stopped = 1;
+    cs->tau = r;
+    if (r <= (double)d.prm.tau_stop) cs->converged = cs->stopped = 1;
   } else if (mode == FIN_RESET) {
-    cs->tau = cs->tau_prev = tau;
-    cs->gamma = gamma_of(d, tau);
+    cs->tau = cs->tau_prev = r;
+    cs->gamma = gamma_of(d, r);
     if (d.prm.max_iters <= 0) cs->stopped = 1;
   } else {
-    d.scal[(size_t)c * S_COUNT + S_TAU] = tau;
+    d.scal[(size_t)c * S_COUNT + S_TAU] = r;
   }
 }
 
@@ -154,7 +158,7 @@ __device__ __forceinline__ void finish_total(const Dev &d, int c, int mode, int 
     v += shfl_xor_u128(v, o);
     q2 += __shfl_xor_sync(0xffffffffu, q2, o);
   }
-  if (threadIdx.x == 0) finish_commit(d, c, mode, v, q2);
+  finish_commit(d, c, mode, v, q2);
 }
 
 // The block's sums to its partial slot; the last block of each copy reduces
@@ -174,10 +178,8 @@ __device__ __forceinline__ void finish_reduce(const Dev &d, int c, int mode, con
   }
   v = block_sum_u128<NT>(v, sh->sm);
   q2 = block_sum_f<NT>(q2, sh->smf);
-  if (threadIdx.x == 0) {
-    finish_commit(d, c, mode, v, q2);
-    d.ctr[(size_t)c * C_COUNT + C_FINISH] = 0u;
-  }
+  if (threadIdx.x < 32) finish_commit(d, c, mode, v, q2);
+  if (threadIdx.x == 0) d.ctr[(size_t)c * C_COUNT + C_FINISH] = 0u;
 }
 
 }  // namespace hp

@@ -95,7 +95,7 @@ struct Dev {
   double abin_q;              // BW * BH
   double mov_area_q;          // the design's movable area (units of 2^-2F): tau's denominator
   double fill_area_q;         // the fillers' area (units of 2^-2F)
-  float area2_bins;           // ((mov_area_q + fill_area_q) / abin_q)^2: the numerator of n_eff
+  double area2_bins;          // ((mov_area_q + fill_area_q) / abin_q)^2: the numerator of n_eff
   double die_xl, die_yl, die_xh, die_yh;
   float fxl, fyl, fxh, fyh;
   float fbw, fbh, fibw, fibh;  // bin width/height and their inverses (FP32)
