@@ -1077,7 +1077,9 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.fbw = (float)bw; d.fbh = (float)bh; d.fibw = (float)(1.0 / bw); d.fibh = (float)(1.0 / bh);
   d.w_bin = std::sqrt(bw * bh);
   d.dref = (double)prm.hpwl_ref * (double)E * d.w_bin;
-  d.lg_mu = prm.mu_base > 0.f && std::isfinite(prm.mu_base) ? std::log2((double)prm.mu_base) : 0.0;
+  const long double lg_mu = prm.mu_base > 0.f && std::isfinite(prm.mu_base) ? std::log2((long double)prm.mu_base) : 0.0L;
+  d.lg_mu = (double)lg_mu;
+  d.lg_mu_lo = (double)(lg_mu - (long double)d.lg_mu);
   d.prm = prm;
   d.has_net_w = nl->net_w ? 1 : 0;
   d.tc = prm.dct_mode == PLACE_DCT_BF16X3 ? 1 : 0;

@@ -102,7 +102,8 @@ struct Dev {
   int BW32, BH32;             // BW, BH (below 2^26: nx, ny >= 16 and nx BW < 2^30)
   float ibw_q, ibh_q;         // 1 / BW, 1 / BH
   double w_bin, dref;
-  double lg_mu;               // log2 mu_base where it is finite and not 0, else 0 (pow takes over)
+  double lg_mu, lg_mu_lo;     // log2 mu_base, rounded and the rest, where it is finite and not
+                              // 0, else 0 (pow takes over)
   int nb_red;                 // partial slots per reduction per copy
   int cell_blocks;            // blocks per copy for per-cell kernels
   int cg_blocks;              // blocks per copy of the cell-gradient kernel (one wave)

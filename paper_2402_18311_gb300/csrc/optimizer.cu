@@ -129,8 +129,8 @@ __device__ __forceinline__ void next_scalars(const Dev &d, const CopyState *cs, 
     s->gamma = gamma_of(d, cs->tau);
   } else if (threadIdx.x == 96 && !first) {
     const double y = 1.0 - (hpwl - cs->hpwl_prev) / d.dref;
-    const double mu = d.lg_mu != 0.0 ? pow_log2(fmin(fmax(y * d.lg_mu, -900.0), 900.0), 1.0, 0.0)
-                                     : pow((double)P.mu_base, y);
+    const double mu = d.lg_mu != 0.0 && fabs(y * d.lg_mu) < 900.0 ? pow_log2(y, d.lg_mu, d.lg_mu_lo)
+                                                                  : pow((double)P.mu_base, y);
     s->mu = fmin(fmax(mu, (double)P.mu_lo), (double)P.mu_hi);
   }
 }
