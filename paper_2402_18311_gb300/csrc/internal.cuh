@@ -59,8 +59,9 @@ struct CopyState {
 // of the step norm's partials (see k_cell_grad).
 enum Slot { S_TAU = 0, S_HPWL, S_WL, S_GW1, S_GD1, S_DG2, S_DV2, S_G2, S_HP64, S_PH, S_PW, S_PV, S_COUNT };
 
-// Last-block counters per copy.
-enum Counter { C_FINISH = 0, C_CELL, C_PRE0, C_UPDATE, C_COUNT };
+// Last-block counters per copy, and a flag: the copy had stopped when the fast
+// transforms' first kernel ran.
+enum Counter { C_FINISH = 0, C_CELL, C_PRE0, C_UPDATE, C_SKIP, C_COUNT };
 
 // The density scatter's ways of adding overlaps to the map (density.cu).
 enum ScatterMode { SCAT_MERGED = 0, SCAT_TABLE = 1, SCAT_DIRECT = 2 };

@@ -66,8 +66,12 @@ __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
   __shared__ FinishShared fs;
   pdl_wait();
   const int c = copy0 + blockIdx.y;
-  CopyState *cs = d.cs + c;
-  if (mode == FIN_ITER && cs->stopped) return;
+  if (mode == FIN_ITER) {
+    const int stopped = d.cs[c].stopped;
+    // for the columns, beside whose blocks the stop test writes it
+    if (blockIdx.x == 0 && threadIdx.x == 0) d.ctr[(size_t)c * C_COUNT + C_SKIP] = stopped;
+    if (stopped) return;
+  }
   const int f = threadIdx.x / T, t = threadIdx.x % T;
   const int xa = 2 * (blockIdx.x * F + f);  // rows xa and xa + 1
   float2 *s = sm + f * padded(N);
@@ -122,8 +126,8 @@ __global__ void __launch_bounds__(row_ffts(LOGN) * (1 << (LOGN - 3)))
 // CP column pairs per block, M / 8 threads each.  One more block per copy
 // reduces the overflow of the row kernel's partials: beside the transforms
 // instead of at the end of that kernel, whose last block held the next one up
-// for 4 us.  (A copy that its stop test ends here may still get a field, which
-// nothing reads.)
+// for 4 us.  The stop test there may end the copy, so the other blocks do not read
+// its flag but what the row kernel found.
 template <int LOGM, int CP>
 __global__ void __launch_bounds__(CP * (1 << (LOGM - 3)))
     k_fft_columns(Dev d, int copy0, int mode, int partials) {
@@ -131,7 +135,7 @@ __global__ void __launch_bounds__(CP * (1 << (LOGM - 3)))
   __shared__ float2 sm[CP * padded(M)];
   pdl_wait();
   const int c = copy0 + blockIdx.y;
-  if (mode == FIN_ITER && d.cs[c].stopped) return;
+  if (mode == FIN_ITER && d.ctr[(size_t)c * C_COUNT + C_SKIP]) return;
   if (blockIdx.x == gridDim.x - 1) {
     if (threadIdx.x < 32) finish_total(d, c, mode, partials);
     return;
