@@ -457,6 +457,13 @@ int place_measure_scatter_floor(place_t *h, int32_t reps, float *ms_scatter, flo
  * without the tensor-core path.  Synchronises; takes about two seconds. */
 int place_test_wait_timeout(place_t *h);
 
+/* Failure-path check of the graph that runs several iterations in one launch
+ * (place_step makes it for handles that iterate on): from now on the memory for
+ * it runs out when it is instantiated (step 1) or uploaded (step 2; 0: no
+ * failure).  The handle then runs one iteration at a time, with the same
+ * results.  Nothing is allocated or launched by this call. */
+int place_test_no_graph_memory(place_t *h, int32_t step);
+
 /* Failure-path check of the index checks of the bounds-checking build
  * (place_info.bounds_checked): one thread tests the index n_cells against
  * the cell count, as a kernel would before a position gather, and touches

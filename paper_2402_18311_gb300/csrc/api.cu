@@ -262,6 +262,7 @@ struct place_t {
   cudaGraphExec_t exec_n = nullptr;
   long long n_iters = 0;
   bool no_runs = false;  // there was no memory for that graph: one at a time
+  int fail_runs = 0;     // place_test_no_graph_memory
   CUtensorMap maps[16];              // tensor maps of the tcgen05 spectral path
   int n_cand_all = 0, n_cand_macro = 0;
   // WireMask: host tables built at create, device copy made on first use
@@ -760,9 +761,16 @@ int launch_iters(place_t *h, int n) {
       for (int k = 0; k < kUnroll; ++k) enqueue_iteration(h->d, h->cap, wst, h->ev_fork, joins, false);
       cudaGraph_t g = nullptr;
       cudaError_t e = cudaStreamEndCapture(h->cap, &g);
+      if (e == cudaSuccess && h->fail_runs == 1) e = cudaErrorMemoryAllocation;
       if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec_n, g, 0);
-      if (g) cudaGraphDestroy(g);
       if (e != cudaSuccess) h->exec_n = nullptr;
+      if (g) cudaGraphDestroy(g);
+      // the upload takes device memory: here, so that no launch does
+      if (e == cudaSuccess) e = h->fail_runs == 2 ? cudaErrorMemoryAllocation : cudaGraphUpload(h->exec_n, h->stream);
+      if (e != cudaSuccess && h->exec_n) {
+        cudaGraphExecDestroy(h->exec_n);
+        h->exec_n = nullptr;
+      }
       if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         h->no_runs = true;
@@ -1712,6 +1720,13 @@ int place_measure_scatter_floor(place_t *h, int32_t reps, float *ms_scatter, flo
   *ms_scatter = t[0] / reps;
   *ms_floor = t[1] / reps;
   return check_dev_err(h);
+}
+
+int place_test_no_graph_memory(place_t *h, int32_t step) {
+  if (!h) return fail(PLACE_EINVAL, "null handle");
+  if (step < 0 || step > 2) return fail(PLACE_EINVAL, "step must be 0, 1 or 2");
+  h->fail_runs = step;
+  return PLACE_OK;
 }
 
 int place_test_bounds_check(place_t *h) {

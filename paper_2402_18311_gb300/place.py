@@ -148,6 +148,7 @@ _SIGS = {
     "place_step_timed": (ct.c_int, [_VP, ct.c_int32, _VP]),
     "place_measure_wa_floor": (ct.c_int, [_VP, ct.c_int32, ct.POINTER(ct.c_float)]),
     "place_test_wait_timeout": (ct.c_int, [_VP]),
+    "place_test_no_graph_memory": (ct.c_int, [_VP, ct.c_int32]),
     "place_test_bounds_check": (ct.c_int, [_VP]),
     "place_measure_scatter_floor": (ct.c_int, [_VP, ct.c_int32, ct.POINTER(ct.c_float),
                                                ct.POINTER(ct.c_float)]),
@@ -422,6 +423,12 @@ def place_test_bounds_check(h):
     """The C return code (PLACE_EINTERNAL expected in the bounds-checking
     build, PLACE_EINVAL in the normal one); does not raise."""
     return lib().place_test_bounds_check(h)
+
+
+def place_test_no_graph_memory(h, step):
+    """The memory for the graph of several iterations runs out at its
+    instantiation (1) or its upload (2; 0: no failure)."""
+    _check(lib().place_test_no_graph_memory(h, step))
 
 
 def place_test_wait_timeout(h):
