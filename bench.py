@@ -152,15 +152,12 @@ def dist_env():
     return rank, world, local
 
 
-def fast_transforms(dct, d):
-    """Whether the handle solves by fast transforms: power-of-two sides (a
-    64 x 64 grid is one cluster's), and the mode left to the library or FP32."""
-    return (dct != 1 and d.nx * d.ny > 4096
-            and all(64 <= n <= 4096 and n & (n - 1) == 0 for n in (d.nx, d.ny)))
+SOLVES = ["fp32", "bf16x3", "fast transforms, fp32", "fp32, one cluster"]
 
 
-def solve_name(dct, d, info):
-    return "fast transforms, fp32" if fast_transforms(dct, d) else ["fp32", "bf16x3"][info.dct_mode]
+def solve_name(place, h):
+    """The Poisson solve that the handle runs."""
+    return SOLVES[place.place_get_solve(h)]
 
 
 def algorithmic(d, info):
@@ -214,6 +211,7 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     h = place.place_create(d, prm, stream=stream.cuda_stream)
     info = place.place_get_info(h)
+    solve = solve_name(place, h)
 
     # untimed iterations to a later phase of the placement (profiling), then
     # the warm-up (which also captures the iteration graph)
@@ -290,7 +288,7 @@ def run_ours(args):
     e2e_v = world * n_e2e / e2e_s
 
     alg = algorithmic(d, info)
-    if fast_transforms(args.dct, d):
+    if solve == SOLVES[2]:
         # one forward and two inverse 2-D transforms (the first half of the
         # forward one is timed with the density stage)
         alg["spectral"] = {"flops": 7.5 * d.nx * d.ny * float(np.log2(d.nx * d.ny))}
@@ -349,12 +347,12 @@ def run_ours(args):
         "metric": METRIC, "value": value, "unit": "iters/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f32+bf16x3" if "bf16" in solve_name(args.dct, d, info) else "f32", "data": "synthetic",
+        "dtype": "f32+bf16x3" if "bf16" in solve else "f32", "data": "synthetic",
         "config": {"workload": args.workload, "desc": desc, "copies_per_gpu": prm.n_copies,
                    "parallelism": f"replicas{world}", "l2": "inputs larger than L2 "
                    "(per-iteration working set > 129 MB)" if args.workload == "large_2m"
                    else "working set fits L2 (no flush)",
-                   "dct_mode": solve_name(args.dct, d, info), "tuning": tuning(info),
+                   "dct_mode": solve, "tuning": tuning(info),
                    "timed_iterations": [args.advance + args.warmup + 1,
                                         args.advance + args.warmup + args.steps]},
         "e2e": {"value": e2e_v, "unit": "iters/s",
@@ -471,6 +469,7 @@ def run_configs(args, place, torch):
     h = place.place_create(d, place.place_default_params(tau_stop=-1.0, max_iters=300,
                                                          dct_mode=place.PLACE_DCT_AUTO))
     info = place.place_get_info(h)
+    solve = solve_name(place, h)
     bh = np.empty(1); bt = np.empty(1); br = np.empty(1, np.int32)
     place.place_step(h, 1)  # graph capture outside the timed region
     place.place_set_positions(h, 0, d.x, d.y)
@@ -481,7 +480,7 @@ def run_configs(args, place, torch):
     rh, rt = place.place_get_hybro_rounds(h, 0)
     place.place_destroy(h)
     out["tiny_1k"] = {"desc": WORKLOADS["tiny_1k"][1], "iterations": 600, "seconds": el,
-                      "iters_per_s": 600 / el, "spectral": solve_name(place.PLACE_DCT_AUTO, d, info),
+                      "iters_per_s": 600 / el, "spectral": solve,
                       "round_hpwl": rh.tolist(), "round_overflow": rt.tolist(),
                       "best_round": int(br[0]), "best_hpwl": float(bh[0]),
                       "note": "300 iterations, Shuffle (all) p = 0.5 seed 0, 300 more; host "
@@ -490,6 +489,7 @@ def run_configs(args, place, torch):
     h = place.place_create(d, place.place_default_params(tau_stop=0.07, max_iters=1000,
                                                          dct_mode=args.dct))
     info = place.place_get_info(h)
+    solve = solve_name(place, h)
     place.place_step(h, 1)
     place.place_set_positions(h, 0, d.x, d.y)
     conv = np.zeros(1, np.int32)
@@ -509,7 +509,7 @@ def run_configs(args, place, torch):
                           "converged": bool(st.converged), "seconds": ms / 1e3,
                           "iters_per_s": 1e3 * st.iter / ms, "final_overflow": float(tv[0]),
                           "final_hpwl": float(hp[0]),
-                          "spectral": solve_name(args.dct, d, info),
+                          "spectral": solve,
                           "note": "to overflow <= 0.07 or 1,000 iterations, CUDA events around "
                                   "the whole run (50-iteration launches, stop flags read back)"}
     return out

@@ -152,7 +152,9 @@ typedef struct place_params {
                              a shared-memory table and direct atomics; 0, 1, 2
                              force one of them.  All give the same map. */
   int32_t gemm_bn;        /* 0 (default): automatic; 64 or 128: tile width of
-                             every tensor-core GEMM stage of the spectral solve */
+                             every tensor-core GEMM stage of the spectral solve
+                             (this and gemm_split do not choose the solve: see
+                             PLACE_DCT_AUTO and place_get_solve) */
   int32_t wa_big_cap;     /* 0 (default): automatic; 32..6144: pins of a net of
                              more than 256 pins kept in shared memory */
   int32_t gemm_split;     /* 0 (default): automatic; 1: one CTA per GEMM tile;
@@ -190,7 +192,7 @@ typedef struct place_info {
                               iteration after a reset adds one: k_precond0) */
   int32_t dct_mode;       /* the resolved mode, PLACE_DCT_FP32 or _BF16X3 (with
                              PLACE_DCT_AUTO on power-of-two sides the fast transforms
-                             solve in either, see there) */
+                             solve in either: place_get_solve tells) */
   int32_t n_fillers;      /* filler cells (0 unless params.fillers) */
   int32_t bounds_checked; /* 1: the library was built with index checks
                            * (-DPLACE_DEBUG_BOUNDS): a failed check makes the
@@ -204,6 +206,15 @@ typedef struct place_info {
   int32_t wa_streams;     /* graph branches the WA classes run on (1..3) */
   int32_t dct_fold;       /* 1: the BF16x3 path has the even/odd split (params.dct_fold) */
 } place_info;
+
+/* The Poisson solve that the handle's iterations and evaluations run.
+ * place_info.dct_mode, dct_fold, gemm_bn and gemm_split describe the tensor
+ * cores' GEMMs wherever a handle has them; only PLACE_SOLVE_GEMM_BF16X3 runs them. */
+#define PLACE_SOLVE_GEMM_FP32 0   /* tiled FP32 GEMMs */
+#define PLACE_SOLVE_GEMM_BF16X3 1 /* the tensor cores' GEMMs */
+#define PLACE_SOLVE_FFT 2         /* FP32 fast transforms */
+#define PLACE_SOLVE_CLUSTER 3     /* FP32, one cluster per copy (at most 4096 bins) */
+int place_get_solve(const place_t *h, int32_t *solve);
 
 /* Optimiser scalars of one copy after its last iteration. */
 typedef struct place_state {

@@ -1578,6 +1578,14 @@ int place_get_info(const place_t *h, place_info *o) {
   return PLACE_OK;
 }
 
+int place_get_solve(const place_t *h, int32_t *solve) {
+  if (!h || !solve) return fail(PLACE_EINVAL, "null argument");
+  *solve = h->d.solve == SOLVE_FFT     ? PLACE_SOLVE_FFT
+           : h->d.solve == SOLVE_SMALL ? PLACE_SOLVE_CLUSTER
+                                       : (h->d.tc ? PLACE_SOLVE_GEMM_BF16X3 : PLACE_SOLVE_GEMM_FP32);
+  return PLACE_OK;
+}
+
 int place_step(place_t *h, int32_t n_iters, int32_t *converged) {
   NvtxRange nvtx_("place_step");
   if (!h) return fail(PLACE_EINVAL, "null handle");

@@ -32,6 +32,10 @@ PLACE_WIREMASK = 2
 PLACE_DCT_AUTO = -1
 PLACE_DCT_FP32 = 0
 PLACE_DCT_BF16X3 = 1
+PLACE_SOLVE_GEMM_FP32 = 0
+PLACE_SOLVE_GEMM_BF16X3 = 1
+PLACE_SOLVE_FFT = 2
+PLACE_SOLVE_CLUSTER = 3
 PLACE_STAGES = ("density", "spectral", "wirelength", "cellgrad", "update")
 
 
@@ -148,6 +152,7 @@ _SIGS = {
     "place_step_timed": (ct.c_int, [_VP, ct.c_int32, _VP]),
     "place_measure_wa_floor": (ct.c_int, [_VP, ct.c_int32, ct.POINTER(ct.c_float)]),
     "place_test_wait_timeout": (ct.c_int, [_VP]),
+    "place_get_solve": (ct.c_int, [_VP, ct.POINTER(ct.c_int32)]),
     "place_test_no_graph_memory": (ct.c_int, [_VP, ct.c_int32]),
     "place_test_bounds_check": (ct.c_int, [_VP]),
     "place_measure_scatter_floor": (ct.c_int, [_VP, ct.c_int32, ct.POINTER(ct.c_float),
@@ -282,6 +287,13 @@ def place_get_info(h):
     o = place_info()
     _check(lib().place_get_info(h, ct.byref(o)))
     return o
+
+
+def place_get_solve(h):
+    """The Poisson solve that runs: one of the PLACE_SOLVE_* values."""
+    o = ct.c_int32()
+    _check(lib().place_get_solve(h, ct.byref(o)))
+    return o.value
 
 
 def place_step(h, n_iters, converged=None):
