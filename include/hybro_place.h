@@ -454,7 +454,7 @@ int place_measure_wa_floor(place_t *h, int32_t reps, float *ms);
  * *ms_floor that of a kernel that makes only the same loads (position and
  * size per movable cell) and one 64-bit reduction into each bin the cell
  * covers, none of the exact overlap arithmetic.  Both use the density map as
- * scratch and leave it cleared (the next density pass rebuilds it).
+ * scratch and leave it zero, as the next density pass expects it.
  * Synchronises. */
 int place_measure_scatter_floor(place_t *h, int32_t reps, float *ms_scatter, float *ms_floor);
 

@@ -6,9 +6,10 @@ Every ``csrc/*.cu`` file is compiled to an object in parallel with
 symbols).  Objects go to ``_build/`` at the repository root.
 
 ``build(variant="bounds")`` builds the same sources with
-``-DPLACE_DEBUG_BOUNDS`` into ``libhybro_place_bounds.so``: every kernel
-checks the indices it forms (CSR offsets, cells, bins, tile rows) and a
-failed check is returned as PLACE_EINTERNAL.  ``build_all()`` builds both.
+``-DPLACE_DEBUG_BOUNDS`` into ``libhybro_place_bounds.so``: the kernels
+check the indices that they form from data (CSR offsets, cells, bins) and the
+tensor-core GEMMs' tile rows, and a failed check is returned as PLACE_EINTERNAL.
+(The indices of the transforms and of the FP32 GEMMs follow from the grid alone.)  ``build_all()`` builds both.
 """
 from __future__ import annotations
 

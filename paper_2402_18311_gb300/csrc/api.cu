@@ -79,7 +79,14 @@ constexpr int kGroupHalfDeg[4] = {0, 8, 32, 256};
 constexpr int kBigCapMax = 3072;
 // the scatter's fixed-rule thresholds on the effective number of occupied
 // bins: merged below the first, the shared table below the second, direct
-// atomics above (the autotuner replaces them by measured crossovers)
+// atomics above (the autotuner replaces them by measured crossovers, 2.2 and
+// about 4000 for the 2.1M-cell design, 2.0 and 570 for the 210k-cell one).
+// Density stage of the 2.1M-cell design in ms, merged / table / direct: 0.071 /
+// 0.063 / 0.68 and 0.072 / 0.083 / 1.23 at 4 bins (iterations 5 and 55), 0.095 /
+// 0.060 / 0.166 at 131, 0.083 / 0.095 / 0.077 at 8024.  Of the 210k-cell one: 0.021 /
+// 0.020 / 0.048 at 13, 0.032 / 0.029 / 0.032 at 422, 0.0231 / 0.0229 / 0.0217 at
+// 4681.  So below the first line merged and table are within 15% of one another,
+// either way; the second lies between the two designs' crossings
 constexpr double kScatterMergedBelow = 32.0;
 constexpr double kScatterTableBelow = 1024.0;
 // the WA classes' fixed rule: two graph branches (the short nets beside the long
@@ -622,8 +629,8 @@ int enqueue_reset(place_t *h, int c0, int n, const NewXy &src) {
 // One Nesterov iteration of every copy (the graph body).  The wirelength
 // kernels depend only on the positions and on gamma_k (from the previous
 // iteration's overflow), so they run on their own branches (d.wa_streams of
-// them) beside the density scatter and the tensor-core Poisson solve, and
-// join before the per-cell gradient.
+// them) beside the density scatter and the Poisson solve, and join before the
+// per-cell gradient.
 void enqueue_iteration(const Dev &d, cudaStream_t st, const cudaStream_t *wst, cudaEvent_t fork,
                        const cudaEvent_t *join, bool with_precond0) {
   const int K = d.K;
@@ -1557,10 +1564,10 @@ int place_get_info(const place_t *h, place_info *o) {
   o->device_bytes = (int64_t)h->mem_bytes;
   int wa = 0;
   for (int c = 0; c < d.n_cls; ++c) wa += d.wa_blocks[c] > 0;
-  // scatter, finish, 4 GEMMs, WA classes, cell grad, precond0, update; the
+  // the steady graph (the first iteration after a reset adds k_precond0): the
+  // scatter, finish and solve (four GEMMs behind a finish, or a fused solve's
+  // three kernels or one), the WA classes, cell gradient and update; the
   // stretched scatter with density stretching, the step redo with backtracking
-  // the steady graph (the first iteration after a reset adds k_precond0)
-  // (a fused solve has the finish in its three kernels or its one)
   const int dens = d.solve == SOLVE_FFT ? 1 + 3 : (d.solve == SOLVE_SMALL ? 1 + 1 : 2 + 4);
   o->kernels_per_iter = dens + wa + 2 + (d.Ms ? 1 : 0) + (d.up ? 1 : 0);
   o->dct_mode = d.tc ? PLACE_DCT_BF16X3 : PLACE_DCT_FP32;
@@ -1719,7 +1726,7 @@ int place_measure_scatter_floor(place_t *h, int32_t reps, float *ms_scatter, flo
     t[0] += a;
     t[1] += b;
   }
-  // the map is scratch here: the next density pass clears and rebuilds it
+  // zero again: a handle with a fused solve scatters into the map as it finds it
   cudaMemsetAsync(d.M, 0, mbytes, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   for (auto &x : ev) cudaEventDestroy(x);

@@ -218,25 +218,11 @@ __device__ __forceinline__ double u128_to_double(u128 v) {
          (double)(unsigned long long)v;
 }
 
-// Last-block pattern: every block has published its partials; returns true
-// (in all threads) for the block that arrives last, which then reduces the
-// partials in a fixed order and resets the counter.
-__device__ __forceinline__ bool arrive_last(unsigned int *ctr, int *sm_flag) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int prev = atomicAdd(ctr, 1u);
-    *sm_flag = (prev == gridDim.x - 1) ? 1 : 0;
-  }
-  __syncthreads();
-  const bool last = *sm_flag != 0;
-  if (last) __threadfence();
-  return last;
-}
-
-// The same where thread 0 alone wrote everything that the last block reads: it
-// alone has to order its writes before the arrival, so the block's other
-// threads do not wait for their own stores.
+// Last-block pattern: thread 0 of every block has published the block's
+// partials; returns true (in all threads) for the block that arrives last, which
+// then reduces the partials in a fixed order and resets the counter.  Thread 0
+// alone wrote what the last block reads, so it alone orders its writes before the
+// arrival, and the block's other threads do not wait for their own stores.
 __device__ __forceinline__ bool arrive_last_t0(unsigned int *ctr, int *sm_flag) {
   if (threadIdx.x == 0) {
     __threadfence();
