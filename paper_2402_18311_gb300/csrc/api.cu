@@ -1092,6 +1092,24 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.fbw = (float)bw; d.fbh = (float)bh; d.fibw = (float)(1.0 / bw); d.fibh = (float)(1.0 / bh);
   d.w_bin = std::sqrt(bw * bh);
   d.dref = (double)prm.hpwl_ref * (double)E * d.w_bin;
+  {
+    // the largest finite pin coordinate: movable cells stay in the die
+    double pos = std::max(std::max(std::fabs(die->xl), std::fabs(die->xh)), std::max(std::fabs(die->yl), std::fabs(die->yh)));
+    double off = 0.0;
+    auto most = [](double &m, float v) {
+      if (std::isfinite(v)) m = std::max(m, (double)std::fabs(v));
+    };
+    for (int i = nl->n_movable; i < nl->n_cells; ++i) {
+      most(pos, nl->x0[i]);
+      most(pos, nl->y0[i]);
+    }
+    for (int j = 0; j < P; ++j) {
+      most(off, nl->pin_dx[j]);
+      most(off, nl->pin_dy[j]);
+    }
+    d.pin_scale = pos + off < 1e38 ? 1.f : 0.5f;
+    d.pin_unscale = 1.0 / d.pin_scale;
+  }
   const long double lg_mu = prm.mu_base > 0.f && std::isfinite(prm.mu_base) ? std::log2((long double)prm.mu_base) : 0.0L;
   d.lg_mu = (double)lg_mu;
   d.lg_mu_lo = (double)(lg_mu - (long double)d.lg_mu);

@@ -103,6 +103,8 @@ struct Dev {
   int BW32, BH32;             // BW, BH (below 2^26: nx, ny >= 16 and nx BW < 2^30)
   float ibw_q, ibh_q;         // 1 / BW, 1 / BH
   double w_bin, dref;
+  float pin_scale;            // exact pin coordinates are formed times this (pairs.cuh)
+  double pin_unscale;         // 1 / pin_scale
   double lg_mu, lg_mu_lo;     // log2 mu_base, rounded and the rest, where it is finite and not
                               // 0, else 0 (pow takes over)
   int nb_red;                 // partial slots per reduction per copy

@@ -1,6 +1,8 @@
 // Exact pin coordinates as pairs of FP32 numbers (wirelength.cu has the
-// reasons): the sum of a cell's position and a pin's offset, halved, as s, the
-// sum rounded, and e, what the rounding dropped.
+// reasons): the sum of a cell's position and a pin's offset as s, the sum rounded,
+// and e, what the rounding dropped.  Both summands are multiplied by d.pin_scale
+// first: 1, or 1/2 on a design whose largest sums might overflow FP32 (there a
+// subnormal number loses its last bit).
 #pragma once
 
 #include <cfloat>
@@ -12,9 +14,9 @@ namespace hp {
 struct Pair {
   float s, e;
 };
-__device__ __forceinline__ Pair pin_coord(float v, float o) {
+__device__ __forceinline__ Pair pin_coord(float v, float o, float scale) {
   Pair p;
-  two_sum(0.5f * v, 0.5f * o, p.s, p.e);
+  two_sum(scale * v, scale * o, p.s, p.e);
   return p;
 }
 __device__ __forceinline__ void pair_max(Pair &m, Pair p) {
@@ -34,8 +36,8 @@ __device__ __forceinline__ PairBox empty_box() {
   const Pair lo{-FLT_MAX, 0.f}, hi{FLT_MAX, 0.f};
   return PairBox{lo, hi, lo, hi};
 }
-__device__ __forceinline__ void box_add(PairBox &b, float2 v, float2 o) {
-  const Pair x = pin_coord(v.x, o.x), y = pin_coord(v.y, o.y);
+__device__ __forceinline__ void box_add(PairBox &b, float2 v, float2 o, float scale) {
+  const Pair x = pin_coord(v.x, o.x, scale), y = pin_coord(v.y, o.y, scale);
   pair_max(b.mx, x); pair_min(b.nx, x);
   pair_max(b.my, y); pair_min(b.ny, y);
 }
@@ -61,7 +63,10 @@ __device__ __forceinline__ double widen(float f) {
 // What the rounding of a pair dropped: nothing of an infinite sum (whose e is not
 // a number).
 __device__ __forceinline__ double pair_rest(Pair p) { return widen(p.e == p.e ? p.e : 0.f); }
-// A pair's number, not halved any more: the exact sum rounded once to FP64.
-__device__ __forceinline__ double pair_value(Pair p) { return 2.0 * (widen(p.s) + pair_rest(p)); }
+// A pair's number, not scaled any more (unscale: 1 / d.pin_scale): the exact sum
+// rounded once to FP64.
+__device__ __forceinline__ double pair_value(Pair p, double unscale) {
+  return unscale * (widen(p.s) + pair_rest(p));
+}
 
 }  // namespace hp

@@ -471,13 +471,11 @@ __global__ void __launch_bounds__(kBigNet) k_wa_big(Dev d, int copy0, int cls, i
 // over the nets are FP64, eight operations a net.  GB300's FP64 pipe takes two
 // operations per clock and SM, and with FP64 minima and maxima per pin and per
 // step of the lanes' reductions the evaluation was bound by nothing else.
-// Coordinates are halved first (exact but for subnormals), so that no FP32 sum
-// overflows.  HPWL and
-// overflow of the 2.1M-cell design: 1.44 -> 0.27 ms.
+// HPWL and overflow of the 2.1M-cell design: 1.44 -> 0.26 ms.
 __device__ __forceinline__ double extent(Pair hi, Pair lo) {
   return (widen(hi.s) - widen(lo.s)) + (pair_rest(hi) - pair_rest(lo));
 }
-// acc + w times the net's half perimeter, halved like its coordinates
+// acc + w times the net's half perimeter, scaled like its coordinates
 __device__ __forceinline__ double box_hpwl(const PairBox &b, float w, double acc) {
   return fma(widen(w), extent(b.mx, b.nx) + extent(b.my, b.ny), acc);
 }
@@ -491,11 +489,11 @@ __device__ __forceinline__ void hpwl_pin(const Dev &d, const float2 *xy, int j, 
   const float2 o = d.pin_off[j];
   int cj = d.pin_cell[j];
   HP_FIX(d.err, cj, d.n_cells, BS_HPWL_CELL);
-  box_add(b, xy[cj], o);
+  box_add(b, xy[cj], o, d.pin_scale);
 }
 template <int NT>
 __device__ __forceinline__ void hpwl_store(const Dev &d, int c, int cls, double acc, double *sm) {
-  const double r = 2.0 * block_sum<NT>(acc, sm);
+  const double r = d.pin_unscale * block_sum<NT>(acc, sm);
   if (threadIdx.x == 0)
     d.part[((size_t)c * S_COUNT + S_HP64) * d.nb_red + d.wa_block_base[cls] + blockIdx.x] = r;
 }
@@ -523,7 +521,7 @@ __global__ void __launch_bounds__(kThreads) k_hpwl_thread(Dev d, int copy0, int 
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (p0 + k < p1) box_add(b, xy[cj[k]], o[k]);
+      if (p0 + k < p1) box_add(b, xy[cj[k]], o[k], d.pin_scale);
     acc = box_hpwl(b, d.net_w ? d.net_w[e] : 1.0f, acc);
   }
   hpwl_store<kThreads>(d, c, cls, acc, sm);
@@ -668,7 +666,7 @@ __global__ void __launch_bounds__(kThreads) k_hpwl_big(Dev d, int copy0, int cls
     }
   }
   if (threadIdx.x == 0)
-    d.part[((size_t)c * S_COUNT + S_HP64) * d.nb_red + d.wa_block_base[cls] + blockIdx.x] = 2.0 * acc;
+    d.part[((size_t)c * S_COUNT + S_HP64) * d.nb_red + d.wa_block_base[cls] + blockIdx.x] = d.pin_unscale * acc;
 }
 
 // Measurement kernel: only the memory operations the WA pass cannot avoid

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kWmNetThreads) k_wm_static(Dev d, WmDev w, int
     int cj = d.pin_cell[j];
     HP_FIX(d.err, cj, d.n_cells, BS_WM_CELL);
     if (cj < d.n_real && d.is_macro[cj]) continue;
-    box_add(b, xy[cj], d.pin_off[j]);
+    box_add(b, xy[cj], d.pin_off[j], d.pin_scale);
     any = true;
   }
   box_reduce<32>(b);
@@ -198,7 +198,9 @@ __global__ void __launch_bounds__(kWmNetThreads) k_wm_static(Dev d, WmDev w, int
     b = sb[threadIdx.x % kWarps];
     box_reduce<kWarps>(b);
     if (threadIdx.x == 0) {
-      const Extent s = any ? Extent{{pair_value(b.nx), pair_value(b.mx), pair_value(b.ny), pair_value(b.my)}}
+      const double un = d.pin_unscale;
+      const Extent s = any ? Extent{{pair_value(b.nx, un), pair_value(b.mx, un), pair_value(b.ny, un),
+                                     pair_value(b.my, un)}}
                            : no_extent();
       if (q1 - q0 == 1) {
         store_extent(sbox, w.dent[q0], s);
