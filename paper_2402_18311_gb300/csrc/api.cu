@@ -1093,21 +1093,22 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   d.w_bin = std::sqrt(bw * bh);
   d.dref = (double)prm.hpwl_ref * (double)E * d.w_bin;
   {
-    // the largest finite pin coordinate: movable cells stay in the die
+    // the largest finite pin coordinate (movable cells stay in the die; finite
+    // numbers are in the order of their bits)
     double pos = std::max(std::max(std::fabs(die->xl), std::fabs(die->xh)), std::max(std::fabs(die->yl), std::fabs(die->yh)));
-    double off = 0.0;
-    auto most = [](double &m, float v) {
-      if (std::isfinite(v)) m = std::max(m, (double)std::fabs(v));
-    };
-    for (int i = nl->n_movable; i < nl->n_cells; ++i) {
-      most(pos, nl->x0[i]);
-      most(pos, nl->y0[i]);
-    }
-    for (int j = 0; j < P; ++j) {
-      most(off, nl->pin_dx[j]);
-      most(off, nl->pin_dy[j]);
-    }
-    d.pin_scale = pos + off < 1e38 ? 1.f : 0.5f;
+    for (int i = nl->n_movable; i < nl->n_cells; ++i)
+      pos = std::max(pos, (double)std::max(std::fabs(nl->x0[i]), std::fabs(nl->y0[i])));
+    unsigned int most = 0u;
+    for (const float *o : {nl->pin_dx, nl->pin_dy})
+      for (int j = 0; j < P; ++j) {
+        unsigned int u;
+        std::memcpy(&u, o + j, sizeof u);
+        u &= 0x7fffffffu;
+        most = std::max(most, u < 0x7f800000u ? u : 0u);
+      }
+    float off;
+    std::memcpy(&off, &most, sizeof off);
+    d.pin_scale = pos + (double)off < 1e38 ? 1.f : 0.5f;
     d.pin_unscale = 1.0 / d.pin_scale;
   }
   const long double lg_mu = prm.mu_base > 0.f && std::isfinite(prm.mu_base) ? std::log2((long double)prm.mu_base) : 0.0L;
