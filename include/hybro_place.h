@@ -56,7 +56,8 @@ extern "C" {
                                kept beside them */
 #define PLACE_DCT_FP32 0   /* FP32 CUDA cores (any grid, multiples of 16): fast
                               transforms where both sides are powers of two (64 ..
-                              4096), one kernel up to 4096 bins, GEMMs otherwise */
+                              4096), one kernel for at most 16 copies of up to 4096
+                              bins, GEMMs otherwise */
 #define PLACE_DCT_BF16X3 1 /* split-BF16 (3 products, FP32 accumulation) on the
                               tcgen05 tensor cores; grids must be multiples of 128 */
 
@@ -213,7 +214,8 @@ typedef struct place_info {
 #define PLACE_SOLVE_GEMM_FP32 0   /* tiled FP32 GEMMs */
 #define PLACE_SOLVE_GEMM_BF16X3 1 /* the tensor cores' GEMMs */
 #define PLACE_SOLVE_FFT 2         /* FP32 fast transforms */
-#define PLACE_SOLVE_CLUSTER 3     /* FP32, one cluster per copy (at most 4096 bins) */
+#define PLACE_SOLVE_CLUSTER 3     /* FP32, one cluster per copy (at most 4096 bins and
+                                   16 copies) */
 int place_get_solve(const place_t *h, int32_t *solve);
 
 /* Optimiser scalars of one copy after its last iteration. */

@@ -191,12 +191,22 @@ int resolve_dct_mode(int mode, int nx, int ny) {
 
 // The Poisson solve of a grid.  In FP32 mode, and where PLACE_DCT_AUTO and the
 // full split of the transforms (dct_fold) leave it to the library: one cluster
-// for a small grid, else the fast transforms on the sides they take.
-// PLACE_DCT_BF16X3 and dct_fold = 0 ask for the tensor cores' GEMMs.  mode:
-// the caller's, before resolve_dct_mode.
-int choose_solve(int mode, int fold, int nx, int ny) {
+// per copy for a small grid and few copies, else the fast transforms on the sides
+// they take.  PLACE_DCT_BF16X3 and dct_fold = 0 ask for the tensor cores' GEMMs.
+// mode: the caller's, before resolve_dct_mode.
+// A cluster's eight blocks each form the copy's whole density and hold a few
+// warps each, which pays while every block has an SM to itself (19 copies on 152
+// SMs); for more the GEMM chain, which gives the same bits, fills the chip better.
+// us per iteration, cluster / GEMMs, at 1, 16, 32, 64 and 256 copies: 1k cells on
+// 64 x 64 bins 31 / 32, 38 / 37, 47 / 43, 67 / 55, 190 / 117; 300 cells on 16 x 16 bins
+// 27 / 37, 29 / 34, 36 / 34, 42 / 39, 109 / 59; 1k cells on 48 x 80 bins 32 / 35,
+// 38 / 40, 49 / 46, 66 / 62, 185 / 132.
+constexpr int kSmallCopies = 16;
+int choose_solve(int mode, int fold, int nx, int ny, int copies) {
   const bool fp32 = resolve_dct_mode(mode, nx, ny) == PLACE_DCT_FP32;
-  if (fp32 && small_grid(nx, ny)) return SOLVE_SMALL;
+  // (above that line a small grid is never the fast transforms': they round
+  // differently, and a copy's bits do not depend on how many there are)
+  if (fp32 && small_grid(nx, ny)) return copies <= kSmallCopies ? SOLVE_SMALL : SOLVE_GEMM;
   if (fft_side(nx) && fft_side(ny) && (fp32 || (mode == PLACE_DCT_AUTO && fold))) return SOLVE_FFT;
   return SOLVE_GEMM;
 }
@@ -1037,7 +1047,7 @@ int place_create(const place_netlist *nl, const place_die *die, const place_bins
   if (prm.fillers != 0 && prm.fillers != 1) return fail(PLACE_EINVAL, "fillers must be 0 or 1");
   if (!(prm.macro_precond > 0.f) || !std::isfinite(prm.macro_precond))
     return fail(PLACE_EINVAL, "macro_precond must be positive and finite");
-  const int solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny);
+  const int solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny, prm.n_copies);
   prm.dct_mode = resolve_dct_mode(prm.dct_mode, bins->nx, bins->ny);
   if (prm.dct_mode != PLACE_DCT_FP32 && prm.dct_mode != PLACE_DCT_BF16X3)
     return fail(PLACE_EINVAL, "unknown dct_mode %d", prm.dct_mode);
@@ -2334,7 +2344,7 @@ extern "C" int place_estimate_device_bytes(const place_netlist *nl, const place_
   d.nx = bins->nx; d.ny = bins->ny; d.G = bins->nx * bins->ny;
   d.Gm = nf ? 2 * d.G : d.G;
   d.has_net_w = nl->net_w ? 1 : 0;
-  d.solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny);
+  d.solve = choose_solve(prm.dct_mode, prm.dct_fold, bins->nx, bins->ny, prm.n_copies);
   prm.dct_mode = resolve_dct_mode(prm.dct_mode, bins->nx, bins->ny);
   d.tc = prm.dct_mode == PLACE_DCT_BF16X3 ? 1 : 0;
   d.bfly = use_fold(d.tc, prm.dct_fold, bins->nx, bins->ny);

@@ -1,4 +1,5 @@
-// Spectral Poisson solve of a small grid (at most 4096 bins, FP32 path) in one
+// Spectral Poisson solve of a small grid (at most 4096 bins, FP32 path, few
+// copies: choose_solve in api.cu) in one
 // kernel: the density finish and the four transforms of spectral.cu by one
 // thread-block cluster per copy.
 //
