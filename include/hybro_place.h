@@ -300,9 +300,10 @@ int place_step_multi(place_t *const *hs, int32_t n, int32_t n_iters, int32_t *co
  * WireMask call allocates device scratch of about
  * K (16 (nx + ny) + 20 ny + 32 (E + S) + 16 (fixed cells + macros)) bytes, E the
  * nets of every macro added up, S the nets that several macros share, freed by
- * place_destroy.  It runs two small kernels per macro, captured
- * into a CUDA graph on the first call for each copy selection and replayed
- * by later calls (the graph is freed by place_destroy).  A design
+ * place_destroy; above 256 MB the copies take turns, as many at a time as fit.
+ * It runs two small kernels per macro (and turn), captured into a CUDA graph on
+ * the first call for each copy selection and replayed by later calls (the graph
+ * is freed by place_destroy).  A design
  * without movable macros only resets the optimiser.  EINVAL on an unknown
  * op or, for Shuffle, p outside [0, 1]; ENOMEM if the scratch cannot be
  * allocated. */

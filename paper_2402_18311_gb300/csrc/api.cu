@@ -826,7 +826,16 @@ int ensure_wiremask(place_t *h) {
   w.n_entries = (int)h->wm_net.size();
   w.n_dnets = (int)h->wm_dptr.size() - 1;
   w.n_shared = h->wm_shared;
-  const size_t K = d.K, n = std::max(w.n_entries, 1);
+  const size_t n = std::max(w.n_entries, 1);
+  // A pass over many copies of a design with many macros goes over a group of
+  // copies at a time, so that its scratch stays below this many bytes (or is one
+  // copy's): every copy's entries at once would be a third of the handle's own
+  // memory where all cells are macros.
+  const double most = 256.0 * (1 << 20);
+  const double per_copy = 32.0 * ((double)n + w.n_shared) + 16.0 * (d.nx + d.ny) + 20.0 * d.ny +
+                          16.0 * ((double)w.n_fixed + w.n_macros);
+  w.group = std::max(1, (int)std::min((double)d.K, std::floor(most / per_copy)));
+  const size_t K = w.group;
   Arena a;
   int *order = nullptr, *mptr = nullptr, *more = nullptr, *mnet = nullptr, *mcell = nullptr, *slot = nullptr,
       *dptr = nullptr, *dent = nullptr, *obst = nullptr;

@@ -226,6 +226,7 @@ struct WmDev {
   int n_entries;        // nets over all macros: mptr[n_macros]
   int n_dnets;          // the distinct ones, and those with several macros
   int n_shared;
+  int group;            // copies per pass: K in the scratch's sizes
   const int *order;     // [n_macros] macros by decreasing area, ties by index
   const int *mptr;      // [n_macros + 1] macro t's nets: entries mptr[t] .. mptr[t+1]
   const int *more;      // [n_macros] some later macro is on one of macro t's nets

@@ -43,11 +43,12 @@
 //     moved extents.
 // So the tables hold one entry per macro and net, and a macro's cost depends on
 // the number of its nets, not on how many macros share them.
-// Copies run side by side (blockIdx.y).  One pass over 32 macros of a 210k-cell design on 512 x 512
-// bins, restored before and read back: 3.7 -> 0.54 ms against one warp per net in FP64
+// Copies run side by side (blockIdx.y; w.group of them).  One pass over 32 macros of
+// a 210k-cell design on 512 x 512 bins, restored before and read back: 3.7 -> 0.54 ms against one warp per net in FP64
 // and four launches a macro.  (Launching each kernel early, by
 // griddepcontrol.launch_dependents at its start or before its last step, took
 // 28 us a macro instead of 15: measured, not taken.)
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -411,13 +412,15 @@ __global__ void __launch_bounds__(kWmThreads) k_wm_select(Dev d, WmDev w, int t,
 }  // namespace
 
 void launch_wiremask(const Dev &d, const WmDev &w, int copy0, int ncopy, cudaStream_t st) {
-  if (w.n_dnets > 0)
-    k_wm_static<<<dim3(w.n_dnets, ncopy), kWmNetThreads, 0, st>>>(d, w, copy0);
   const int lines = (d.nx + d.ny + kWmLines - 1) / kWmLines;
-  for (int t = 0; t < w.n_macros; ++t) {
-    const int ranges = (w.n_fixed + t + kWmLines - 1) / kWmLines;
-    launch_pdl(k_wm_mask, dim3(lines + ranges, ncopy), dim3(kWmLines), 0, st, d, w, t, copy0, lines);
-    launch_pdl(k_wm_select, dim3(d.ny, ncopy), dim3(kWmThreads), 0, st, d, w, t, copy0);
+  for (int c = copy0; c < copy0 + ncopy; c += w.group) {
+    const int k = std::min(w.group, copy0 + ncopy - c);
+    if (w.n_dnets > 0) k_wm_static<<<dim3(w.n_dnets, k), kWmNetThreads, 0, st>>>(d, w, c);
+    for (int t = 0; t < w.n_macros; ++t) {
+      const int ranges = (w.n_fixed + t + kWmLines - 1) / kWmLines;
+      launch_pdl(k_wm_mask, dim3(lines + ranges, k), dim3(kWmLines), 0, st, d, w, t, c, lines);
+      launch_pdl(k_wm_select, dim3(d.ny, k), dim3(kWmThreads), 0, st, d, w, t, c);
+    }
   }
 }
 
