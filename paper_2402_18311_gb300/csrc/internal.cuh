@@ -56,8 +56,11 @@ struct CopyState {
 // Reduction slots (FP64) per copy: each kernel that reduces writes one value
 // per block into its slot range; a reducer sums them in a fixed order.
 // S_PH, S_PW and S_PV: the cell-gradient blocks' shares of the WA kernels' and
-// of the step norm's partials (see k_cell_grad).
-enum Slot { S_TAU = 0, S_HPWL, S_WL, S_GW1, S_GD1, S_DG2, S_DV2, S_G2, S_HP64, S_PH, S_PW, S_PV, S_COUNT };
+// of the step norm's partials (see k_cell_grad), in ranges that are idle there
+// (the overflow's partials are in tau_part; the others are an evaluation's and
+// the first step's).
+enum Slot { S_TAU = 0, S_HPWL, S_WL, S_GW1, S_GD1, S_DG2, S_DV2, S_G2, S_HP64, S_COUNT,
+            S_PH = S_TAU, S_PW = S_HP64, S_PV = S_G2 };
 
 // Last-block counters per copy, and a flag: the copy had stopped when the fast
 // transforms' first kernel ran.
